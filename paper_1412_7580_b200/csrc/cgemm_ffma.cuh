@@ -7,15 +7,21 @@
 // (m contiguous); B likewise [2][bins][N][ldb] or, with transB, [2][bins][K][ldb];
 // C is [2][bins][M][ldc].
 //
-// CTA tile 64 x 64 of one bin, 256 threads, each thread a 4 x 4 block of complex
-// outputs (64 FFMAs per k against four 16-byte shared loads); k-blocks of 16 arrive by
-// asynchronous copies, double-buffered.  This is the exact
-// fp32 path and the fallback for shapes too small for the tensor-core kernel.
+// CTA tile 64 x 64 (or 64 x 96) of one bin, 128 threads, each thread 8 x 4 (8 x 6) complex outputs;
+// k-blocks of 16 arrive by asynchronous copies, double-buffered.  Bound by the fp32 pipe: 77-83 % of
+// its cycles busy (counters of S128 f96 f'256 n = 32 fprop and S128 f384 f'384 n = 16 accGrad), 51 and
+// 57 TFLOP/s.  With scalar multiply-adds, one per issue slot, the same tiles took 302 / 318 / 361 us on
+// the first layer's three passes and 447 / 452 / 459 us on the second's; packed in pairs they take
+// 254 / 258 / 273 and 372 / 353 / 342 us (results bit for bit the same).  This is the exact fp32 path
+// and the one for shapes too small for the tensor-core kernel.
 #pragma once
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "dep_launch.cuh"
+#include "f32x2.cuh"
 
 namespace fc {
 
@@ -56,14 +62,18 @@ __host__ __device__ inline int herm_bin(int b, int n) {
     return kx * nc + 1 + (b - (kx - nc) * (nc - 2));
 }
 
-constexpr int FG_BM = 64, FG_BN = 64, FG_BK = 16, FG_PAD = 4, FG_T = 256;
+constexpr int FG_BM = 64, FG_BK = 16, FG_PAD = 4, FG_T = 128;
 
-// 4-byte asynchronous copy global -> shared; `ok` false writes a zero (zero-fill of the
+// Asynchronous copy global -> shared of 4 or 16 bytes; `ok` false writes zeros (zero-fill of the
 // ragged edges of M, N and K).
-__device__ __forceinline__ void fg_cp4(float* dst, const float* src, bool ok) {
+template <int BYTES>
+__device__ __forceinline__ void fg_cp(float* dst, const float* src, bool ok) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-    const int nbytes = ok ? 4 : 0;
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(nbytes) : "memory");
+    const int nbytes = ok ? BYTES : 0;
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(nbytes) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(nbytes) : "memory");
 }
 
 // TA / TB: operand stored [K][rows] instead of [rows][K]; CA / CB: use its complex conjugate.
@@ -71,8 +81,12 @@ __device__ __forceinline__ void fg_cp4(float* dst, const float* src, bool ok) {
 // are in flight while block kb is multiplied.
 // BN: columns of a tile, 64 (4 per thread) or 96 (6 per thread; chosen where it leaves fewer
 // padded columns, e.g. N = 96: one tile of 96 instead of 64 + 32 of 64).
+// A thread owns 8 rows x TN columns.  The rows are packed in pairs (fma.f32x2: two multiply-adds
+// per issue slot; the pairs of A come ready from the 16-byte shared loads, the values of B are
+// duplicated into both halves): per k 16 TN packed multiply-adds, which keep the fp32 pipe busy
+// for 32 TN cycles, against 4 + TN / 2 shared loads and 2 TN duplications in the free issue slots.
 template <bool TA, bool TB, bool CA, bool CB, int BN>
-__global__ void __launch_bounds__(FG_T) cgemm_ffma_kernel(const GemmParams p) {
+__global__ void __launch_bounds__(FG_T, BN == 64 ? 4 : 3) cgemm_ffma_kernel(const GemmParams p) {
     static_assert(BN == 64 || BN == 96, "16 thread columns of 4 or 6 outputs");
     constexpr int TN = BN / 16;
     __shared__ __align__(16) float sA[2][2][FG_BK][FG_BM + FG_PAD];
@@ -94,65 +108,49 @@ __global__ void __launch_bounds__(FG_T) cgemm_ffma_kernel(const GemmParams p) {
     const size_t imA = (size_t)p.bins * planeA, imB = (size_t)p.bins * planeB,
                  imC = (size_t)p.bins * planeC;
 
-    const int tx = tid & 15, ty = tid >> 4;      // 16 x 16 threads
-    const int lk = tid & 15, lr = tid >> 4;      // loader, k-contiguous operand: k within block, row group
-    const int tr = tid & 63, tk = tid >> 6;      // loader, row-contiguous operand: row, k group
+    const int tx = tid & 15, ty = tid >> 4;      // 16 x 8 threads
 
-    // global -> shared as [k][row]; lanes run along the contiguous index of each operand
+    // global -> shared as [k][row]; lanes run along the contiguous index of each operand.  A
+    // row-contiguous operand moves in 16-byte pieces (its leading dimension is a multiple of 4;
+    // a piece that straddles the last row brings in padding, which only reaches outputs that
+    // are not stored), a k-contiguous one is transposed by 4-byte copies.
+    auto issue_op = [&](auto TRANS, auto& s, const float* base, size_t im, int ld, int r_blk, int rows, int k0) {
+        constexpr int ROWS = (int)(sizeof(s[0][0]) / sizeof(float)) - FG_PAD;
+        if constexpr (decltype(TRANS)::value) {
+            constexpr int PIECES = ROWS / 4;
+#pragma unroll
+            for (int i = tid; i < PIECES * FG_BK; i += FG_T) {
+                const int kk = i / PIECES, r = 4 * (i - kk * PIECES);
+                const bool ok = (k0 + kk < p.K) && (r_blk + r < rows);
+                const float* src = ok ? base + (size_t)(k0 + kk) * ld + r_blk + r : base;
+                fg_cp<16>(&s[0][kk][r], src, ok);
+                fg_cp<16>(&s[1][kk][r], src + im, ok);
+            }
+        } else {
+            const int lk = tid & 15, lr = tid >> 4, k = k0 + lk;
+            const float* src0 = base + (size_t)(r_blk + lr) * ld + k;
+#pragma unroll
+            for (int it = 0; it < ROWS / 8; ++it) {
+                const int r = lr + 8 * it;
+                const bool ok = (k < p.K) && (r_blk + r < rows);
+                const float* src = ok ? src0 + (size_t)(8 * it) * ld : base;
+                fg_cp<4>(&s[0][lk][r], src, ok);
+                fg_cp<4>(&s[1][lk][r], src + im, ok);
+            }
+        }
+    };
     auto issue = [&](int k0, int st) {
-        if constexpr (!TA) {
-            const int k = k0 + lk;
-#pragma unroll
-            for (int it = 0; it < FG_BM / 16; ++it) {
-                const int r = lr + 16 * it, m = m_blk + r;
-                const bool ok = (k < p.K) && (m < p.M);
-                const float* src = ok ? Ab + (size_t)m * p.lda + k : Ab;
-                fg_cp4(&sA[st][0][lk][r], src, ok);
-                fg_cp4(&sA[st][1][lk][r], src + imA, ok);
-            }
-        } else {
-            const int m = m_blk + tr;
-#pragma unroll
-            for (int it = 0; it < FG_BK / 4; ++it) {
-                const int kk = tk + 4 * it, k = k0 + kk;
-                const bool ok = (k < p.K) && (m < p.M);
-                const float* src = ok ? Ab + (size_t)k * p.lda + m : Ab;
-                fg_cp4(&sA[st][0][kk][tr], src, ok);
-                fg_cp4(&sA[st][1][kk][tr], src + imA, ok);
-            }
-        }
-        if constexpr (!TB) {
-            const int k = k0 + lk;
-#pragma unroll
-            for (int it = 0; it < BN / 16; ++it) {
-                const int r = lr + 16 * it, n = n_blk + r;
-                const bool ok = (k < p.K) && (n < p.N);
-                const float* src = ok ? Bb + (size_t)n * p.ldb + k : Bb;
-                fg_cp4(&sB[st][0][lk][r], src, ok);
-                fg_cp4(&sB[st][1][lk][r], src + imB, ok);
-            }
-        } else {
-#pragma unroll
-            for (int rr = tr; rr < BN; rr += 64) {
-                const int n = n_blk + rr;
-#pragma unroll
-                for (int it = 0; it < FG_BK / 4; ++it) {
-                    const int kk = tk + 4 * it, k = k0 + kk;
-                    const bool ok = (k < p.K) && (n < p.N);
-                    const float* src = ok ? Bb + (size_t)k * p.ldb + n : Bb;
-                    fg_cp4(&sB[st][0][kk][rr], src, ok);
-                    fg_cp4(&sB[st][1][kk][rr], src + imB, ok);
-                }
-            }
-        }
+        issue_op(std::integral_constant<bool, TA>{}, sA[st], Ab, imA, p.lda, m_blk, p.M, k0);
+        issue_op(std::integral_constant<bool, TB>{}, sB[st], Bb, imB, p.ldb, n_blk, p.N, k0);
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    float cr[4][TN], ci[4][TN];
+    // rows ty*4 .. +3 and 32 + ty*4 .. +3: the 16-byte loads of the 8 thread rows cover whole lines
+    F2 cr[4][TN], ci[4][TN];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) cr[i][j] = ci[i][j] = 0.0f;
+        for (int j = 0; j < TN; ++j) cr[i][j].b = ci[i][j].b = 0ull;
 
     const int k_blocks = (p.K + FG_BK - 1) / FG_BK;
     issue(0, 0);
@@ -165,12 +163,16 @@ __global__ void __launch_bounds__(FG_T) cgemm_ffma_kernel(const GemmParams p) {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();                                            // ... and for everyone
-#pragma unroll
+#pragma unroll 4
         for (int kk = 0; kk < FG_BK; ++kk) {
-            const float4 a_r = *reinterpret_cast<const float4*>(&sA[st][0][kk][ty * 4]);
-            const float4 a_i = *reinterpret_cast<const float4*>(&sA[st][1][kk][ty * 4]);
-            const float ar[4] = {a_r.x, a_r.y, a_r.z, a_r.w};
-            const float ai[4] = {a_i.x, a_i.y, a_i.z, a_i.w};
+            F2 ar[4], ai[4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const ulonglong2 v_r = *reinterpret_cast<const ulonglong2*>(&sA[st][0][kk][32 * h + ty * 4]);
+                const ulonglong2 v_i = *reinterpret_cast<const ulonglong2*>(&sA[st][1][kk][32 * h + ty * 4]);
+                ar[2 * h].b = v_r.x; ar[2 * h + 1].b = v_r.y;
+                ai[2 * h].b = v_i.x; ai[2 * h + 1].b = v_i.y;
+            }
             float br[TN], bi[TN];
             if constexpr (TN == 4) {
                 const float4 b_r = *reinterpret_cast<const float4*>(&sB[st][0][kk][tx * 4]);
@@ -187,16 +189,25 @@ __global__ void __launch_bounds__(FG_T) cgemm_ffma_kernel(const GemmParams p) {
                 }
             }
             // (ar + i sa ai)(br + i sb bi), sa / sb = -1 for a conjugated operand:
-            // re = ar br - sa sb ai bi,  im = sb ar bi + sa ai br
+            // re = ar br - sa sb ai bi,  im = sb ar bi + sa ai br; the signs ride on the values
+            // of B, which are duplicated anyway
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < TN; ++j) {
+                const F2 rr = f2_pack(br[j], br[j]);
+                const float nb = (CA != CB) ? bi[j] : -bi[j];
+                const F2 ii = f2_pack(nb, nb);
+                const float sb = CB ? -bi[j] : bi[j];
+                const F2 ri = f2_pack(sb, sb);
+                const float sr = CA ? -br[j] : br[j];
+                const F2 ir = f2_pack(sr, sr);
 #pragma unroll
-                for (int j = 0; j < TN; ++j) {
-                    cr[i][j] = fmaf(ar[i], br[j], cr[i][j]);
-                    cr[i][j] = fmaf((CA != CB) ? ai[i] : -ai[i], bi[j], cr[i][j]);
-                    ci[i][j] = fmaf(CB ? -ar[i] : ar[i], bi[j], ci[i][j]);
-                    ci[i][j] = fmaf(CA ? -ai[i] : ai[i], br[j], ci[i][j]);
+                for (int i = 0; i < 4; ++i) {
+                    cr[i][j] = f2_fma(ar[i], rr, cr[i][j]);
+                    cr[i][j] = f2_fma(ai[i], ii, cr[i][j]);
+                    ci[i][j] = f2_fma(ar[i], ri, ci[i][j]);
+                    ci[i][j] = f2_fma(ai[i], ir, ci[i][j]);
                 }
+            }
         }
         __syncthreads();                                            // stage st may be refilled
     }
@@ -204,23 +215,30 @@ __global__ void __launch_bounds__(FG_T) cgemm_ffma_kernel(const GemmParams p) {
     const int n0 = n_blk + tx * TN;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int m = m_blk + ty * 4 + i;
-        if (m >= p.M) continue;
-        float* o_r = Cb + (size_t)m * p.ldc + n0;
-        float* o_i = o_r + imC;
-        bool vec = false;
-        if constexpr (TN == 4) {
-            if (n0 + 3 < p.N) {
-                *reinterpret_cast<float4*>(o_r) = make_float4(cr[i][0], cr[i][1], cr[i][2], cr[i][3]);
-                *reinterpret_cast<float4*>(o_i) = make_float4(ci[i][0], ci[i][1], ci[i][2], ci[i][3]);
-                vec = true;
-            }
+        float lo_r[TN], hi_r[TN], lo_i[TN], hi_i[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            f2_unpack(cr[i][j], lo_r[j], hi_r[j]);
+            f2_unpack(ci[i][j], lo_i[j], hi_i[j]);
         }
-        if (!vec) {
+        auto put = [&](int m, const float (&vr)[TN], const float (&vi)[TN]) {
+            if (m >= p.M) return;
+            float* o_r = Cb + (size_t)m * p.ldc + n0;
+            float* o_i = o_r + imC;
+            if constexpr (TN == 4) {
+                if (n0 + 3 < p.N) {
+                    *reinterpret_cast<float4*>(o_r) = make_float4(vr[0], vr[1], vr[2], vr[3]);
+                    *reinterpret_cast<float4*>(o_i) = make_float4(vi[0], vi[1], vi[2], vi[3]);
+                    return;
+                }
+            }
 #pragma unroll
             for (int j = 0; j < TN; ++j)
-                if (n0 + j < p.N) { o_r[j] = cr[i][j]; o_i[j] = ci[i][j]; }
-        }
+                if (n0 + j < p.N) { o_r[j] = vr[j]; o_i[j] = vi[j]; }
+        };
+        const int m = m_blk + 32 * (i >> 1) + ty * 4 + 2 * (i & 1);
+        put(m, lo_r, lo_i);
+        put(m + 1, hi_r, hi_i);
     }
 }
 
@@ -245,7 +263,7 @@ static cudaError_t launch_cgemm_ffma_bn(const GemmParams& p, cudaStream_t st) {
 static cudaError_t launch_cgemm_ffma(const GemmParams& p, cudaStream_t st) {
     // the tile width that pads N the least (on a tie the 64-wide tile: 10 % faster per multiply-add, measured)
     const int pad64 = (p.N + 63) / 64 * 64, pad96 = (p.N + 95) / 96 * 96;
-    return pad96 < pad64 ? launch_cgemm_ffma_bn<96>(p, st) : launch_cgemm_ffma_bn<FG_BN>(p, st);
+    return pad96 < pad64 ? launch_cgemm_ffma_bn<96>(p, st) : launch_cgemm_ffma_bn<64>(p, st);
 }
 
 }  // namespace fc
