@@ -2,25 +2,22 @@
 // paper's Section 5 evaluates), with the zero-padding fused into the load and
 // crop, scale and accumulate fused into the store.
 //
-// A CTA of 128 threads takes a tile of consecutive signals.  The tile is copied
-// between global and shared memory with fully coalesced accesses (consecutive
-// threads, consecutive addresses); in shared memory every signal sits at an odd
-// pitch, so that threads working on different signals hit different banks.
-//   n <= 64 : one thread per signal, the whole real transform in registers.
-//   n >= 128: four threads per signal.  The real transform of length n is a complex
-//             transform of length n/2 on z_j = x_2j + i x_2j+1 (Supplement 8.2 notation)
-//             plus a Hermitian post-pass; the complex transform is split over the four
-//             threads by one radix-4 decimation-in-frequency step applied while loading,
-//             each thread finishing with an n/8-point register transform; the post-pass
-//             (which pairs bins k and n/2-k, held by different threads) runs on the
-//             shared-memory copy.  The inverse mirrors this: pre-pass in shared memory,
-//             then the split inverse complex transform.
+//   n <= 64 : a CTA of 128 threads takes a tile of consecutive signals, one thread per
+//             signal, the whole real transform in registers.  The tile is copied between
+//             global and shared memory with coalesced accesses; in shared memory every signal
+//             sits at an odd pitch, so that threads working on different signals hit
+//             different banks.
+//   n >= 128: T = n/32 threads per signal, a warp works on its own on 32/T consecutive signals
+//             (no CTA barrier anywhere).  The real transform of length n is a complex
+//             transform of length M = n/2 = 16 T on z_j = x_2j + i x_2j+1 (Supplement 8.2
+//             notation) plus a Hermitian post-pass; see F1Warp below.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "fft_core.cuh"
+#include "fft_kernels.cuh"
 
 namespace fc {
 
@@ -38,8 +35,7 @@ struct Fft1dParams {
 };
 
 template <int N> struct F1Cfg {
-    static constexpr int TPT = (N <= 64) ? 1 : 4;           // threads per signal
-    static constexpr int TB = F1_THREADS / TPT;             // signals per CTA
+    static constexpr int TB = F1_THREADS;                   // signals per CTA, one per thread
     static constexpr int NC = N / 2 + 1;
     static constexpr int PITCH_C = NC | 1;                  // complex pitch (float2 units), odd
     static constexpr int PITCH_R = N | 1;                   // real pitch of a full-length signal, odd
@@ -54,16 +50,11 @@ __device__ __forceinline__ void f1_cp_async(void* smem_dst, const void* gmem_src
                  : "memory");
 }
 
-// cos and sin of 2 pi k / n for a run-time k (post- and pre-pass of the split transforms)
-__device__ __forceinline__ void f1_twiddle(int k, int n, float& c, float& s) {
-    sincospif(2.0f * (float)k / (float)n, &s, &c);
-}
-
 template <int N>
 __global__ void __launch_bounds__(F1_THREADS)
 fft1d_r2c_kernel(const Fft1dParams p) {
     using C = F1Cfg<N>;
-    constexpr int TB = C::TB, NC = C::NC, PC = C::PITCH_C, M = N / 2;
+    constexpr int TB = C::TB, NC = C::NC, PC = C::PITCH_C;
     extern __shared__ __align__(16) unsigned char f1_smem[];
     float* sR = reinterpret_cast<float*>(f1_smem);
     float2* sC = reinterpret_cast<float2*>(f1_smem);
@@ -86,7 +77,7 @@ fft1d_r2c_kernel(const Fft1dParams p) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
-    if constexpr (C::TPT == 1) {
+    {
         float Xr[NC], Xi[NC];
         {
             float v[N];
@@ -103,58 +94,6 @@ fft1d_r2c_kernel(const Fft1dParams p) {
             constexpr int k = decltype(K)::value;
             orow[k] = make_float2(Xr[k], Xi[k]);
         });
-    } else {
-        // quarter Q of the complex transform of length M: warp-uniform Q, lane = signal
-        constexpr int L = M / 4;
-        const int Q = tid / TB, t = tid - Q * TB;
-        float ar[L], ai[L];
-        {
-            const float* row = sR + t * pr;
-            auto load = [&](auto J) -> float2 {
-                constexpr int j = decltype(J)::value;
-                float2 z;
-                z.x = (t < cnt && 2 * j < len) ? row[2 * j] : 0.0f;
-                z.y = (t < cnt && 2 * j + 1 < len) ? row[2 * j + 1] : 0.0f;
-                return z;
-            };
-            if (Q == 0) load_split4<M, false, 0>(load, ar, ai);
-            else if (Q == 1) load_split4<M, false, 1>(load, ar, ai);
-            else if (Q == 2) load_split4<M, false, 2>(load, ar, ai);
-            else load_split4<M, false, 3>(load, ar, ai);
-        }
-        cfft<L, false>(ar, ai);             // ar/ai[m] = Z_{4m+Q}
-        __syncthreads();
-        {
-            float2* zrow = sC + t * PC + Q;
-            static_for<L>([&](auto Mm) {
-                constexpr int m = decltype(Mm)::value;
-                zrow[4 * m] = make_float2(ar[m], ai[m]);
-            });
-        }
-        __syncthreads();
-        // Hermitian post-pass on the shared copy: X_k = E_k + w_N^k O_k, X_{M-k} = conj(E_k - w_N^k O_k)
-        // with 2 E_k = Z_k + conj Z_{M-k}, 2 O_k = -i (Z_k - conj Z_{M-k}); one (signal, k) pair per step
-        for (int it = tid; it < TB * (M / 2 + 1); it += F1_THREADS) {
-            const int tt = it % TB, k = it / TB;
-            float2* z = sC + tt * PC;
-            if (k == 0) {
-                const float2 a = z[0];
-                z[0] = make_float2(a.x + a.y, 0.0f);
-                z[M] = make_float2(a.x - a.y, 0.0f);
-            } else if (2 * k == M) {
-                const float2 a = z[k];
-                z[k] = make_float2(a.x, -a.y);
-            } else {
-                float c, s;
-                f1_twiddle(k, N, c, s);
-                const float2 a = z[k], b = z[M - k];
-                const float er = a.x + b.x, ei = a.y - b.y;
-                const float orr = a.y + b.y, oi = b.x - a.x;
-                const float tr = 0.5f * (s * oi + c * orr), ti = 0.5f * (c * oi - s * orr);
-                z[k] = make_float2(0.5f * er + tr, 0.5f * ei + ti);
-                z[M - k] = make_float2(0.5f * er - tr, ti - 0.5f * ei);
-            }
-        }
     }
     __syncthreads();
 
@@ -170,7 +109,7 @@ template <int N>
 __global__ void __launch_bounds__(F1_THREADS)
 fft1d_c2r_kernel(const Fft1dParams p) {
     using C = F1Cfg<N>;
-    constexpr int TB = C::TB, NC = C::NC, PC = C::PITCH_C, PR = C::PITCH_R, M = N / 2;
+    constexpr int TB = C::TB, NC = C::NC, PC = C::PITCH_C, PR = C::PITCH_R;
     extern __shared__ __align__(16) unsigned char f1_smem[];
     float* sR = reinterpret_cast<float*>(f1_smem);
     float2* sC = reinterpret_cast<float2*>(f1_smem);
@@ -189,7 +128,7 @@ fft1d_c2r_kernel(const Fft1dParams p) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
-    if constexpr (C::TPT == 1) {
+    {
         float v[N];
         {
             float Xr[NC], Xi[NC];
@@ -207,48 +146,6 @@ fft1d_c2r_kernel(const Fft1dParams p) {
             constexpr int j = decltype(J)::value;
             orow[j] = v[j];
         });
-    } else {
-        // pre-pass on the shared copy: Z'_k = (X_k + conj X_{M-k}) + i w_N^{-k} (X_k - conj X_{M-k})
-        for (int it = tid; it < TB * (M / 2 + 1); it += F1_THREADS) {
-            const int tt = it % TB, k = it / TB;
-            float2* z = sC + tt * PC;
-            if (k == 0) {
-                const float x0 = z[0].x, xm = z[M].x;
-                z[0] = make_float2(x0 + xm, x0 - xm);
-            } else if (2 * k == M) {
-                const float2 a = z[k];
-                z[k] = make_float2(2.0f * a.x, -2.0f * a.y);
-            } else {
-                float c, s;
-                f1_twiddle(k, N, c, s);
-                const float2 a = z[k], b = z[M - k];
-                const float er = a.x + b.x, ei = a.y - b.y;
-                const float dr = a.x - b.x, di = a.y + b.y;
-                const float ur = c * dr - s * di, ui = s * dr + c * di;
-                z[k] = make_float2(er - ui, ei + ur);
-                z[M - k] = make_float2(er + ui, ur - ei);
-            }
-        }
-        __syncthreads();
-        constexpr int L = M / 4;
-        const int Q = tid / TB, t = tid - Q * TB;
-        float ar[L], ai[L];
-        {
-            const float2* row = sC + t * PC;
-            auto load = [&](auto J) -> float2 { return row[decltype(J)::value]; };
-            if (Q == 0) load_split4<M, true, 0>(load, ar, ai);
-            else if (Q == 1) load_split4<M, true, 1>(load, ar, ai);
-            else if (Q == 2) load_split4<M, true, 2>(load, ar, ai);
-            else load_split4<M, true, 3>(load, ar, ai);
-        }
-        cfft<L, true>(ar, ai);              // ar/ai[m] = z_{4m+Q} = x_{2(4m+Q)} + i x_{2(4m+Q)+1}, times N
-        __syncthreads();
-        float* orow = sR + t * PR + 2 * Q;
-        static_for<L>([&](auto Mm) {
-            constexpr int m = decltype(Mm)::value;
-            orow[8 * m] = ar[m];
-            orow[8 * m + 1] = ai[m];
-        });
     }
     __syncthreads();
 
@@ -265,6 +162,332 @@ fft1d_c2r_kernel(const Fft1dParams p) {
         r += dr; j += dj;
         if (j >= len) { j -= len; ++r; }
     }
+}
+
+// ---------------------------------------------------------------------------
+// n = 128 and 256: T threads per signal, SPW signals per warp.
+// Forward:  z_j with j = t + T m sits in thread t; with q = k + 16 r
+//   Z_q = sum_t w_T^{t r} [ w_M^{t k} sum_m z_{t + T m} w_16^{m k} ],
+// a 16-point transform per thread, a twiddle, an exchange inside the warp's shared buffer, and a
+// T-point transform per residue class k.  The Hermitian post-pass pairs Z_q with Z_{M-q}, i.e.
+// the classes k and 16 - k, so a thread takes both of them and the post-pass stays in registers.
+// Thread 0 of a signal takes the classes 0 and 8, which pair with themselves; its values are
+// moved by selects so that all threads run the same eight pairs (bin M/2 is left over there).
+// The inverse runs the same steps backwards.  All twiddles that depend on the thread are
+// evaluated once per thread; signals are walked with a grid stride.
+// Signals travel as one bulk asynchronous copy per warp and direction (consecutive signals are
+// contiguous): the next signals are requested as soon as the current ones are in registers, and
+// the results of two groups may still be on their way out.
+// Bound by HBM: 262,143 signals of 250 samples (n = 256) 207 -> 102 us forward and 138 -> 102 us
+// inverse, 5.2 TB/s of samples and spectra; 524,288 signals of 128 samples (n = 128) 147 -> 98
+// and 126 -> 96 us, 5.5 TB/s (before: four threads per signal and a CTA barrier between the steps,
+// 4-byte copies, twiddles of the post-pass evaluated per pair).
+// ---------------------------------------------------------------------------
+template <int N>
+struct F1Warp {
+    static constexpr int M = N / 2, NC = M + 1, T = M / 16, SPW = 32 / T, CPT = 16 / T;
+    static constexpr int EROW = T + 1;                              // exchange: class pitch
+    static constexpr int EP = 16 * EROW + (T == 8 ? 8 : 4);         // exchange: signal pitch, conflict-free across a half warp
+    static constexpr int WARPS = 4;
+    static constexpr int EXCH_BYTES = SPW * EP * 8;
+    static constexpr int IN_BYTES = SPW * NC * 8;                   // spectra, or at most as many samples
+    static constexpr size_t SMEM = (size_t)WARPS * (2 * EXCH_BYTES + IN_BYTES);
+    static_assert(EXCH_BYTES >= SPW * NC * 8 && EXCH_BYTES >= SPW * N * 4, "the exchange buffer holds the results");
+    static_assert(EXCH_BYTES % 16 == 0 && IN_BYTES % 16 == 0, "a warp's buffers are whole 16-byte units");
+};
+
+template <int N>
+struct F1WarpRoles {
+    using C = F1Warp<N>;
+    int t, s, cls[C::CPT], kp[8];
+    float pc[8], ps[8];             // w_N^kp = (pc, -ps)
+    __device__ __forceinline__ explicit F1WarpRoles(int lane) {
+        constexpr int T = C::T, H = T / 2;
+        s = lane / T; t = lane - s * T;
+        cls[0] = t; cls[1] = t ? 16 - t : 8;
+        if constexpr (C::CPT == 4) { cls[2] = t ? 8 - t : 4; cls[3] = 16 - cls[2]; }
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+            if (p < T) kp[p] = (t == 0 && p >= H) ? 8 + 16 * (p - H) : t + 16 * p;
+            else kp[p] = cls[C::CPT - 2] + 16 * (p - T);
+            sincospif(2.0f * (float)kp[p] / (float)N, &ps[p], &pc[p]);
+        }
+    }
+};
+
+// Bulk copy of a warp's signals into its input buffer, or plain loads where that is not possible
+// (ragged last group, misaligned tensor); true if the copy is asynchronous.
+__device__ __forceinline__ bool f1w_fetch(float* dst, const float* src, int words, bool whole, uint32_t bar, int lane) {
+    if (whole && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+        if (lane == 0) {
+            fk_mbar_expect_tx(bar, (uint32_t)words * 4u);
+            fk_bulk_g2s(fk_smem_u32(dst), src, (uint32_t)words * 4u, bar);
+        }
+        return true;
+    }
+    for (int i = lane; i < words; i += 32) dst[i] = __ldg(src + i);
+    return false;
+}
+
+template <int N>
+__global__ void __launch_bounds__(128, 4)
+fft1d_warp_r2c_kernel(const Fft1dParams p) {
+    using C = F1Warp<N>;
+    constexpr int M = C::M, NC = C::NC, T = C::T, H = T / 2, SPW = C::SPW, CPT = C::CPT, EP = C::EP, EROW = C::EROW;
+    extern __shared__ __align__(128) unsigned char f1_smem_w[];
+    __shared__ __align__(8) unsigned long long bar_storage[C::WARPS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, len = p.len;
+    const uint32_t bar = fk_smem_u32(&bar_storage[warp]);
+    unsigned char* mine = f1_smem_w + (size_t)warp * (2 * C::EXCH_BYTES + C::IN_BYTES);
+    float* sIn = reinterpret_cast<float*>(mine + 2 * C::EXCH_BYTES);
+    if (lane == 0) {
+        fk_mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    const F1WarpRoles<N> ro(lane);
+    const int t = ro.t;
+    const bool t0 = t == 0;
+    float tc[16], ts[16];                                   // w_M^{t k} = (tc, -ts)
+#pragma unroll
+    for (int k = 1; k < 16; ++k) sincospif(2.0f * (float)(t * k) / (float)M, &ts[k], &tc[k]);
+
+    const long long groups = (p.batch + SPW - 1) / SPW, stride = (long long)gridDim.x * C::WARPS;
+    auto count = [&](long long g) { const long long left = p.batch - g * SPW; return left < SPW ? (int)left : SPW; };
+    auto fetch = [&](long long g) {
+        const int c = count(g);
+        return f1w_fetch(sIn, p.real_in + g * SPW * len, c * len, c == SPW, bar, lane);
+    };
+    long long g = (long long)blockIdx.x * C::WARPS + warp;
+    bool pending = g < groups ? fetch(g) : false;
+    uint32_t phase = 0;
+    for (int buf = 0; g < groups; g += stride, buf ^= 1) {
+        float2* ex = reinterpret_cast<float2*>(mine + buf * C::EXCH_BYTES);
+        __syncwarp();
+        if (pending) {
+            if (!fk_mbar_wait(bar, phase, 0)) break;
+            phase ^= 1u;
+        }
+        float zr[16], zi[16];
+        {
+            const float* row = sIn + ro.s * len + 2 * t;
+            const int left = len - 2 * t;                   // samples from this thread's first one on
+            if ((len & 1) == 0) {
+                static_for<16>([&](auto Mm) {
+                    constexpr int o = 2 * T * decltype(Mm)::value;
+                    const float2 v = (o < left) ? *reinterpret_cast<const float2*>(row + o) : make_float2(0.0f, 0.0f);
+                    zr[decltype(Mm)::value] = v.x; zi[decltype(Mm)::value] = v.y;
+                });
+            } else {
+                static_for<16>([&](auto Mm) {
+                    constexpr int o = 2 * T * decltype(Mm)::value;
+                    zr[decltype(Mm)::value] = (o < left) ? row[o] : 0.0f;
+                    zi[decltype(Mm)::value] = (o + 1 < left) ? row[o + 1] : 0.0f;
+                });
+            }
+        }
+        cfft<16, false>(zr, zi);
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // this buffer's last store
+        __syncwarp();                       // ... and every lane has its samples
+        pending = g + stride < groups ? fetch(g + stride) : false;
+        float2* e = ex + ro.s * EP;
+        static_for<16>([&](auto K) {
+            constexpr int k = decltype(K)::value;
+            if constexpr (k == 0) e[t] = make_float2(zr[0], zi[0]);
+            else e[k * EROW + t] = make_float2(fc_fma(ts[k], zi[k], tc[k] * zr[k]), fc_fma(-ts[k], zr[k], tc[k] * zi[k]));
+        });
+        __syncwarp();
+        float Zr[CPT][T], Zi[CPT][T];
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) {
+            const float2* a = e + ro.cls[c] * EROW;
+            static_for<T>([&](auto R) {
+                const float2 v = a[decltype(R)::value];
+                Zr[c][decltype(R)::value] = v.x; Zi[c][decltype(R)::value] = v.y;
+            });
+            cfft<T, false>(Zr[c], Zi[c]);                   // Z_{cls + 16 r}
+        }
+        __syncwarp();                                       // the exchange is over: the buffer becomes the spectra
+        float2* o = ex + ro.s * NC;
+        auto pair = [&](auto P, float pr, float pi, float qr, float qi) {
+            constexpr int q = decltype(P)::value;
+            const float hc = 0.5f * ro.pc[q], hs = 0.5f * ro.ps[q];
+            const float er = pr + qr, ei = pi - qi, orr = pi + qi, oi = qr - pr;    // 2 E, 2 O
+            const float tr = fc_fma(hs, oi, hc * orr), ti = fc_fma(-hs, orr, hc * oi);
+            o[ro.kp[q]] = make_float2(fc_fma(0.5f, er, tr), fc_fma(0.5f, ei, ti));
+            o[M - ro.kp[q]] = make_float2(fc_fma(0.5f, er, -tr), fc_fma(-0.5f, ei, ti));
+        };
+        static_for<T>([&](auto P) {
+            constexpr int q = decltype(P)::value;
+            float pr = Zr[0][q], pi = Zi[0][q], qr = Zr[1][T - 1 - q], qi = Zi[1][T - 1 - q];
+            if constexpr (q < H) {
+                constexpr int j = q == 0 ? 0 : T - q;
+                qr = t0 ? Zr[0][j] : qr; qi = t0 ? Zi[0][j] : qi;
+            } else {
+                constexpr int l = T - 1 - (q - H);
+                pr = t0 ? Zr[1][q - H] : pr; pi = t0 ? Zi[1][q - H] : pi;
+                qr = t0 ? Zr[1][l] : qr; qi = t0 ? Zi[1][l] : qi;
+            }
+            pair(P, pr, pi, qr, qi);
+        });
+        if constexpr (CPT == 4) {
+            static_for<T>([&](auto P) {
+                constexpr int q = decltype(P)::value;
+                pair(std::integral_constant<int, T + q>{}, Zr[2][q], Zi[2][q], Zr[3][T - 1 - q], Zi[3][T - 1 - q]);
+            });
+        }
+        if (t0) o[M / 2] = make_float2(Zr[0][H], -Zi[0][H]);
+        const int cnt = count(g);
+        float2* dst = p.spec_out + g * SPW * NC;
+        if (cnt == SPW && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) fk_bulk_s2g(dst, fk_smem_u32(ex), (uint32_t)(SPW * NC * 8));
+        } else {
+            __syncwarp();
+            for (int i = lane; i < cnt * NC; i += 32) dst[i] = ex[i];
+        }
+        if (lane == 0) fk_bulk_commit();
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+template <int N>
+__global__ void __launch_bounds__(128, 4)
+fft1d_warp_c2r_kernel(const Fft1dParams p) {
+    using C = F1Warp<N>;
+    constexpr int M = C::M, NC = C::NC, T = C::T, H = T / 2, SPW = C::SPW, CPT = C::CPT, EP = C::EP, EROW = C::EROW;
+    extern __shared__ __align__(128) unsigned char f1_smem_w[];
+    __shared__ __align__(8) unsigned long long bar_storage[C::WARPS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, len = p.len;
+    const uint32_t bar = fk_smem_u32(&bar_storage[warp]);
+    unsigned char* mine = f1_smem_w + (size_t)warp * (2 * C::EXCH_BYTES + C::IN_BYTES);
+    float2* sIn = reinterpret_cast<float2*>(mine + 2 * C::EXCH_BYTES);
+    if (lane == 0) {
+        fk_mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    const F1WarpRoles<N> ro(lane);
+    const int t = ro.t;
+    const bool t0 = t == 0;
+    float tc[CPT][T], ts[CPT][T];                           // w_M^{-cls r} = (tc, +ts)
+#pragma unroll
+    for (int c = 0; c < CPT; ++c)
+#pragma unroll
+        for (int r = 1; r < T; ++r) sincospif(2.0f * (float)(ro.cls[c] * r) / (float)M, &ts[c][r], &tc[c][r]);
+    const float scale = p.scale;
+    const bool acc = p.accumulate != 0;
+
+    const long long groups = (p.batch + SPW - 1) / SPW, stride = (long long)gridDim.x * C::WARPS;
+    auto count = [&](long long g) { const long long left = p.batch - g * SPW; return left < SPW ? (int)left : SPW; };
+    auto fetch = [&](long long g) {
+        const int c = count(g);
+        return f1w_fetch(reinterpret_cast<float*>(sIn), reinterpret_cast<const float*>(p.spec_in + g * SPW * NC), c * NC * 2,
+                         c == SPW, bar, lane);
+    };
+    long long g = (long long)blockIdx.x * C::WARPS + warp;
+    bool pending = g < groups ? fetch(g) : false;
+    uint32_t phase = 0;
+    for (int buf = 0; g < groups; g += stride, buf ^= 1) {
+        unsigned char* region = mine + buf * C::EXCH_BYTES;
+        __syncwarp();
+        if (pending) {
+            if (!fk_mbar_wait(bar, phase, 0)) break;
+            phase ^= 1u;
+        }
+        // pre-pass: Z'_k = (X_k + conj X_{M-k}) + i w_N^{-k} (X_k - conj X_{M-k}), pair by pair
+        float Pr[8], Pi[8], Qr[8], Qi[8];
+        const float2* x = sIn + ro.s * NC;
+        static_for<8>([&](auto Pp) {
+            constexpr int q = decltype(Pp)::value;
+            float2 a = x[ro.kp[q]], b = x[M - ro.kp[q]];
+            if constexpr (q == 0) { a.y = t0 ? 0.0f : a.y; b.y = t0 ? 0.0f : b.y; }     // bins 0 and n/2
+            const float er = a.x + b.x, ei = a.y - b.y, dr = a.x - b.x, di = a.y + b.y;
+            const float ur = fc_fma(-ro.ps[q], di, ro.pc[q] * dr), ui = fc_fma(ro.ps[q], dr, ro.pc[q] * di);
+            Pr[q] = er - ui; Pi[q] = ei + ur;
+            Qr[q] = er + ui; Qi[q] = ur - ei;
+        });
+        const float2 mid = x[M / 2];
+        float Zr[CPT][T], Zi[CPT][T];
+        static_for<T>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            Zr[0][i] = Pr[i]; Zi[0][i] = Pi[i];
+            if constexpr (i == H) { Zr[0][i] = t0 ? 2.0f * mid.x : Pr[i]; Zi[0][i] = t0 ? -2.0f * mid.y : Pi[i]; }
+            if constexpr (i > H)  { Zr[0][i] = t0 ? Qr[T - i] : Pr[i]; Zi[0][i] = t0 ? Qi[T - i] : Pi[i]; }
+            if constexpr (i < H) { Zr[1][i] = t0 ? Pr[i + H] : Qr[T - 1 - i]; Zi[1][i] = t0 ? Pi[i + H] : Qi[T - 1 - i]; }
+            else { Zr[1][i] = t0 ? Qr[T - 1 - i + H] : Qr[T - 1 - i]; Zi[1][i] = t0 ? Qi[T - 1 - i + H] : Qi[T - 1 - i]; }
+            if constexpr (CPT == 4) {
+                Zr[2][i] = Pr[T + i]; Zi[2][i] = Pi[T + i];
+                Zr[3][i] = Qr[T + T - 1 - i]; Zi[3][i] = Qi[T + T - 1 - i];
+            }
+        });
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // this buffer's last store
+        __syncwarp();                       // ... and every lane has its bins
+        pending = g + stride < groups ? fetch(g + stride) : false;
+        float2* e = reinterpret_cast<float2*>(region) + ro.s * EP;
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) {
+            cfft<T, true>(Zr[c], Zi[c]);
+            float2* a = e + ro.cls[c] * EROW;
+            static_for<T>([&](auto R) {
+                constexpr int r = decltype(R)::value;
+                if constexpr (r == 0) a[0] = make_float2(Zr[c][0], Zi[c][0]);
+                else a[r] = make_float2(fc_fma(-ts[c][r], Zi[c][r], tc[c][r] * Zr[c][r]), fc_fma(ts[c][r], Zr[c][r], tc[c][r] * Zi[c][r]));
+            });
+        }
+        __syncwarp();
+        float zr[16], zi[16];
+        static_for<16>([&](auto K) {
+            constexpr int k = decltype(K)::value;
+            const float2 v = e[k * EROW + t];
+            zr[k] = v.x; zi[k] = v.y;
+        });
+        cfft<16, true>(zr, zi);             // z_{t + T m} = x_{2(t + T m)} + i x_{2(t + T m) + 1}, times N
+        __syncwarp();                       // the exchange is over: the buffer becomes the samples
+        float* img = reinterpret_cast<float*>(region);
+        {
+            float* row = img + ro.s * len + 2 * t;
+            const int left = len - 2 * t;
+            if ((len & 1) == 0) {
+                static_for<16>([&](auto Mm) {
+                    constexpr int m = decltype(Mm)::value, o = 2 * T * m;
+                    if (o < left) *reinterpret_cast<float2*>(row + o) = make_float2(zr[m] * scale, zi[m] * scale);
+                });
+            } else {
+                static_for<16>([&](auto Mm) {
+                    constexpr int m = decltype(Mm)::value, o = 2 * T * m;
+                    if (o < left) row[o] = zr[m] * scale;
+                    if (o + 1 < left) row[o + 1] = zi[m] * scale;
+                });
+            }
+        }
+        const int cnt = count(g);
+        float* dst = p.real_out + g * SPW * len;
+        if (!acc && cnt == SPW && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) fk_bulk_s2g(dst, fk_smem_u32(img), (uint32_t)(SPW * len * 4));
+        } else {
+            __syncwarp();
+            for (int i = lane; i < cnt * len; i += 32) dst[i] = acc ? dst[i] + img[i] : img[i];
+        }
+        if (lane == 0) fk_bulk_commit();
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+template <int N>
+static cudaError_t launch_fft1d_warp(const Fft1dParams& p, bool inverse, cudaStream_t st) {
+    using C = F1Warp<N>;
+    const long long groups = (p.batch + C::SPW - 1) / C::SPW;
+    auto kern = inverse ? fft1d_warp_c2r_kernel<N> : fft1d_warp_r2c_kernel<N>;
+    int grid = 0;
+    const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(kern), 32 * C::WARPS, C::SMEM,
+                                          (groups + C::WARPS - 1) / C::WARPS, &grid);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, 32 * C::WARPS, C::SMEM, st>>>(p);
+    return cudaGetLastError();
 }
 
 template <int N>
@@ -285,8 +508,8 @@ static cudaError_t launch_fft1d(int n, const Fft1dParams& p, bool inverse, cudaS
         case 16:  return launch_fft1d_n<16>(p, inverse, st);
         case 32:  return launch_fft1d_n<32>(p, inverse, st);
         case 64:  return launch_fft1d_n<64>(p, inverse, st);
-        case 128: return launch_fft1d_n<128>(p, inverse, st);
-        case 256: return launch_fft1d_n<256>(p, inverse, st);
+        case 128: return launch_fft1d_warp<128>(p, inverse, st);
+        case 256: return launch_fft1d_warp<256>(p, inverse, st);
     }
     return cudaErrorInvalidValue;
 }

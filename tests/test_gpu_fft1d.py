@@ -112,3 +112,25 @@ def test_argument_checks():
     assert L.fft1d_r2c(z, one, 1, 8, 8, z) == b.EINVAL
     assert L.fft1d_c2r(one, one, 1, 8, 9, 1.0, 0, z) == b.EINVAL
     assert L.fft1d_c2r(one, one, 0, 8, 8, 1.0, 0, z) == b.EINVAL
+
+
+@pytest.mark.parametrize("n", [128, 256])
+@pytest.mark.parametrize("batch,ln", [(1, 1), (3, 2), (4, 101), (8, 66), (9, 97), (2600, 120), (5000, 127)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_signals_shared_by_a_warp(n, batch, ln, offset):
+    """Groups of 32 / (n / 32) signals per warp: a ragged last group, lengths of either parity, more
+    groups than resident warps, tensors that do not start on a 16-byte boundary."""
+    import torch
+    import oracle
+    import paper_1412_7580_b200 as fc
+    from paper_1412_7580_b200 import workloads as wl
+    x = wl.make_planes(batch, 1, ln, seed=n + batch + ln)[:, 0, :].copy()
+    xd = torch.empty(batch * ln + offset, device="cuda")[offset:].view(batch, ln)
+    xd.copy_(torch.from_numpy(x))
+    X = torch.full((batch * (n // 2 + 1) + offset, 2), float("nan"), device="cuda")[offset:].view(batch, n // 2 + 1, 2)
+    back = torch.full((batch * ln + offset,), float("nan"), device="cuda")[offset:].view(batch, ln)
+    fc.fft1d_r2c(xd, X, n)
+    fc.fft1d_c2r(X, back, n, 1.0 / n)
+    got = X.cpu().numpy().astype(np.float64)
+    assert relerr(got[..., 0] + 1j * got[..., 1], oracle.dft1d_r2c(x, n)) <= TOL
+    assert relerr(back.cpu().numpy().astype(np.float64), x.astype(np.float64)) <= TOL
