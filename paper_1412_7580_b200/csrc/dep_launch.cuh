@@ -32,26 +32,40 @@ __device__ __forceinline__ void dep_wait() {
 //    1-7 % shorter passes at n <= 64 with the tensor-core contraction;
 //  * the forward transforms as dependents of the previous pass's inverse transform gain
 //    nothing at n <= 32, and at n = 64 a training step took 1.14 ms instead of 0.74;
-//  * with the two-pass transforms (n = 128) a pass is 0.5 % longer with the contraction as a
+//  * at n = 128 a pass is 0.5 % longer with the contraction as a
 //    dependent and 2.5 % longer with the inverse transform as one (2-6 % over the sweep);
 //  * the FFMA contraction at n <= 16 with a long reduction (K > 64) loses up to 12 % (its
 //    small CTAs share SMs with the waiting CTAs of the inverse transform); with K <= 64 the
 //    passes are shorter (24 -> 21 us on an S8 f4 f'8 16 x 16 layer).
 // The callers set the flag accordingly; everything else is launched the plain way.
 template <typename... KArgs, typename... Args>
-static cudaError_t dep_launch(bool overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t st, Args&&... args) {
+static cudaError_t dep_launch(bool overlap, int cluster, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (overlap) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = overlap ? 1 : 0;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t dep_launch(bool overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t st, Args&&... args) {
+    return dep_launch(overlap, 1, kern, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 }  // namespace fc

@@ -10,17 +10,16 @@
 // X_k = sum_j x_j exp(-2 pi i jk/N), unnormalised; the inverse uses the
 // conjugate roots and is unnormalised as well (the caller applies 1/n^2).
 //
-// The functions are __host__ __device__ so the arithmetic can also be exercised
-// by a host-side unit harness; the product only ever runs them on the GPU.
+// The functions are templates over the value type V: float, or F2 (f32x2.cuh), which carries the
+// same element of two independent transforms through packed instructions -- twice the
+// transforms for the same number of issued instructions, bit for bit the same results.
 #pragma once
 
 #include <utility>
 
-#if defined(__CUDACC__)
-#define FC_HD __host__ __device__ __forceinline__
-#else
-#define FC_HD inline
-#endif
+#include "f32x2.cuh"
+
+#define FC_HD __device__ __forceinline__
 
 namespace fc {
 
@@ -90,13 +89,23 @@ constexpr int bitrev(int v, int bits) {
     return r;
 }
 
-FC_HD float fc_fma(float a, float b, float c) {
-#if defined(__CUDA_ARCH__)
-    return __fmaf_rn(a, b, c);
-#else
-    return __builtin_fmaf(a, b, c);
-#endif
+FC_HD float fc_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+// The operations the transforms are written in, for both value types; c is a compile-time constant.
+FC_HD float vfma(float c, float x, float y) { return __fmaf_rn(c, x, y); }
+FC_HD float vmul(float c, float x) { return c * x; }
+__host__ __device__ constexpr unsigned long long f2_const(float c) {
+    return ((unsigned long long)__builtin_bit_cast(unsigned, c) << 32) | __builtin_bit_cast(unsigned, c);
 }
+FC_HD F2 vfma(float c, F2 x, F2 y) { return f2_fma(F2{f2_const(c)}, x, y); }
+FC_HD F2 f2_mul(F2 x, F2 y) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.b) : "l"(x.b), "l"(y.b));
+    return r;
+}
+FC_HD F2 vmul(float c, F2 x) { return f2_mul(x, F2{f2_const(c)}); }
+// A complex value.
+template <class V> struct Cx { V x, y; };
 
 // ---------------------------------------------------------------------------
 // In-register complex FFT, radix-2 decimation in time.
@@ -105,14 +114,14 @@ FC_HD float fc_fma(float a, float b, float c) {
 // A butterfly with a non-trivial twiddle costs six FMAs:
 //   u' = u + w v  (two chained FMAs per component),  v' = 2u - u' (one FMA).
 // ---------------------------------------------------------------------------
-template <int N, bool INV>
-FC_HD void cfft(float (&re)[N], float (&im)[N]) {
+template <int N, bool INV, class V>
+FC_HD void cfft(V (&re)[N], V (&im)[N]) {
     static_assert(N >= 1 && (N & (N - 1)) == 0, "power of two");
     if constexpr (N == 1) {
         return;
     } else {
         constexpr int BITS = ilog2(N);
-        float br[N], bi[N];
+        V br[N], bi[N];
         static_for<N>([&](auto I) {
             constexpr int i = decltype(I)::value;
             br[i] = re[bitrev(i, BITS)];
@@ -126,7 +135,7 @@ FC_HD void cfft(float (&re)[N], float (&im)[N]) {
                 constexpr int j = b % half;
                 constexpr int p = (b / half) * len + j;
                 constexpr int q = p + half;
-                const float ur = br[p], ui = bi[p], vr = br[q], vi = bi[q];
+                const V ur = br[p], ui = bi[p], vr = br[q], vi = bi[q];
                 if constexpr (j == 0) {
                     br[p] = ur + vr; bi[p] = ui + vi;
                     br[q] = ur - vr; bi[q] = ui - vi;
@@ -143,11 +152,11 @@ FC_HD void cfft(float (&re)[N], float (&im)[N]) {
                     constexpr float c = Tw<len, j>::c;
                     constexpr float s = INV ? -Tw<len, j>::s : Tw<len, j>::s;
                     // w = (c, -s): w v = (c vr + s vi, c vi - s vr)
-                    const float nr = fc_fma(s, vi, fc_fma(c, vr, ur));
-                    const float ni = fc_fma(-s, vr, fc_fma(c, vi, ui));
+                    const V nr = vfma(s, vi, vfma(c, vr, ur));
+                    const V ni = vfma(-s, vr, vfma(c, vi, ui));
                     br[p] = nr; bi[p] = ni;
-                    br[q] = fc_fma(2.0f, ur, -nr);
-                    bi[q] = fc_fma(2.0f, ui, -ni);
+                    br[q] = vfma(2.0f, ur, -nr);
+                    bi[q] = vfma(2.0f, ui, -ni);
                 }
             });
         });
@@ -165,18 +174,18 @@ FC_HD void cfft(float (&re)[N], float (&im)[N]) {
 // z_j = x_2j + i x_2j+1, Z = FFT_M(z); with E = FFT of the even samples and O =
 // FFT of the odd samples, X_k = E_k + w_N^k O_k and X_{M-k} = conj(E_k - w_N^k O_k).
 // ---------------------------------------------------------------------------
-template <int N>
-FC_HD void rfft(const float (&x)[N], float (&Xr)[N / 2 + 1], float (&Xi)[N / 2 + 1]) {
+template <int N, class V>
+FC_HD void rfft(const V (&x)[N], V (&Xr)[N / 2 + 1], V (&Xi)[N / 2 + 1]) {
     constexpr int M = N / 2;
-    float zr[M], zi[M];
+    V zr[M], zi[M];
     static_for<M>([&](auto J) {
         constexpr int j = decltype(J)::value;
         zr[j] = x[2 * j];
         zi[j] = x[2 * j + 1];
     });
     cfft<M, false>(zr, zi);
-    Xr[0] = zr[0] + zi[0]; Xi[0] = 0.0f;
-    Xr[M] = zr[0] - zi[0]; Xi[M] = 0.0f;
+    Xr[0] = zr[0] + zi[0]; Xi[0] = V{};
+    Xr[M] = zr[0] - zi[0]; Xi[M] = V{};
     if constexpr (M >= 2) {
         Xr[M / 2] = zr[M / 2];
         Xi[M / 2] = -zi[M / 2];
@@ -186,16 +195,16 @@ FC_HD void rfft(const float (&x)[N], float (&Xr)[N / 2 + 1], float (&Xi)[N / 2 +
             constexpr int k = decltype(K)::value + 1;
             constexpr float hc = 0.5f * Tw<N, k>::c;
             constexpr float hs = 0.5f * Tw<N, k>::s;
-            const float ar = zr[k], ai = zi[k], brr = zr[M - k], bii = zi[M - k];
-            const float er = ar + brr, ei = ai - bii;     // 2 E_k
-            const float orr = ai + bii, oi = brr - ar;    // 2 O_k
+            const V ar = zr[k], ai = zi[k], brr = zr[M - k], bii = zi[M - k];
+            const V er = ar + brr, ei = ai - bii;     // 2 E_k
+            const V orr = ai + bii, oi = brr - ar;    // 2 O_k
             // T = (w_N^k / 2) * (2 O_k), w = (c, -s)
-            const float tr = fc_fma(hs, oi, hc * orr);
-            const float ti = fc_fma(-hs, orr, hc * oi);
-            Xr[k] = fc_fma(0.5f, er, tr);
-            Xi[k] = fc_fma(0.5f, ei, ti);
-            Xr[M - k] = fc_fma(0.5f, er, -tr);
-            Xi[M - k] = fc_fma(-0.5f, ei, ti);
+            const V tr = vfma(hs, oi, vmul(hc, orr));
+            const V ti = vfma(-hs, orr, vmul(hc, oi));
+            Xr[k] = vfma(0.5f, er, tr);
+            Xi[k] = vfma(0.5f, ei, ti);
+            Xr[M - k] = vfma(0.5f, er, -tr);
+            Xi[M - k] = vfma(-0.5f, ei, ti);
         });
     }
 }
@@ -206,27 +215,27 @@ FC_HD void rfft(const float (&x)[N], float (&Xr)[N / 2 + 1], float (&Xi)[N / 2 +
 // Z'_k = (X_k + conj X_{M-k}) + i w_N^{-k} (X_k - conj X_{M-k}); the
 // unnormalised inverse FFT_M of Z' is N (x_2j + i x_2j+1).
 // ---------------------------------------------------------------------------
-template <int N>
-FC_HD void irfft(const float (&Xr)[N / 2 + 1], const float (&Xi)[N / 2 + 1], float (&x)[N]) {
+template <int N, class V>
+FC_HD void irfft(const V (&Xr)[N / 2 + 1], const V (&Xi)[N / 2 + 1], V (&x)[N]) {
     constexpr int M = N / 2;
-    float zr[M], zi[M];
+    V zr[M], zi[M];
     zr[0] = Xr[0] + Xr[M];
     zi[0] = Xr[0] - Xr[M];
     if constexpr (M >= 2) {
-        zr[M / 2] = 2.0f * Xr[M / 2];
-        zi[M / 2] = -2.0f * Xi[M / 2];
+        zr[M / 2] = vmul(2.0f, Xr[M / 2]);
+        zi[M / 2] = vmul(-2.0f, Xi[M / 2]);
     }
     if constexpr (M >= 4) {
         static_for<M / 2 - 1>([&](auto K) {
             constexpr int k = decltype(K)::value + 1;
             constexpr float c = Tw<N, k>::c;
             constexpr float s = Tw<N, k>::s;
-            const float pr = Xr[k], pi = Xi[k], qr = Xr[M - k], qi = Xi[M - k];
-            const float er = pr + qr, ei = pi - qi;   // E = P + conj Q
-            const float dr = pr - qr, di = pi + qi;   // D = P - conj Q
+            const V pr = Xr[k], pi = Xi[k], qr = Xr[M - k], qi = Xi[M - k];
+            const V er = pr + qr, ei = pi - qi;   // E = P + conj Q
+            const V dr = pr - qr, di = pi + qi;   // D = P - conj Q
             // U = w_N^{-k} D with w^{-k} = (c, +s): U = (c dr - s di, c di + s dr)
-            const float ur = fc_fma(-s, di, c * dr);
-            const float ui = fc_fma(s, dr, c * di);
+            const V ur = vfma(-s, di, vmul(c, dr));
+            const V ui = vfma(s, dr, vmul(c, di));
             // Z'_k = E + iU = (er - ui, ei + ur); Z'_{M-k} = conj(E - iU) = (er + ui, -(ei - ur))
             zr[k] = er - ui;     zi[k] = ei + ur;
             zr[M - k] = er + ui; zi[M - k] = ur - ei;
@@ -241,38 +250,6 @@ FC_HD void irfft(const float (&Xr)[N / 2 + 1], const float (&Xi)[N / 2 + 1], flo
 }
 
 // ---------------------------------------------------------------------------
-// One decimation-in-frequency split of an N-point transform over two
-// cooperating threads: given all N inputs, thread q in {0,1} forms the N/2
-// inputs of the half-size transform whose outputs are X_{2k+q}:
-//   q = 0: a_j = x_j + x_{j+N/2}        q = 1: a_j = (x_j - x_{j+N/2}) w_N^{+-j}
-// ---------------------------------------------------------------------------
-template <int N, bool INV, int Q>
-FC_HD void dif_split(const float (&xr)[N], const float (&xi)[N], float (&ar)[N / 2],
-                     float (&ai)[N / 2]) {
-    constexpr int M = N / 2;
-    static_for<M>([&](auto J) {
-        constexpr int j = decltype(J)::value;
-        if constexpr (Q == 0) {
-            ar[j] = xr[j] + xr[j + M];
-            ai[j] = xi[j] + xi[j + M];
-        } else {
-            const float dr = xr[j] - xr[j + M], di = xi[j] - xi[j + M];
-            if constexpr (j == 0) {
-                ar[j] = dr; ai[j] = di;
-            } else if constexpr (4 * j == N) {
-                if constexpr (!INV) { ar[j] = di; ai[j] = -dr; }
-                else                { ar[j] = -di; ai[j] = dr; }
-            } else {
-                constexpr float c = Tw<N, j>::c;
-                constexpr float s = INV ? -Tw<N, j>::s : Tw<N, j>::s;
-                ar[j] = fc_fma(s, di, c * dr);
-                ai[j] = fc_fma(-s, dr, c * di);
-            }
-        }
-    });
-}
-
-// ---------------------------------------------------------------------------
 // Real-input FFT of length N split over two cooperating threads.  Both threads
 // see all N samples; thread Q in {0,1} returns the bins k = 2i + Q of the
 // Hermitian half 0..N/2 in O[i]: Q = 0 gets k = 0, 2, .., N/2 (N/4 + 1 bins),
@@ -283,36 +260,36 @@ FC_HD void dif_split(const float (&xr)[N], const float (&xi)[N], float (&ar)[N /
 // pairs Z_k with Z_{M-k}, and k and M-k have the same parity, so it stays inside
 // the thread.
 // ---------------------------------------------------------------------------
-template <int N, int Q, class Load>
-FC_HD void rfft_half_split(Load&& x, float (&ar)[N / 4], float (&ai)[N / 4]) {
+template <int N, int Q, class Load, class V>
+FC_HD void rfft_half_split(Load&& x, V (&ar)[N / 4], V (&ai)[N / 4]) {
     static_assert(N >= 8, "needs an even quarter length");
     constexpr int M = N / 2, H = M / 2;
     static_for<H>([&](auto J) {
         constexpr int j = decltype(J)::value;
-        const float lr = x(std::integral_constant<int, 2 * j>{});
-        const float li = x(std::integral_constant<int, 2 * j + 1>{});
-        const float hr = x(std::integral_constant<int, 2 * j + M>{});
-        const float hi = x(std::integral_constant<int, 2 * j + M + 1>{});
+        const V lr = x(std::integral_constant<int, 2 * j>{});
+        const V li = x(std::integral_constant<int, 2 * j + 1>{});
+        const V hr = x(std::integral_constant<int, 2 * j + M>{});
+        const V hi = x(std::integral_constant<int, 2 * j + M + 1>{});
         if constexpr (Q == 0) {
             ar[j] = lr + hr; ai[j] = li + hi;
         } else {
-            const float dr = lr - hr, di = li - hi;
+            const V dr = lr - hr, di = li - hi;
             if constexpr (j == 0) {
                 ar[j] = dr; ai[j] = di;
             } else if constexpr (4 * j == M) {
                 ar[j] = di; ai[j] = -dr;
             } else {
                 constexpr float c = Tw<M, j>::c, s = Tw<M, j>::s;
-                ar[j] = fc_fma(s, di, c * dr);
-                ai[j] = fc_fma(-s, dr, c * di);
+                ar[j] = vfma(s, di, vmul(c, dr));
+                ai[j] = vfma(-s, dr, vmul(c, di));
             }
         }
     });
 }
 // Second half of rfft_half: the N/4-point FFT and the Hermitian post-pass; every bin is
 // handed to emit(i, re, im) with i a compile-time index (bin k = 2i + Q) as soon as it exists.
-template <int N, int Q, class Emit>
-FC_HD void rfft_half_finish(float (&ar)[N / 4], float (&ai)[N / 4], Emit&& emit) {
+template <int N, int Q, class Emit, class V>
+FC_HD void rfft_half_finish(V (&ar)[N / 4], V (&ai)[N / 4], Emit&& emit) {
     constexpr int M = N / 2, H = M / 2;
     cfft<H, false>(ar, ai);                       // ar/ai[m] = Z_{2m+Q}
     auto pair = [&](auto K) {                     // bins k and M-k from Z_k and Z_{M-k}
@@ -320,17 +297,17 @@ FC_HD void rfft_half_finish(float (&ar)[N / 4], float (&ai)[N / 4], Emit&& emit)
         constexpr int m = (k - Q) / 2, mp = (M - k - Q) / 2;
         constexpr float hc = 0.5f * Tw<N, k>::c;
         constexpr float hs = 0.5f * Tw<N, k>::s;
-        const float pr = ar[m], pi = ai[m], qr = ar[mp], qi = ai[mp];
-        const float er = pr + qr, ei = pi - qi;       // 2 E_k
-        const float orr = pi + qi, oi = qr - pr;      // 2 O_k
-        const float tr = fc_fma(hs, oi, hc * orr);
-        const float ti = fc_fma(-hs, orr, hc * oi);
-        emit(std::integral_constant<int, m>{}, fc_fma(0.5f, er, tr), fc_fma(0.5f, ei, ti));
-        emit(std::integral_constant<int, mp>{}, fc_fma(0.5f, er, -tr), fc_fma(-0.5f, ei, ti));
+        const V pr = ar[m], pi = ai[m], qr = ar[mp], qi = ai[mp];
+        const V er = pr + qr, ei = pi - qi;       // 2 E_k
+        const V orr = pi + qi, oi = qr - pr;      // 2 O_k
+        const V tr = vfma(hs, oi, vmul(hc, orr));
+        const V ti = vfma(-hs, orr, vmul(hc, oi));
+        emit(std::integral_constant<int, m>{}, vfma(0.5f, er, tr), vfma(0.5f, ei, ti));
+        emit(std::integral_constant<int, mp>{}, vfma(0.5f, er, -tr), vfma(-0.5f, ei, ti));
     };
     if constexpr (Q == 0) {
-        emit(std::integral_constant<int, 0>{}, ar[0] + ai[0], 0.0f);          // k = 0
-        emit(std::integral_constant<int, H>{}, ar[0] - ai[0], 0.0f);          // k = M
+        emit(std::integral_constant<int, 0>{}, ar[0] + ai[0], V{});          // k = 0
+        emit(std::integral_constant<int, H>{}, ar[0] - ai[0], V{});          // k = M
         emit(std::integral_constant<int, H / 2>{}, ar[H / 2], -ai[H / 2]);    // k = M/2
         static_for<H / 2 - 1>([&](auto I) {            // k = 2, 4, .., M/2 - 2
             pair(std::integral_constant<int, 2 * (decltype(I)::value + 1)>{});
@@ -341,35 +318,24 @@ FC_HD void rfft_half_finish(float (&ar)[N / 4], float (&ai)[N / 4], Emit&& emit)
         });
     }
 }
-template <int N, int Q, class Load>
-FC_HD void rfft_half(Load&& x, float (&Or)[N / 4 + 1], float (&Oi)[N / 4 + 1]) {
-    float ar[N / 4], ai[N / 4];
-    rfft_half_split<N, Q>(static_cast<Load&&>(x), ar, ai);
-    rfft_half_finish<N, Q>(ar, ai, [&](auto I, float re, float im) {
-        Or[decltype(I)::value] = re;
-        Oi[decltype(I)::value] = im;
-    });
-}
-
 // ---------------------------------------------------------------------------
 // One radix-4 decimation-in-frequency step of an N-point complex transform split
 // over four cooperating threads.  All threads see the N inputs through load(j)
-// (a float2); thread Q in {0..3} forms the N/4 inputs of the quarter-size
+// (a complex value); thread Q in {0..3} forms the N/4 inputs of the quarter-size
 // transform whose outputs are X_{4m+Q}:
 //   a_j = (x_j + u^Q x_{j+L} + u^2Q x_{j+2L} + u^3Q x_{j+3L}) w_N^{+-Qj},  L = N/4,
 // with u = -i forward and +i inverse.
 // ---------------------------------------------------------------------------
-template <int N, bool INV, int Q, int J>
-FC_HD void split4_elem(const float2 x0, const float2 x1, const float2 x2, const float2 x3, float& outr,
-                       float& outi) {
-    float tr, ti;
+template <int N, bool INV, int Q, int J, class C, class V>
+FC_HD void split4_elem(const C x0, const C x1, const C x2, const C x3, V& outr, V& outi) {
+    V tr, ti;
     if constexpr (Q == 0) {
         tr = (x0.x + x2.x) + (x1.x + x3.x); ti = (x0.y + x2.y) + (x1.y + x3.y);
     } else if constexpr (Q == 2) {
         tr = (x0.x + x2.x) - (x1.x + x3.x); ti = (x0.y + x2.y) - (x1.y + x3.y);
     } else {
-        const float dr = x0.x - x2.x, di = x0.y - x2.y;     // x_j - x_{j+2L}
-        const float er = x1.x - x3.x, ei = x1.y - x3.y;     // x_{j+L} - x_{j+3L}
+        const V dr = x0.x - x2.x, di = x0.y - x2.y;     // x_j - x_{j+2L}
+        const V er = x1.x - x3.x, ei = x1.y - x3.y;     // x_{j+L} - x_{j+3L}
         // forward Q = 1 (inverse Q = 3): d - i e;   forward Q = 3 (inverse Q = 1): d + i e
         if constexpr ((Q == 1) != INV) { tr = dr + ei; ti = di - er; }
         else                           { tr = dr - ei; ti = di + er; }
@@ -380,18 +346,18 @@ FC_HD void split4_elem(const float2 x0, const float2 x1, const float2 x2, const 
         constexpr float c = Tw<N, Q * J>::c;
         constexpr float s = INV ? -Tw<N, Q * J>::s : Tw<N, Q * J>::s;
         // w = (c, -s): w t = (c tr + s ti, c ti - s tr)
-        outr = fc_fma(s, ti, c * tr);
-        outi = fc_fma(-s, tr, c * ti);
+        outr = vfma(s, ti, vmul(c, tr));
+        outi = vfma(-s, tr, vmul(c, ti));
     }
 }
-template <int N, bool INV, int Q, class Load>
-FC_HD void load_split4(Load&& load, float (&ar)[N / 4], float (&ai)[N / 4]) {
+template <int N, bool INV, int Q, class Load, class V>
+FC_HD void load_split4(Load&& load, V (&ar)[N / 4], V (&ai)[N / 4]) {
     constexpr int L = N / 4;
     static_for<L>([&](auto J) {
         constexpr int j = decltype(J)::value;
-        const float2 x0 = load(J), x1 = load(std::integral_constant<int, j + L>{});
-        const float2 x2 = load(std::integral_constant<int, j + 2 * L>{});
-        const float2 x3 = load(std::integral_constant<int, j + 3 * L>{});
+        const auto x0 = load(J), x1 = load(std::integral_constant<int, j + L>{});
+        const auto x2 = load(std::integral_constant<int, j + 2 * L>{});
+        const auto x3 = load(std::integral_constant<int, j + 3 * L>{});
         split4_elem<N, INV, Q, j>(x0, x1, x2, x3, ar[j], ai[j]);
     });
 }
@@ -399,33 +365,33 @@ FC_HD void load_split4(Load&& load, float (&ar)[N / 4], float (&ai)[N / 4]) {
 // ---------------------------------------------------------------------------
 // Inverse of the real-input FFT split over two cooperating threads (decimation
 // in time).  Thread Q in {0,1} reads the bins k = Q (mod 2) of the Hermitian half
-// through X(k) (a float2; X(0) must return (Re X_0, Re X_{N/2}) -- both bins are
+// through X(k) (a complex value; X(0) must return (Re X_0, Re X_{N/2}) -- both bins are
 // real), forms Z'_{2m+Q} with the pre-pass of irfft (k and M-k have the same
 // parity) and runs an M/2-point inverse FFT.  Result: Q = 0 returns E_j, Q = 1
 // returns w_M^{-j} O_j (j < M/2); then z_j = E_j + w^{-j} O_j and
 // z_{j+M/2} = E_j - w^{-j} O_j, with x_2j = Re z_j, x_2j+1 = Im z_j (times N).
 // ---------------------------------------------------------------------------
-template <int N, int Q, class LoadX>
-FC_HD void irfft_half(LoadX&& X, float (&er)[N / 4], float (&ei)[N / 4]) {
+template <int N, int Q, class LoadX, class V>
+FC_HD void irfft_half(LoadX&& X, V (&er)[N / 4], V (&ei)[N / 4]) {
     static_assert(N >= 8, "needs an even quarter length");
     constexpr int M = N / 2, H = M / 2;
     auto pair = [&](auto K) {
         constexpr int k = decltype(K)::value;
         constexpr int m = (k - Q) / 2, mp = (M - k - Q) / 2;
         constexpr float c = Tw<N, k>::c, s = Tw<N, k>::s;
-        const float2 P = X(K), Qv = X(std::integral_constant<int, M - k>{});
-        const float sr = P.x + Qv.x, si = P.y - Qv.y;   // P + conj Q
-        const float dr = P.x - Qv.x, di = P.y + Qv.y;   // P - conj Q
-        const float ur = fc_fma(-s, di, c * dr);        // w_N^{-k} D
-        const float ui = fc_fma(s, dr, c * di);
+        const auto P = X(K), Qv = X(std::integral_constant<int, M - k>{});
+        const V sr = P.x + Qv.x, si = P.y - Qv.y;   // P + conj Q
+        const V dr = P.x - Qv.x, di = P.y + Qv.y;   // P - conj Q
+        const V ur = vfma(-s, di, vmul(c, dr));        // w_N^{-k} D
+        const V ui = vfma(s, dr, vmul(c, di));
         er[m] = sr - ui;  ei[m] = si + ur;
         er[mp] = sr + ui; ei[mp] = ur - si;
     };
     if constexpr (Q == 0) {
-        const float2 dc = X(std::integral_constant<int, 0>{});
+        const auto dc = X(std::integral_constant<int, 0>{});
         er[0] = dc.x + dc.y; ei[0] = dc.x - dc.y;
-        const float2 mid = X(std::integral_constant<int, H>{});
-        er[H / 2] = 2.0f * mid.x; ei[H / 2] = -2.0f * mid.y;
+        const auto mid = X(std::integral_constant<int, H>{});
+        er[H / 2] = vmul(2.0f, mid.x); ei[H / 2] = vmul(-2.0f, mid.y);
         static_for<H / 2 - 1>([&](auto I) {
             pair(std::integral_constant<int, 2 * (decltype(I)::value + 1)>{});
         });
@@ -439,9 +405,9 @@ FC_HD void irfft_half(LoadX&& X, float (&er)[N / 4], float (&ei)[N / 4]) {
         static_for<H - 1>([&](auto J) {
             constexpr int j = decltype(J)::value + 1;
             constexpr float c = Tw<M, j>::c, s = Tw<M, j>::s;
-            const float a = er[j], b = ei[j];
-            er[j] = fc_fma(-s, b, c * a);
-            ei[j] = fc_fma(s, a, c * b);
+            const V a = er[j], b = ei[j];
+            er[j] = vfma(-s, b, vmul(c, a));
+            ei[j] = vfma(s, a, vmul(c, b));
         });
     }
 }

@@ -1,0 +1,304 @@
+// Forward 2-D R2C transform of large planes (n = 128) with the rows ky split over CTAs.
+//
+// The half spectrum of a tile of 8 planes (528 KB) does not fit shared memory, and 8 planes are the
+// least that give the frequency-major rows the 32 bytes the memory system needs.  So a work item is
+// a tile of 8 planes and ONE FOURTH of the rows ky: the rows (r, 8 - r) mod 8 for class r = 0 .. 3.
+// Every item reads all samples of its planes -- the four items of a tile run next to each other, so
+// that the samples come from HBM once and from the L2 three times -- but computes only its own rows:
+// the first butterflies of a decimation in frequency leave 16 of the 128 points of a column, one
+// 16-point transform yields the rows ky = 8m + r, m < 16, and those above n/2 are the conjugates of
+// the rows 8m' + (8 - r) (Section 5.2: Hermitian symmetry).  No work is done twice, except loads, and
+// nothing passes through a scratch area between the two 1-D passes.
+//
+// Per item, 512 threads, two planes per thread in packed fp32 pairs (f32x2.cuh):
+//   A. thread = (pair of planes, column): coalesced loads straight into the first butterflies,
+//      16-point FFT, 16 rows to shared memory ([pair][row][column], 16 bytes per element);
+//   B. thread = (row, t of 8): a 128-point row is 16 points per thread, a twiddle, an exchange in
+//      place (the slots a thread writes are the slots it has read), then 8 points for two residue
+//      classes; results form the staging tile [lo][part * n + kx][hi][plane], which overlays the rows;
+//   C. one TMA store per residue lo of the rows (ky = 8 hi + lo): boxes of 8 planes x 8 hi x 2n.
+// Row ky = 0 carries ky = n/2 as (re, im) and is taken apart in the staging tile.  The store of an
+// item overlaps phase A of the next.
+//
+// Bound by phase A: the rate at which the L2 hands out the samples (4 x the planes, 5 TB/s).  Measured
+// against the kernel it replaced (one CTA per tile, half spectrum through a scratch area in global
+// memory): 4,096 planes of 128 x 128 231 -> 215 us, 91 planes of 97 x 101 59 -> 22 us (a fourth of the
+// work per CTA and four times the CTAs), 150 planes of 120 x 117 50 -> 39 us.  Tried and not kept: rows
+// known to exist loaded without a test (30 instead of 49 M instructions for 2,048 planes, 4,096 planes
+// in 237 us: more loads at once, queued in the load unit), four threads per column with the next
+// planes' loads in flight (265 us), loads that bypass the L1 (267 us).
+#pragma once
+
+#include "fft_big.cuh"
+
+namespace fc {
+
+struct SplitGeom {
+    static constexpr int N = 128, M = 64, NC = 65, G = 8, PR = 4, T = 512, CLASSES = 4;
+    static constexpr int RP = N + 1;                     // 16-byte units per row (odd)
+    static constexpr int PP = 16 * RP + 2;               // per pair of planes (2 mod 8): 8 lanes = 2 rows x 4 pairs, conflict-free
+    static constexpr size_t MID = (size_t)PR * PP * 16;
+    static constexpr size_t STAGE = (size_t)2 * 2 * N * 8 * G * 4;
+    static constexpr size_t BUF = ((MID > STAGE ? MID : STAGE) + 127) / 128 * 128;
+    static constexpr size_t NY = (size_t)2 * N * G * 4;
+    static constexpr size_t SMEM = BUF + NY;
+};
+
+// w_128^{t k} for t < 8, k < 16, both components duplicated for packed operations
+struct SplitTwiddles { unsigned long long c[8][16], s[8][16]; };
+constexpr SplitTwiddles make_split_twiddles() {
+    SplitTwiddles w{};
+    for (int t = 0; t < 8; ++t)
+        for (int k = 0; k < 16; ++k) {
+            w.c[t][k] = f2_const(static_cast<float>(cx_cos2pi(t * k, 128)));
+            w.s[t][k] = f2_const(static_cast<float>(cx_sin2pi(t * k, 128)));
+        }
+    return w;
+}
+__constant__ SplitTwiddles c_split_tw = make_split_twiddles();
+// (re, im) times w = (c, -s)
+__device__ __forceinline__ void split_rotate(F2& re, F2& im, unsigned long long c_, unsigned long long s_) {
+    const F2 c{c_}, s{s_};
+    const F2 x = f2_fma(s, im, f2_mul(c, re));
+    im = f2_mul(c, im) - f2_mul(s, re);
+    re = x;
+}
+
+// [2][N][NC][R][ld] as (col, row, lo, hi, part*N + kx) with ky = 8 hi + lo
+static inline bool split_make_map(CUtensorMap* map, const float* spec, const FftParams& p) {
+    tc_encode_fn enc = tc_get_encode();
+    if (!enc) return false;
+    constexpr int N = SplitGeom::N, NC = SplitGeom::NC;
+    const cuuint64_t mat = (cuuint64_t)p.R * p.ld * 4;
+    cuuint64_t dims[5] = {(cuuint64_t)p.C, (cuuint64_t)p.R, 8, 8, (cuuint64_t)2 * N};
+    cuuint64_t strides[4] = {(cuuint64_t)p.ld * 4, mat, mat * 8, mat * NC};
+    cuuint32_t box[5] = {8u, 1u, 1u, 8u, (cuuint32_t)2 * N};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float*>(spec), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+__device__ __forceinline__ void fk_tma_store_5d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3, int c4) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];"
+        ::"l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+        : "memory");
+}
+
+// Phase A of class R: first butterflies of a column (x(row) -> both planes' sample), twiddles, 16-point
+// FFT; put(row, re, im) with row = 8 * (second residue) + hi; release() comes before the first put.
+template <int R, class Load, class Release, class Put>
+__device__ __forceinline__ void split_column(Load&& x, Release&& release, Put&& put) {
+    if constexpr (R == 0) {
+        F2 y[32], Xr[17], Xi[17];
+        static_for<16>([&](auto J) {
+            constexpr int j = decltype(J)::value;
+            auto at = [&](auto V) { return x(std::integral_constant<int, j + 16 * decltype(V)::value>{}); };
+            const F2 x0 = at(std::integral_constant<int, 0>{}), x1 = at(std::integral_constant<int, 1>{});
+            const F2 x2 = at(std::integral_constant<int, 2>{}), x3 = at(std::integral_constant<int, 3>{});
+            const F2 x4 = at(std::integral_constant<int, 4>{}), x5 = at(std::integral_constant<int, 5>{});
+            const F2 x6 = at(std::integral_constant<int, 6>{}), x7 = at(std::integral_constant<int, 7>{});
+            y[j] = (x0 + x4) + (x2 + x6);
+            y[j + 16] = (x1 + x5) + (x3 + x7);
+        });
+        rfft<32>(y, Xr, Xi);                                // X[k] = row ky = 4k
+        release();
+        put(std::integral_constant<int, 0>{}, Xr[0], Xr[16]);
+        static_for<15>([&](auto K) {
+            constexpr int k = decltype(K)::value + 1;
+            put(std::integral_constant<int, (k & 1) * 8 + k / 2>{}, Xr[k], Xi[k]);
+        });
+    } else {
+        F2 ar[16], ai[16];
+        static_for<16>([&](auto J) {
+            constexpr int j = decltype(J)::value;
+            auto at = [&](auto V) { return x(std::integral_constant<int, j + 16 * decltype(V)::value>{}); };
+            const F2 x0 = at(std::integral_constant<int, 0>{}), x1 = at(std::integral_constant<int, 1>{});
+            const F2 x2 = at(std::integral_constant<int, 2>{}), x3 = at(std::integral_constant<int, 3>{});
+            const F2 x4 = at(std::integral_constant<int, 4>{}), x5 = at(std::integral_constant<int, 5>{});
+            const F2 x6 = at(std::integral_constant<int, 6>{}), x7 = at(std::integral_constant<int, 7>{});
+            F2 re, im;                                      // sum_v x_v w_8^{R v}
+            if constexpr (R == 2) {
+                re = (x0 + x4) - (x2 + x6);
+                im = (x3 + x7) - (x1 + x5);
+            } else {
+                constexpr float s = Tw<8, 1>::c;
+                const F2 d0 = x0 - x4, d1 = x1 - x5, d3 = x3 - x7;
+                if constexpr (R == 1) {
+                    re = vfma(s, d1 - d3, d0);
+                    im = vfma(-s, d1 + d3, x6 - x2);
+                } else {
+                    re = vfma(s, d3 - d1, d0);
+                    im = vfma(-s, d1 + d3, x2 - x6);
+                }
+            }
+            if constexpr (j == 0) {
+                ar[0] = re; ai[0] = im;
+            } else {
+                constexpr float c = Tw<128, R * j>::c, sn = Tw<128, R * j>::s;
+                ar[j] = vfma(sn, im, vmul(c, re));
+                ai[j] = vfma(-sn, re, vmul(c, im));
+            }
+        });
+        cfft<16, false>(ar, ai);                            // row ky = 8m + R
+        release();
+        static_for<16>([&](auto Mm) {
+            constexpr int m = decltype(Mm)::value;
+            if constexpr (m < 8) put(std::integral_constant<int, m>{}, ar[m], ai[m]);
+            else put(std::integral_constant<int, 8 + 15 - m>{}, ar[m], -ai[m]);
+        });
+    }
+}
+
+__global__ void __launch_bounds__(SplitGeom::T, 1)
+r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUtensorMap tmNy0,
+                 const __grid_constant__ CUtensorMap tmS1, const __grid_constant__ CUtensorMap tmNy1,
+                 const FftParams p0, const FftParams p1) {
+    using Gm = SplitGeom;
+    constexpr int N = Gm::N, M = Gm::M, G = Gm::G, PR = Gm::PR, RP = Gm::RP, PP = Gm::PP;
+    extern __shared__ __align__(128) unsigned char fc_smem[];
+    ulonglong2* sMid = reinterpret_cast<ulonglong2*>(fc_smem);
+    unsigned long long* sStage = reinterpret_cast<unsigned long long*>(fc_smem);
+    unsigned long long* sNy = reinterpret_cast<unsigned long long*>(fc_smem + Gm::BUF);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int jA = tid / N, cA = tid - jA * N;              // A: pair of planes, column
+    const int blk = warp >> 3, t = warp & 7;                // B: residue of the rows, part of the row
+    ulonglong2* rowp = sMid + (lane & 3) * PP + (blk * 8 + (lane >> 2)) * RP;
+    const int items0 = Gm::CLASSES * p0.num_tiles, items = items0 + Gm::CLASSES * p1.num_tiles;
+
+    dep_trigger();
+    dep_wait();                     // no global access above this line
+
+    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+        const bool second = item >= items0;
+        const FftParams& p = second ? p1 : p0;
+        const int it = second ? item - items0 : item;
+        const int tile = it / Gm::CLASSES, cls = it - tile * Gm::CLASSES;
+        const int row = tile / p.tiles_per_row, c0 = (tile - row * p.tiles_per_row) * G;
+        const int h = p.h, w = p.w;
+
+        // ---- A: columns; a column past the plane reads no sample and writes zeros ----
+        {
+            const int left = p.C - c0 - 2 * jA;             // planes from this thread's pair on
+            const int live = (left > 0 && cA < w) ? h : 0;
+            const float* s0 = p.real_in + ((size_t)row * p.C + c0 + (left > 0 ? 2 * jA : 0)) * (size_t)(h * w) + cA;
+            const int other = left > 1 ? h * w : 0;
+            auto x = [&](auto Row) -> F2 {
+                constexpr int r = decltype(Row)::value;
+                float u = 0.0f, v = 0.0f;
+                if (r < live) {
+                    const float* q = s0 + r * w;
+                    u = __ldg(q);
+                    v = __ldg(q + other);
+                }
+                return f2_pack(u, v);
+            };
+            auto release = [&]() {  // the previous item's store has read the buffer
+                if (tid == 0) fk_bulk_wait_read();
+                __syncthreads();
+            };
+            ulonglong2* dst = sMid + jA * PP + cA;
+            auto put = [&](auto K, F2 re, F2 im) { dst[decltype(K)::value * RP] = make_ulonglong2(re.b, im.b); };
+            if (cls == 0)      split_column<0>(x, release, put);
+            else if (cls == 1) split_column<1>(x, release, put);
+            else if (cls == 2) split_column<2>(x, release, put);
+            else               split_column<3>(x, release, put);
+        }
+        __syncthreads();
+
+        // ---- B: rows ----
+        {
+            F2 ar[16], ai[16];
+            static_for<16>([&](auto Mm) {
+                constexpr int m = decltype(Mm)::value;
+                const ulonglong2 v = rowp[t + 8 * m];
+                ar[m].b = v.x; ai[m].b = v.y;
+            });
+            cfft<16, false>(ar, ai);
+            static_for<16>([&](auto K) {
+                constexpr int k = decltype(K)::value;
+                if constexpr (k == 0) {
+                    rowp[t] = make_ulonglong2(ar[0].b, ai[0].b);
+                } else {
+                    split_rotate(ar[k], ai[k], c_split_tw.c[t][k], c_split_tw.s[t][k]);
+                    rowp[8 * k + t] = make_ulonglong2(ar[k].b, ai[k].b);
+                }
+            });
+        }
+        __syncthreads();
+        {
+            F2 zr[2][8], zi[2][8];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                static_for<8>([&](auto U) {
+                    const ulonglong2 v = rowp[8 * (t + 8 * c) + decltype(U)::value];
+                    zr[c][decltype(U)::value].b = v.x; zi[c][decltype(U)::value].b = v.y;
+                });
+                cfft<8, false>(zr[c], zi[c]);               // F[kx = t + 8c + 16r]
+            }
+            __syncthreads();                                // the rows are in registers: the buffer becomes the staging tile
+            unsigned long long* o = sStage + ((size_t)(blk * 2 * N) + t) * (8 * PR) + lane;
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                static_for<8>([&](auto Rr) {
+                    constexpr int r = decltype(Rr)::value;
+                    o[(8 * c + 16 * r) * (8 * PR)] = zr[c][r].b;
+                    o[(N + 8 * c + 16 * r) * (8 * PR)] = zi[c][r].b;
+                });
+        }
+        if (cls == 0) {
+            // row ky = 0 of every plane holds Z = FFT(X_0 + i X_{N/2}):
+            // X_0[k] = (Z_k + conj Z_{-k}) / 2,  X_{N/2}[k] = (Z_k - conj Z_{-k}) / (2i)
+            __syncthreads();
+            if (tid < PR * (M + 1)) {
+                const int j = tid & (PR - 1), k = tid >> 2, kp = (N - k) & (N - 1);
+                constexpr int PITCH = 8 * PR;
+                unsigned long long* a = sStage + j;
+                const F2 fr{a[k * PITCH]}, fi{a[(N + k) * PITCH]}, gr{a[kp * PITCH]}, gi{a[(N + kp) * PITCH]};
+                const F2 x0r = vmul(0.5f, fr + gr), x0i = vmul(0.5f, fi - gi), y0i = vmul(0.5f, gi - fi);
+                const F2 xnr = vmul(0.5f, fi + gi), xni = vmul(0.5f, gr - fr), yni = vmul(0.5f, fr - gr);
+                a[k * PITCH] = x0r.b;  a[(N + k) * PITCH] = x0i.b;
+                unsigned long long* b = sNy + j;
+                b[k * PR] = xnr.b;  b[(N + k) * PR] = xni.b;
+                if (kp != k) {
+                    a[kp * PITCH] = x0r.b; a[(N + kp) * PITCH] = y0i.b;
+                    b[kp * PR] = xnr.b; b[(N + kp) * PR] = yni.b;
+                }
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (tid == 0) {
+            const CUtensorMap* tm = second ? &tmS1 : &tmS0;
+            const uint32_t src = fk_smem_u32(sStage);
+            fk_tma_store_5d(tm, src, c0, row, cls, 0, 0);
+            fk_tma_store_5d(tm, src + (uint32_t)(Gm::STAGE / 2), c0, row, cls == 0 ? 4 : 8 - cls, 0, 0);
+            if (cls == 0) fk_tma_store_4d(second ? &tmNy1 : &tmNy0, fk_smem_u32(sNy), c0, row, M, 0);
+            fk_bulk_commit();
+        }
+    }
+    if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
+// Forward transform of one operand, or of two in one launch (pb may be null).
+static cudaError_t launch_r2c_split(FftParams pa, const FftParams* pb_in, cudaStream_t st) {
+    using Gm = SplitGeom;
+    FftParams pb{};
+    CUtensorMap m[4];
+    memset(m, 0, sizeof(m));
+    if (!fill_tiling<Gm::G>(pa)) return cudaErrorInvalidValue;
+    if (!split_make_map(&m[0], pa.spec_out, pa) || !big_make_map<128>(&m[1], pa.spec_out, pa, 1)) return cudaErrorInvalidValue;
+    if (pb_in) {
+        pb = *pb_in;
+        if (!fill_tiling<Gm::G>(pb)) return cudaErrorInvalidValue;
+        if (!split_make_map(&m[2], pb.spec_out, pb) || !big_make_map<128>(&m[3], pb.spec_out, pb, 1)) return cudaErrorInvalidValue;
+    }
+    const long long items = (long long)Gm::CLASSES * ((long long)pa.num_tiles + pb.num_tiles);
+    if (items > 0x3fffffffLL) return cudaErrorInvalidValue;
+    int grid = 0;
+    const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(r2c_split_kernel), Gm::T, Gm::SMEM, items, &grid);
+    if (e != cudaSuccess) return e;
+    return dep_launch(false, r2c_split_kernel, dim3(grid), dim3(Gm::T), Gm::SMEM, st, m[0], m[1], m[2], m[3], pa, pb);
+}
+
+}  // namespace fc

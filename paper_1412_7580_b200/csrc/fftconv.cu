@@ -15,6 +15,7 @@
 #include "cgemm_tc.cuh"
 #include "fft_kernels.cuh"
 #include "fft_big.cuh"
+#include "fft_split.cuh"
 #include "fft_small.cuh"
 #include "fft_sub.cuh"
 #include "fft1d.cuh"
@@ -246,22 +247,19 @@ int run_pass(conv_plan_s* plan, int pass, const float* a_in, const float* b_in, 
     };
     const bool timing = plan->timing && plan->ev_made;
     auto mark = [&](int i) { if (timing) cudaEventRecord(plan->ev[i], st); };
-    // large planes run the two-pass transforms (one launch per operand, scratch behind the spectra)
+    // large planes: forward transform with the rows split over CTAs, inverse transform through a scratch
+    // area behind the spectra
     const bool tiled = plan->n != plan->n_full;
     const bool big = !tiled && fc::big_uses_two_pass(plan->n);
     float* scratch = reinterpret_cast<float*>(base + align_up(spectra_bytes(plan), kAlign));
     const size_t scratch_bytes = tiled ? 0 : fc::big_scratch_bytes(plan->n);
-    // One forward launch: both operands in one kernel (one-pass transforms), or one operand.
+    // One forward launch: both operands in one kernel, or one operand.
     auto forward = [&](const fc::FftParams& pa, const fc::FftParams* pb) -> cudaError_t {
-        g_launches.fetch_add((big && pb) ? 2 : 1, std::memory_order_relaxed);
-        if (!big) {
-            // wide planes at n = 64: the sub-batched kernels (rows twice as long); else the plain ones
-            const cudaError_t es = fc::launch_r2c_sub_any(plan->n, pa, pb, st);
-            return es != cudaErrorNotSupported ? es : fc::launch_r2c<true>(plan->n, pa, pb, st);
-        }
-        cudaError_t e = fc::launch_r2c_two_pass(plan->n, pa, scratch, scratch_bytes, st);
-        if (e == cudaSuccess && pb) e = fc::launch_r2c_two_pass(plan->n, *pb, scratch, scratch_bytes, st);
-        return e;
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        if (big) return fc::launch_r2c_split(pa, pb, st);
+        // wide planes at n = 64: the sub-batched kernels (rows twice as long); else the plain ones
+        const cudaError_t es = fc::launch_r2c_sub_any(plan->n, pa, pb, st);
+        return es != cudaErrorNotSupported ? es : fc::launch_r2c<true>(plan->n, pa, pb, st);
     };
     // Small planes (the filters of fprop and bprop) take the pruned-DFT kernel, whose stores are
     // whole 128-byte lines; it runs after the other operand's transform, as its programmatic
@@ -384,7 +382,7 @@ int run_pass(conv_plan_s* plan, int pass, const float* a_in, const float* b_in, 
     // whose loads are whole 128-byte lines; everything else the butterfly kernels
     cudaError_t ie = plan->small_planes ? fc::launch_c2r_small(plan->n, ip, st) : cudaErrorNotSupported;
     if (ie == cudaErrorNotSupported)
-        ie = big ? fc::launch_c2r_two_pass(plan->n, ip, scratch, scratch_bytes, st)
+        ie = big ? fc::launch_c2r_big(ip, scratch, scratch_bytes, st)
                  : fc::launch_c2r<true>(plan->n, ip, st);
     if (ie != cudaSuccess) return FFTCONV_ECUDA;
     mark(4);

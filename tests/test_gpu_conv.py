@@ -247,3 +247,20 @@ def test_steps_back_to_back_without_synchronisation(dims):
         assert relerr(dx.cpu().numpy().astype(np.float64), oracle.bprop(dy, w, s.h, s.w)) <= TOL[eff[1]]
         assert relerr(dw.cpu().numpy().astype(np.float64), oracle.accgrad(dy, x, s.kh, s.kw)) <= TOL[eff[2]]
     fc.conv_plan_destroy(p)
+
+
+@pytest.mark.parametrize("dims", [
+    # S, f, fp, h, w, kh, kw, n: tiles of 8 planes shared by clusters of 8, 4 and 2 CTAs; one plane, an odd
+    # number of planes, a full tile and one plane more; planes shorter or narrower than half of the basis
+    (1, 1, 1, 128, 128, 3, 3, 128), (1, 9, 8, 30, 128, 14, 15, 128), (2, 3, 17, 128, 20, 16, 3, 128),
+    (25, 1, 2, 66, 65, 3, 3, 128), (40, 2, 1, 65, 67, 5, 3, 128),
+])
+def test_large_planes_at_the_edges_of_their_tiles(dims):
+    import oracle
+    from paper_1412_7580_b200 import workloads as wl
+    s = wl.ConvShape("large", *dims, cfg=7, point=sum(dims))
+    x, w, dy = wl.make_x(s), wl.make_w(s), wl.make_dy(s)
+    y, dx, dw, eff = run_gpu(s, x, w, dy, 1)
+    assert relerr(y, oracle.fprop(x, w)) <= TOL[eff[0]]
+    assert relerr(dx, oracle.bprop(dy, w, s.h, s.w)) <= TOL[eff[1]]
+    assert relerr(dw, oracle.accgrad(dy, x, s.kh, s.kw)) <= TOL[eff[2]]
