@@ -1,0 +1,222 @@
+// Per-bin complex contraction with FP32 FFMA for small matrices (operands and layouts as in
+// cgemm_ffma.cuh): one warp per tile of one bin, WM x WN outputs with WM = 4 .. 64 and WM * WN = 256.
+//
+// With few samples or few planes a bin's matrices are a few kilobytes and there are thousands of bins,
+// so what counts is not to multiply padding: a tile of 64 x 64 (cgemm_ffma.cuh) or 128 x 128
+// (cgemm_tc.cuh) costs the same whatever it holds.  Here the tile shape follows the matrix (the WM that
+// pads the least), every warp works alone (no CTA barrier), and the copies of the next k-block -- of
+// the same tile or of the warp's next one -- are in flight while a block is multiplied.  A lane owns 4 rows
+// x 2 columns; rows are packed in pairs (fma.f32x2), and the four real products of the complex one have
+// accumulators of their own, so that the conjugates are signs applied once at the end.
+#pragma once
+
+#include "cgemm_ffma.cuh"
+#include "fft_kernels.cuh"
+
+namespace fc {
+
+template <int WM>
+struct SmallGemm {
+    static constexpr int LM = WM / 4, LN = 32 / LM, WN = 2 * LN, BK = 8, WARPS = 4;
+    static constexpr int PA = WM + 4, PB = WN + 4;                  // floats per k-row in shared memory
+    static constexpr int STAGE = 2 * BK * (PA + PB);                // floats: A re, A im, B re, B im
+    static constexpr size_t SMEM = (size_t)WARPS * 2 * STAGE * sizeof(float);
+};
+
+template <int WM>
+__global__ void __launch_bounds__(128)
+cgemm_small_kernel(const GemmParams p, const int m_tiles, const int n_tiles, const int items) {
+    using Gm = SmallGemm<WM>;
+    constexpr int LN = Gm::LN, WN = Gm::WN, BK = Gm::BK, PA = Gm::PA, PB = Gm::PB;
+    extern __shared__ __align__(128) unsigned char fc_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* ring = reinterpret_cast<float*>(fc_smem) + (size_t)warp * 2 * Gm::STAGE;
+    const int lm = lane / LN, ln = lane - lm * LN;
+    const size_t planeA = (size_t)(p.transA ? p.K : p.M) * p.lda, planeB = (size_t)(p.transB ? p.K : p.N) * p.ldb,
+                 planeC = (size_t)p.M * p.ldc;
+    const size_t imA = (size_t)p.bins * planeA, imB = (size_t)p.bins * planeB, imC = (size_t)p.bins * planeC;
+    const int k_blocks = (p.K + BK - 1) / BK, stride = gridDim.x * Gm::WARPS;
+
+    dep_trigger();
+    dep_wait();                     // no global access above this line
+
+    auto locate = [&](int item, int& bin, int& m0, int& n0) {
+        const int nt = item % n_tiles, rest = item / n_tiles, b = rest / m_tiles;
+        n0 = nt * WN;
+        m0 = (rest - b * m_tiles) * WM;
+        bin = p.herm_n ? herm_bin(b, p.herm_n) : b;
+    };
+    // k-block of one operand -> [part][k][row]; rows and k past the edge are zero-filled.  A row-contiguous
+    // operand moves in 16-byte pieces (a piece that straddles the last row brings in padding, which only
+    // reaches outputs that are not stored), a k-contiguous one is transposed by 4-byte copies.
+    auto copy = [&](auto ROWS_, float* dst, const float* base, size_t im, int ld, bool trans, int r0, int rows, int k0) {
+        constexpr int ROWS = decltype(ROWS_)::value, PITCH = ROWS + 4;
+        if (trans) {
+            for (int i = lane; i < ROWS / 4 * BK; i += 32) {
+                const int kk = i / (ROWS / 4), r = 4 * (i - kk * (ROWS / 4));
+                const bool ok = (k0 + kk < p.K) && (r0 + r < rows);
+                const float* src = ok ? base + (size_t)(k0 + kk) * ld + r0 + r : base;
+                fg_cp<16>(dst + kk * PITCH + r, src, ok);
+                fg_cp<16>(dst + (BK + kk) * PITCH + r, src + im, ok);
+            }
+        } else {
+            for (int i = lane; i < ROWS * BK; i += 32) {
+                const int r = i / BK, kk = i - r * BK;
+                const bool ok = (k0 + kk < p.K) && (r0 + r < rows);
+                const float* src = ok ? base + (size_t)(r0 + r) * ld + k0 + kk : base;
+                fg_cp<4>(dst + kk * PITCH + r, src, ok);
+                fg_cp<4>(dst + (BK + kk) * PITCH + r, src + im, ok);
+            }
+        }
+    };
+    auto issue = [&](int item, int kb, int st) {
+        if (item < items) {
+            int bin, m0, n0;
+            locate(item, bin, m0, n0);
+            float* s = ring + st * Gm::STAGE;
+            copy(std::integral_constant<int, WM>{}, s, p.A + (size_t)bin * planeA, imA, p.lda, p.transA != 0, m0, p.M, kb * BK);
+            copy(std::integral_constant<int, WN>{}, s + 2 * BK * PA, p.B + (size_t)bin * planeB, imB, p.ldb, p.transB != 0, n0, p.N, kb * BK);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    int item = blockIdx.x * Gm::WARPS + warp, kb = 0, st = 0;
+    issue(item, 0, 0);
+    F2 rr[2][2], ii[2][2], ri[2][2], ir[2][2];          // [pair of rows][column]: ar br, ai bi, ar bi, ai br
+    while (item < items) {
+        const bool last = kb + 1 == k_blocks;
+        issue(last ? item + stride : item, last ? 0 : kb + 1, st ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        if (kb == 0) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) rr[i][j].b = ii[i][j].b = ri[i][j].b = ir[i][j].b = 0ull;
+        }
+        const float* sA = ring + st * Gm::STAGE + lm * 4;
+        const float* sB = ring + st * Gm::STAGE + 2 * BK * PA + ln * 2;
+#pragma unroll
+        for (int k = 0; k < BK; ++k) {
+            const ulonglong2 ar = *reinterpret_cast<const ulonglong2*>(sA + k * PA);
+            const ulonglong2 ai = *reinterpret_cast<const ulonglong2*>(sA + (BK + k) * PA);
+            const float2 br = *reinterpret_cast<const float2*>(sB + k * PB);
+            const float2 bi = *reinterpret_cast<const float2*>(sB + (BK + k) * PB);
+            const F2 b_r[2] = {f2_pack(br.x, br.x), f2_pack(br.y, br.y)}, b_i[2] = {f2_pack(bi.x, bi.x), f2_pack(bi.y, bi.y)};
+            const F2 a_r[2] = {F2{ar.x}, F2{ar.y}}, a_i[2] = {F2{ai.x}, F2{ai.y}};
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    rr[i][j] = f2_fma(a_r[i], b_r[j], rr[i][j]);
+                    ii[i][j] = f2_fma(a_i[i], b_i[j], ii[i][j]);
+                    ri[i][j] = f2_fma(a_r[i], b_i[j], ri[i][j]);
+                    ir[i][j] = f2_fma(a_i[i], b_r[j], ir[i][j]);
+                }
+        }
+        __syncwarp();                                   // stage st may be refilled
+        if (last) {
+            // (ar + i sa ai)(br + i sb bi), sa / sb = -1 for a conjugated operand:
+            // re = ar br - sa sb ai bi,  im = sb ar bi + sa ai br
+            int bin, m0, n0;
+            locate(item, bin, m0, n0);
+            const float sa = p.conjA ? -1.0f : 1.0f, sb = p.conjB ? -1.0f : 1.0f, sab = -sa * sb;
+            const int n = n0 + 2 * ln;
+            float* c = p.C + (size_t)bin * planeC + n;
+            auto put = [&](int m, float r0, float r1, float i0, float i1) {
+                if (m >= p.M || n >= p.N) return;
+                float* o = c + (size_t)m * p.ldc;
+                if (n + 1 < p.N) {
+                    *reinterpret_cast<float2*>(o) = make_float2(r0, r1);
+                    *reinterpret_cast<float2*>(o + imC) = make_float2(i0, i1);
+                } else {
+                    o[0] = r0;
+                    o[imC] = i0;
+                }
+            };
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                float re[2][2], im[2][2];               // [row of the pair][column]
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    float a0, a1, b0, b1;
+                    f2_unpack(rr[i][j], a0, a1); f2_unpack(ii[i][j], b0, b1);
+                    re[0][j] = fmaf(sab, b0, a0); re[1][j] = fmaf(sab, b1, a1);
+                    f2_unpack(ri[i][j], a0, a1); f2_unpack(ir[i][j], b0, b1);
+                    im[0][j] = fmaf(sa, b0, sb * a0); im[1][j] = fmaf(sa, b1, sb * a1);
+                }
+                const int m = m0 + 4 * lm + 2 * i;
+                put(m, re[0][0], re[0][1], im[0][0], im[0][1]);
+                put(m + 1, re[1][0], re[1][1], im[1][0], im[1][1]);
+            }
+            item += stride;
+            kb = 0;
+        } else {
+            ++kb;
+        }
+        st ^= 1;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Tile height that pads an M x N matrix the least, and the padded area.
+static inline int small_gemm_shape(int M, int N, long long& area) {
+    int best = 0;
+    area = 0;
+    for (int wm = 4; wm <= 64; wm *= 2) {
+        const int wn = 256 / wm;
+        const long long a = (long long)((M + wm - 1) / wm * wm) * ((N + wn - 1) / wn * wn);
+        if (best == 0 || a < area) { best = wm; area = a; }
+    }
+    return best;
+}
+
+template <int WM>
+static cudaError_t launch_cgemm_small_t(const GemmParams& p, cudaStream_t st) {
+    using Gm = SmallGemm<WM>;
+    const int m_tiles = (p.M + WM - 1) / WM, n_tiles = (p.N + Gm::WN - 1) / Gm::WN;
+    const long long items = (long long)(p.herm_n ? herm_kept_bins(p.herm_n) : p.bins) * m_tiles * n_tiles;
+    if (items > 0x3fffffffLL) return cudaErrorInvalidValue;
+    auto kern = cgemm_small_kernel<WM>;
+    int grid = 0;
+    const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(kern), 128, Gm::SMEM, (items + Gm::WARPS - 1) / Gm::WARPS, &grid);
+    if (e != cudaSuccess) return e;
+    return dep_launch(p.overlap != 0, kern, dim3(grid), dim3(128), Gm::SMEM, st, p, m_tiles, n_tiles, (int)items);
+}
+static cudaError_t launch_cgemm_small(const GemmParams& p, cudaStream_t st) {
+    if (p.herm_n && (p.herm_n < 8 || p.bins != p.herm_n * (p.herm_n / 2 + 1))) return cudaErrorInvalidValue;
+    long long area;
+    switch (small_gemm_shape(p.M, p.N, area)) {
+        case 4:  return launch_cgemm_small_t<4>(p, st);
+        case 8:  return launch_cgemm_small_t<8>(p, st);
+        case 16: return launch_cgemm_small_t<16>(p, st);
+        case 32: return launch_cgemm_small_t<32>(p, st);
+        default: return launch_cgemm_small_t<64>(p, st);
+    }
+}
+
+// Where the small tiles are faster, from the rates measured on B200 (bins of n = 64, microseconds, small /
+// other): they reach about 15 TFLOP/s of padded multiply-adds (4-byte transposing copies of k-contiguous
+// operands included), the 64 x 64 tiles about 50, and a 128 x 128 tensor-core tile takes an SM about
+// 0.45 us plus 0.6 us per k-block of 32 whatever it holds.
+//   against 64 x 64 tiles: M, N, K = 4, 4, 194: 53 / 240;  4, 194, 4: 16 / 83;  32, 32, 32: 34 / 46;
+//                          64, 64, 16: 64 / 30
+//   against tensor cores:  1, 64, 16: 12 / 27;  16, 16, 16: 12 / 20;  4, 194, 4: 16 / 65;  7, 6, 42: 20 / 28;
+//                          32, 32, 32: 34 / 20;  2, 7, 310 (n = 32): 48 / 33
+static inline bool small_gemm_beats_ffma(int M, int N, int K) {
+    long long area;
+    small_gemm_shape(M, N, area);
+    const long long n64 = (N + 63) / 64 * 64, n96 = (N + 95) / 96 * 96;
+    const long long other = (long long)((M + 63) / 64 * 64) * (n96 < n64 ? n96 : n64);
+    return area * ((K + 7) / 8 * 8) * 50 < other * ((K + 15) / 16 * 16) * 15;
+}
+static inline bool small_gemm_beats_tc(int M, int N, int K) {
+    long long area;
+    small_gemm_shape(M, N, area);
+    const double tiles = (double)((M + 127) / 128) * ((N + 127) / 128);
+    const double tc_us = tiles / 148.0 * (0.45 + 0.6 * ((K + 31) / 32));
+    const double small_us = 8.0 * (double)area * ((K + 7) / 8 * 8) / 15e6;
+    return small_us < 0.8 * tc_us;
+}
+
+}  // namespace fc

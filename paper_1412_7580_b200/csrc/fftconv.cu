@@ -12,6 +12,7 @@
 #include <new>
 
 #include "cgemm_ffma.cuh"
+#include "cgemm_small.cuh"
 #include "cgemm_tc.cuh"
 #include "fft_kernels.cuh"
 #include "fft_big.cuh"
@@ -169,6 +170,14 @@ int resolve_math(const conv_plan_s& p, const PassDesc& d) {
     const bool fits = fc::tc_shape_supported(d.M, d.N, d.K);
     if (p.math == FFTCONV_MATH_TF32) return fits ? FFTCONV_MATH_TF32 : FFTCONV_MATH_FP32;
     return (fits && fc::tc_shape_profitable(d.M, d.N, d.K)) ? FFTCONV_MATH_TF32 : FFTCONV_MATH_FP32;
+}
+
+// The contraction of all (kept) bins.  `tensor`: TF32 precision is enough; matrices too small to fill a
+// tensor-core tile take the exact kernel with small tiles in either case.
+cudaError_t contract(const fc::GemmParams& gp, bool tensor, int* status, cudaStream_t st) {
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (tensor) return fc::small_gemm_beats_tc(gp.M, gp.N, gp.K) ? fc::launch_cgemm_small(gp, st) : fc::launch_cgemm_tc(gp, status, st);
+    return fc::small_gemm_beats_ffma(gp.M, gp.N, gp.K) ? fc::launch_cgemm_small(gp, st) : fc::launch_cgemm_ffma(gp, st);
 }
 
 size_t pass_bytes(const conv_plan_s& p, int pass) {
@@ -357,13 +366,9 @@ int run_pass(conv_plan_s* plan, int pass, const float* a_in, const float* b_in, 
         plan->cached[d.a.kind] = a_in;
         plan->cached[d.b.kind] = b_in;
     }
-    g_launches.fetch_add(1, std::memory_order_relaxed);
     gp.overlap = (overlap && (need_a || need_b)) ? 1 : 0;       // predecessor: this pass's forward transforms
     gp.herm_n = herm_n;
-    cudaError_t ge;
-    if (tensor) ge = fc::launch_cgemm_tc(gp, status, st);
-    else ge = fc::launch_cgemm_ffma(gp, st);
-    if (ge != cudaSuccess) return FFTCONV_ECUDA;
+    if (contract(gp, tensor, status, st) != cudaSuccess) return FFTCONV_ECUDA;
     }
     mark(3);
 
@@ -859,19 +864,12 @@ FFTCONV_API int fftconv_bin_contract(const float* A, const float* B, float* C, i
         eff = (fc::tc_shape_supported(M, N, K) && fc::tc_shape_profitable(M, N, K))
                   ? FFTCONV_MATH_TF32 : FFTCONV_MATH_FP32;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    cudaError_t e;
+    if (eff != FFTCONV_MATH_TF32 && eff != FFTCONV_MATH_FP32) return FFTCONV_EUNSUPPORTED;
     if (eff == FFTCONV_MATH_TF32) {
         if (!fc::tc_shape_supported(M, N, K)) return FFTCONV_EUNSUPPORTED;
         if (!status_word) return FFTCONV_EINVAL;
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        e = fc::launch_cgemm_tc(gp, status_word, st);
-    } else if (eff == FFTCONV_MATH_FP32) {
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        e = fc::launch_cgemm_ffma(gp, st);
-    } else {
-        return FFTCONV_EUNSUPPORTED;
     }
-    return e == cudaSuccess ? FFTCONV_OK : FFTCONV_ECUDA;
+    return contract(gp, eff == FFTCONV_MATH_TF32, status_word, st) == cudaSuccess ? FFTCONV_OK : FFTCONV_ECUDA;
 }
 
 FFTCONV_API const char* fftconv_status_string(int status) {

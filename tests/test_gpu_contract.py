@@ -87,3 +87,13 @@ FLAGS = [
                                    (4, 64, 96, 128), (2, 8, 8, 4)])
 def test_contraction_layouts_and_conjugates(shape, math, flags):
     assert run(*shape, math=math, seed=9, **flags) <= TOL[math]
+
+
+# tiles of one warp (4 x 64 .. 64 x 4): every tile shape, edges and remainders of rows, columns and k-blocks
+@pytest.mark.parametrize("flags", FLAGS)
+@pytest.mark.parametrize("math", [1, 2])
+@pytest.mark.parametrize("shape", [(40, 1, 1, 1), (9, 4, 64, 8), (9, 3, 65, 9), (9, 8, 32, 7), (9, 7, 33, 17), (9, 16, 16, 16),
+                                   (9, 15, 17, 3), (9, 32, 8, 24), (9, 33, 7, 2), (9, 64, 4, 8), (9, 70, 3, 5),
+                                   (5, 2, 3, 203), (3000, 2, 5, 3)])
+def test_contraction_of_small_matrices(shape, math, flags):
+    assert run(*shape, math=math, seed=11, **flags) <= TOL[math]
