@@ -23,7 +23,11 @@
 //               overlapped with the next tile's MMAs through two accumulator
 //               buffers (2 x 256 TMEM columns).
 // The per-bin problems are small and the kernel streams: it is bound by HBM
-// bytes (two spectra in, one out), not by tensor throughput.
+// bytes (two spectra in, one out), not by tensor throughput.  Matrices narrower
+// than a tile are fetched and multiplied only as far as they go (rows of the
+// boxes, N of the instructions, k-steps), which also makes room for a fourth stage:
+// M, N, K = 50, 90, 67 over the bins of n = 32 22.0 -> 18.5 us, 24, 100, 200 (n = 64)
+// 96 -> 83 us, 100, 10, 200 (n = 64) 88-120 -> 75-95 us; full tiles unchanged.
 //
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises the
 // caller's status word, drains what it issued, frees its tensor memory and
@@ -49,7 +53,10 @@ constexpr uint32_t TC_TILE_BYTES = TC_BM * TC_BK * 4;            // one 128 x 32
 constexpr uint32_t TC_STAGE_BYTES = 4 * TC_TILE_BYTES;           // A_re, A_im, B_re, B_im
 constexpr uint32_t TC_EPI_BUF_BYTES = 32 * 128;                  // 32 rows x 32 fp32, one TMA store box
 constexpr uint32_t TC_EPI_BYTES = 4 * 2 * TC_EPI_BUF_BYTES;      // 4 warps x 2 buffers
-constexpr uint32_t tc_smem_bytes(int stages) { return 1024 + stages * TC_STAGE_BYTES + TC_EPI_BYTES + 256; }
+// Narrow matrices leave room for more stages than three, but more than four do not pay (S64 f64 f'128,
+// n = 64: 62 us with three, 59 with four, 65 with six).
+constexpr int TC_MAX_STAGES = 4;
+constexpr uint32_t tc_smem_bytes(int stages) { return 1024 + stages * TC_STAGE_BYTES + TC_EPI_BYTES + 512; }
 constexpr uint32_t TC_SMEM_BYTES = tc_smem_bytes(TC_STAGES);
 // A launch that shares the SMs with a transform kernel (the filter spectrum produced range by range
 // beside the contraction) runs a ring of two stages and leaves 64 KB of shared memory to that kernel.
@@ -67,6 +74,12 @@ struct TcParams {
     int nc, ky_begin, ky_count; // ky_count > 0: local bin b -> kx = b / ky_count, ky = ky_begin + b % ky_count
     int late_trigger;           // let the dependent launch start after this one's wait instead of before it
     int herm_n;                 // > 0: the launch runs the kept bins of GemmParams::herm_n (local bin -> herm_bin)
+    // Matrices narrower than a tile: rows of A and B that are fetched, and columns that are multiplied.
+    // What lies beyond them in shared memory is left over from earlier stages and only reaches
+    // outputs that are not stored.
+    int rows_a, rows_b;         // K-major: rows of a TMA box; MN-major: a multiple of 32, one box each
+    int mma_n;                  // N of the instructions (multiple of 16)
+    int stages;                 // stages of the ring: as many as its shared memory holds, at most TC_MAX_STAGES
 };
 
 static inline bool tc_shape_supported(int M, int N, int K) {
@@ -195,7 +208,9 @@ __host__ __device__ constexpr uint32_t tc_idesc(int M, int N, bool negA, bool mn
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-template <bool TA, bool TB, int ST>
+// FULL: matrices of at least a tile in both directions; everything that TcParams says about the part of a
+// tile in use is then a constant (with run-time values the layers made of full tiles are 0.5 % slower).
+template <bool TA, bool TB, int ST, bool FULL>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ CUtensorMap tmC, const TcParams p) {
@@ -205,20 +220,24 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t epi = tiles + ST * TC_STAGE_BYTES;        // epilogue staging, 1024-aligned
     uint8_t* ctl = tc_raw + (tiles - raw_addr) + ST * TC_STAGE_BYTES + TC_EPI_BYTES;
     const uint32_t bars = epi + TC_EPI_BYTES;
-    // barrier slots (8 bytes each): full[3] empty[3] tfull[2] tempty[2] drain
+    // barrier slots (8 bytes each): full[4] empty[4] tfull[2] tempty[2] drain
     auto full = [&](int s) { return bars + 8u * s; };
-    auto empty = [&](int s) { return bars + 8u * (ST + s); };
-    auto tfull = [&](int b) { return bars + 8u * (2 * ST + b); };
-    auto tempty = [&](int b) { return bars + 8u * (2 * ST + 2 + b); };
-    const uint32_t drain = bars + 8u * (2 * ST + 4);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ctl + 128);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(ctl + 136);
+    auto empty = [&](int s) { return bars + 8u * (TC_MAX_STAGES + s); };
+    auto tfull = [&](int b) { return bars + 8u * (2 * TC_MAX_STAGES + b); };
+    auto tempty = [&](int b) { return bars + 8u * (2 * TC_MAX_STAGES + 2 + b); };
+    const uint32_t drain = bars + 8u * (2 * TC_MAX_STAGES + 4);
+    // a stage holds the rows that are fetched: A_re, A_im, B_re, B_im, each a multiple of 1024 bytes
+    const uint32_t a_bytes = FULL ? TC_TILE_BYTES : 128u * (uint32_t)p.rows_a, b_bytes = FULL ? TC_TILE_BYTES : 128u * (uint32_t)p.rows_b;
+    const uint32_t stage_bytes = 2u * (a_bytes + b_bytes);
+    const int stages = FULL ? ST : p.stages;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ctl + 400);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(ctl + 408);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (!p.late_trigger) dep_trigger();
     if (tid == 0) {
-        for (int s = 0; s < ST; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
+        for (int s = 0; s < stages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(tfull(b), 1); mbar_init(tempty(b), 128); }
         mbar_init(drain, 1);
         *abort_flag = 0;
@@ -254,48 +273,51 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (warp == 0) {
         if (lane == 0) {
             // ---- producer ------------------------------------------------------
-            int it = 0;
+            const int blocks_a = FULL ? 4 : p.rows_a >> 5, blocks_b = FULL ? 4 : p.rows_b >> 5;
+            int it = 0, s = 0;
+            uint32_t ph = 0;
             bool ok = true;
             for (int t = blockIdx.x; ok && t < num_tiles; t += gridDim.x) {
                 const int n_t = t % p.n_tiles;
                 const int m_t = (t / p.n_tiles) % p.m_tiles;
                 const int bin = global_bin(t / (p.n_tiles * p.m_tiles));
                 for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-                    const int s = it % ST;
-                    const uint32_t ph = (uint32_t)(it / ST) & 1u;
                     if (!mbar_wait(empty(s), ph ^ 1u, abort_flag, p.wait_cycles)) { ok = false; break; }
-                    const uint32_t dst = tiles + s * TC_STAGE_BYTES;
-                    mbar_expect_tx(full(s), TC_STAGE_BYTES);
+                    const uint32_t dst = tiles + s * stage_bytes;
+                    mbar_expect_tx(full(s), stage_bytes);
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
                         if constexpr (!TA) {
-                            tma_load_3d(dst + part * TC_TILE_BYTES, &tmA, kb * TC_BK, m_t * TC_BM,
+                            tma_load_3d(dst + part * a_bytes, &tmA, kb * TC_BK, m_t * TC_BM,
                                         part * p.bins + bin, full(s));
                         } else {
 #pragma unroll
                             for (int blk = 0; blk < 4; ++blk)
-                                tma_load_3d(dst + part * TC_TILE_BYTES + blk * 4096, &tmA,
+                                if (blk < blocks_a)
+                                    tma_load_3d(dst + part * a_bytes + blk * 4096, &tmA,
                                             m_t * TC_BM + blk * 32, kb * TC_BK, part * p.bins + bin, full(s));
                         }
                         if constexpr (!TB) {
-                            tma_load_3d(dst + (2 + part) * TC_TILE_BYTES, &tmB, kb * TC_BK, n_t * TC_BN,
+                            tma_load_3d(dst + 2 * a_bytes + part * b_bytes, &tmB, kb * TC_BK, n_t * TC_BN,
                                         part * p.bins + bin, full(s));
                         } else {
 #pragma unroll
                             for (int blk = 0; blk < 4; ++blk)
-                                tma_load_3d(dst + (2 + part) * TC_TILE_BYTES + blk * 4096, &tmB,
+                                if (blk < blocks_b)
+                                    tma_load_3d(dst + 2 * a_bytes + part * b_bytes + blk * 4096, &tmB,
                                             n_t * TC_BN + blk * 32, kb * TC_BK, part * p.bins + bin, full(s));
                         }
                     }
+                    if (++s == stages) { s = 0; ph ^= 1u; }
                 }
             }
             if (!ok) {
                 give_up();
                 // let the copies already issued land before the CTA's memory goes away
-                const int back = it < ST ? it : ST;
+                const int back = it < stages ? it : stages;
                 for (int j = it - back; j < it; ++j) {
                     const long long t0 = clock64();
-                    while (!mbar_try_wait(full(j % ST), (uint32_t)(j / ST) & 1u) &&
+                    while (!mbar_try_wait(full(j % stages), (uint32_t)(j / stages) & 1u) &&
                            clock64() - t0 < TC_WAIT_CYCLES) {}
                 }
             }
@@ -303,13 +325,14 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     } else if (warp == 1) {
         if (lane == 0) {
             // ---- MMA issuer ----------------------------------------------------
-            constexpr uint32_t idesc_pos = tc_idesc(TC_BM, TC_BN, false, TA, TB);
-            constexpr uint32_t idesc_neg = tc_idesc(TC_BM, TC_BN, true, TA, TB);
+            const uint32_t idesc_pos = tc_idesc(TC_BM, FULL ? TC_BN : p.mma_n, false, TA, TB);
+            const uint32_t idesc_neg = tc_idesc(TC_BM, FULL ? TC_BN : p.mma_n, true, TA, TB);
             // (Ar + i sA Ai)(Br + i sB Bi): re = ArBr - sA sB AiBi ; im = sB ArBi + sA AiBr
             const uint32_t id_ii = (p.conjA != p.conjB) ? idesc_pos : idesc_neg;
             const uint32_t id_ri = p.conjB ? idesc_neg : idesc_pos;
             const uint32_t id_ir = p.conjA ? idesc_neg : idesc_pos;
-            int it = 0, tl = 0;
+            int tl = 0, s = 0;
+            uint32_t ph = 0;
             bool ok = true;
             for (int t = blockIdx.x; ok && t < num_tiles; t += gridDim.x, ++tl) {
                 const int buf = tl & 1;
@@ -317,23 +340,22 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 tc_fence_after_sync();
                 const uint32_t d_re = tmem_base + (uint32_t)buf * 256u;
                 const uint32_t d_im = d_re + 128u;
-                for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-                    const int s = it % ST;
-                    if (!mbar_wait(full(s), (uint32_t)(it / ST) & 1u, abort_flag, p.wait_cycles)) { ok = false; break; }
+                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    if (!mbar_wait(full(s), ph, abort_flag, p.wait_cycles)) { ok = false; break; }
                     tc_fence_after_sync();
-                    const uint32_t src = tiles + s * TC_STAGE_BYTES;
+                    const uint32_t src = tiles + s * stage_bytes;
                     const uint64_t a_re = TA ? tc_smem_desc_mn(src) : tc_smem_desc(src);
-                    const uint64_t a_im = TA ? tc_smem_desc_mn(src + TC_TILE_BYTES)
-                                             : tc_smem_desc(src + TC_TILE_BYTES);
-                    const uint64_t b_re = TB ? tc_smem_desc_mn(src + 2 * TC_TILE_BYTES)
-                                             : tc_smem_desc(src + 2 * TC_TILE_BYTES);
-                    const uint64_t b_im = TB ? tc_smem_desc_mn(src + 3 * TC_TILE_BYTES)
-                                             : tc_smem_desc(src + 3 * TC_TILE_BYTES);
+                    const uint64_t a_im = TA ? tc_smem_desc_mn(src + a_bytes) : tc_smem_desc(src + a_bytes);
+                    const uint32_t src_b = src + 2 * a_bytes;
+                    const uint64_t b_re = TB ? tc_smem_desc_mn(src_b) : tc_smem_desc(src_b);
+                    const uint64_t b_im = TB ? tc_smem_desc_mn(src_b + b_bytes) : tc_smem_desc(src_b + b_bytes);
                     // per k-step of 8: K-major advances 32 bytes inside the swizzled row,
                     // MN-major advances eight 128-byte k-rows (address field is in 16 B units)
                     constexpr uint64_t stepA = TA ? 64 : 2, stepB = TB ? 64 : 2;
+                    const int steps = FULL ? TC_BK / 8 : (p.K - kb * TC_BK + 7) >> 3;      // k-steps past the summed length would only add zeros
 #pragma unroll
                     for (int k = 0; k < TC_BK / 8; ++k) {
+                        if (k >= steps) break;
                         const uint64_t da = stepA * k, db = stepB * k;
                         const uint32_t acc = (kb | k) != 0 ? 1u : 0u;
                         tc_mma_tf32(d_re, a_re + da, b_re + db, idesc_pos, acc);
@@ -342,6 +364,7 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         tc_mma_tf32(d_im, a_im + da, b_re + db, id_ir, 1u);
                     }
                     tc_commit(empty(s));          // stage reusable once these MMAs have read it
+                    if (++s == stages) { s = 0; ph ^= 1u; }
                 }
                 if (ok) tc_commit(tfull(buf));    // accumulators complete
             }
@@ -418,9 +441,9 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 }
 
 // ---- host side -------------------------------------------------------------
-template <bool TA, bool TB, int ST>
-static cudaError_t launch_cgemm_tc_t(const GemmParams& g, int* status, cudaStream_t st, int sm_count) {
-    auto kern = cgemm_tc_kernel<TA, TB, ST>;
+template <bool TA, bool TB, int ST, bool FULL>
+static cudaError_t launch_cgemm_tc_f(const GemmParams& g, int* status, cudaStream_t st, int sm_count) {
+    auto kern = cgemm_tc_kernel<TA, TB, ST, FULL>;
     static std::atomic<unsigned long long> attr_set_devices{0};     // one bit per device ordinal
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
@@ -433,15 +456,22 @@ static cudaError_t launch_cgemm_tc_t(const GemmParams& g, int* status, cudaStrea
     CUtensorMap tmA, tmB, tmC;
     // k-contiguous: rows = M (or N), cols = K, box 32 k x 128 rows;
     // row-contiguous: rows = K, cols = M (or N), box 32 rows-of-the-matrix x 32 k.
+    auto cover = [](int rows, int unit, int tile) { const int r = (rows + unit - 1) / unit * unit; return r < tile ? r : tile; };
+    TcParams p{};
+    // (FULL: M > 120 and N > 112, so that all of these come out as a whole tile)
+    p.rows_a = cover(g.M, TA ? 32 : 8, TC_BM);
+    p.rows_b = cover(g.N, TB ? 32 : 16, TC_BN);
+    p.mma_n = cover(g.N, 16, TC_BN);
+    const int fit = (int)(ST * TC_STAGE_BYTES / (256u * (uint32_t)(p.rows_a + p.rows_b)));
+    p.stages = fit < TC_MAX_STAGES ? fit : TC_MAX_STAGES;
     const bool okA = TA ? tc_make_map(&tmA, g.A, g.bins, g.K, g.M, g.lda, 32, TC_BK,
                                       CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)
-                        : tc_make_map(&tmA, g.A, g.bins, g.M, g.K, g.lda, TC_BK, TC_BM);
+                        : tc_make_map(&tmA, g.A, g.bins, g.M, g.K, g.lda, TC_BK, p.rows_a);
     const bool okB = TB ? tc_make_map(&tmB, g.B, g.bins, g.K, g.N, g.ldb, 32, TC_BK,
                                       CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)
-                        : tc_make_map(&tmB, g.B, g.bins, g.N, g.K, g.ldb, TC_BK, TC_BN);
+                        : tc_make_map(&tmB, g.B, g.bins, g.N, g.K, g.ldb, TC_BK, p.rows_b);
     const bool okC = tc_make_map(&tmC, g.C, g.bins, g.M, g.N, g.ldc, 32, 32);
     if (!okA || !okB || !okC) return cudaErrorInvalidValue;
-    TcParams p{};
     p.bins = g.bins; p.M = g.M; p.N = g.N; p.K = g.K;
     p.m_tiles = (g.M + TC_BM - 1) / TC_BM;
     p.n_tiles = (g.N + TC_BN - 1) / TC_BN;
@@ -468,6 +498,11 @@ static cudaError_t launch_cgemm_tc_t(const GemmParams& g, int* status, cudaStrea
     return dep_launch(g.overlap != 0, kern, dim3(grid), dim3(TC_THREADS), tc_smem_bytes(ST), st, tmA, tmB, tmC, p);
 }
 
+template <bool TA, bool TB, int ST>
+static cudaError_t launch_cgemm_tc_t(const GemmParams& g, int* status, cudaStream_t st, int sm_count) {
+    return g.M > TC_BM - 8 && g.N > TC_BN - 16 ? launch_cgemm_tc_f<TA, TB, ST, true>(g, status, st, sm_count)
+                                               : launch_cgemm_tc_f<TA, TB, ST, false>(g, status, st, sm_count);
+}
 static cudaError_t launch_cgemm_tc(const GemmParams& g, int* status, cudaStream_t st) {
     const int sm_count = fft_sm_count();        // of the current device
     if (sm_count < 1) return cudaErrorInvalidDevice;

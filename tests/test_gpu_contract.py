@@ -97,3 +97,12 @@ def test_contraction_layouts_and_conjugates(shape, math, flags):
                                    (5, 2, 3, 203), (3000, 2, 5, 3)])
 def test_contraction_of_small_matrices(shape, math, flags):
     assert run(*shape, math=math, seed=11, **flags) <= TOL[math]
+
+
+# tensor-core tiles used in part: rows of the boxes (8, 16, 32 at a time), N of the instructions (16), k-steps
+# (8) and stages of the ring, and the line at which a tile counts as full (M > 120 and N > 112)
+@pytest.mark.parametrize("flags", FLAGS[:3])
+@pytest.mark.parametrize("shape", [(200, 121, 113, 33), (200, 120, 113, 64), (200, 121, 112, 40), (200, 33, 97, 65),
+                                   (200, 65, 33, 96), (200, 40, 200, 8), (200, 136, 48, 72)])
+def test_tf32_tiles_used_in_part(shape, flags):
+    assert run(*shape, math=2, seed=13, **flags) <= TOL[2]
