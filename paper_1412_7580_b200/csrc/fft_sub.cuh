@@ -97,26 +97,29 @@ r2c_sub_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__
     };
     // Copy of the real planes of an item.  Sets `pending` if (part of) it is asynchronous (wait on
     // the barrier) and `plain` if threads stored (part of) it themselves (barrier before reading).
+    // The item keeps its misalignment in shared memory (`off` samples), as in r2c_kernel.
     bool pending = false, plain = false;
+    int off = 0;
     auto stage = [&](const Item& it) {
         const FftParams& p = it.second ? p1 : p0;
         const int hw = p.h * p.w;
         const float* src = p.real_in + ((size_t)it.row * p.C + it.c0) * hw;
         const int total = it.gcount * hw;
-        if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-            const int bulk = total & ~3;
-            if (is_loader && bulk > 0) {
-                fk_mbar_expect_tx(bar, (uint32_t)bulk * 4u);
-                fk_bulk_g2s(fk_smem_u32(sIn), src, (uint32_t)bulk * 4u, bar);
-            }
-            if (tid < total - bulk) sIn[bulk + tid] = __ldg(src + bulk + tid);
-            pending = bulk > 0;
-            plain = total != bulk;
-            return;
+        const int mis = (int)(reinterpret_cast<uintptr_t>(src) >> 2) & 3;
+        const int head = min((4 - mis) & 3, total);
+        const int bulk = (total - head) & ~3;
+        float* dst = sIn + mis;
+        if (is_loader && bulk > 0) {
+            fk_mbar_expect_tx(bar, (uint32_t)bulk * 4u);
+            fk_bulk_g2s(fk_smem_u32(dst + head), src + head, (uint32_t)bulk * 4u, bar);
         }
-        for (int i = tid; i < total; i += T) sIn[i] = __ldg(src + i);
-        pending = false;
-        plain = true;
+        if (tid < total - bulk) {
+            const int i = tid < head ? tid : bulk + tid;
+            dst[i] = __ldg(src + i);
+        }
+        off = mis;
+        pending = bulk > 0;
+        plain = total != bulk;
     };
 
     uint32_t phase = 0;
@@ -148,7 +151,7 @@ r2c_sub_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__
             const bool act = (gA < gcount) && (cA < w);
             if (act) {
                 float v[N];
-                const float* src = sIn + gA * hw + cA;
+                const float* src = sIn + off + gA * hw + cA;
                 if (h > M) {
                     static_for<N>([&](auto Rr) {
                         constexpr int r = decltype(Rr)::value;
@@ -271,11 +274,11 @@ static cudaError_t launch_r2c_sub(FftParams pa, const FftParams* pb_in, cudaStre
         if (pb_in && (pb_in->win || 2 * pb_in->w <= N)) return cudaErrorNotSupported;
         FftParams pb{};
         if (!fill_tiling<GS>(pa)) return cudaErrorInvalidValue;
-        int in_bytes = real_tile_bytes(G, pa.h, pa.w);
+        int in_bytes = real_tile_bytes(G, pa.real_in, pa.h, pa.w);
         if (pb_in) {
             pb = *pb_in;
             if (!fill_tiling<GS>(pb)) return cudaErrorInvalidValue;
-            const int b = real_tile_bytes(G, pb.h, pb.w);
+            const int b = real_tile_bytes(G, pb.real_in, pb.h, pb.w);
             if (b > in_bytes) in_bytes = b;
         }
         if ((size_t)in_bytes < SubGeom<N, G, SUB>::MID_BYTES) in_bytes = (int)SubGeom<N, G, SUB>::MID_BYTES;

@@ -264,3 +264,19 @@ def test_large_planes_at_the_edges_of_their_tiles(dims):
     assert relerr(y, oracle.fprop(x, w)) <= TOL[eff[0]]
     assert relerr(dx, oracle.bprop(dy, w, s.h, s.w)) <= TOL[eff[1]]
     assert relerr(dw, oracle.accgrad(dy, x, s.kh, s.kw)) <= TOL[eff[2]]
+
+
+@pytest.mark.parametrize("dims", [
+    # S, f, fp, h, w, kh, kw, n: odd planes in odd numbers, so that the tiles of a matrix row start at any
+    # multiple of 4 bytes; at n = 64 more tiles than the GPU has CTAs for
+    (9, 33, 3, 31, 31, 5, 5, 32), (5, 51, 7, 7, 7, 3, 3, 8), (13, 97, 1, 57, 57, 3, 3, 64),
+])
+def test_odd_planes_in_odd_numbers(dims):
+    import oracle
+    from paper_1412_7580_b200 import workloads as wl
+    s = wl.ConvShape("odd", *dims, cfg=7, point=sum(dims))
+    x, w, dy = wl.make_x(s), wl.make_w(s), wl.make_dy(s)
+    y, dx, dw, eff = run_gpu(s, x, w, dy, 1)
+    assert relerr(y, oracle.fprop(x, w)) <= TOL[eff[0]]
+    assert relerr(dx, oracle.bprop(dy, w, s.h, s.w)) <= TOL[eff[1]]
+    assert relerr(dw, oracle.accgrad(dy, x, s.kh, s.kw)) <= TOL[eff[2]]

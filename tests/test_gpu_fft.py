@@ -146,3 +146,24 @@ def test_bare_transforms_with_a_spectrum_that_is_only_8_byte_aligned(n, batch, h
     torch.cuda.synchronize()
     assert torch.equal(back_a, back_u)
     assert relerr(back_a.cpu().numpy().astype(np.float64), x.astype(np.float64)) <= TOL_FFT
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("n,batch,h,w", [(8, 20011, 3, 5), (16, 10007, 13, 13), (32, 4001, 9, 31), (64, 1803, 57, 35),
+                                         (64, 1, 1, 1), (128, 303, 65, 67)])
+def test_planes_that_start_at_any_multiple_of_4_bytes(n, batch, h, w, shift):
+    """Odd planes in odd numbers, more of them than the CTAs take in one go: the tiles of a launch
+    start at every multiple of 4 bytes, wherever the first plane starts."""
+    import torch
+    import paper_1412_7580_b200 as fc
+    from paper_1412_7580_b200 import workloads as wl
+    x = wl.make_planes(batch, h, w, seed=n + shift)
+    buf = torch.full((batch * h * w + 4,), float("nan"), device="cuda")
+    xd = buf[shift:shift + batch * h * w].view(batch, h, w)
+    xd.copy_(torch.from_numpy(x))
+    assert xd.data_ptr() % 16 == 4 * shift
+    out = torch.full((batch, n, n // 2 + 1, 2), float("nan"), device="cuda")
+    fc.fft2d_r2c(xd, out, n)
+    ref = np.fft.rfft2(x.astype(np.float64), s=(n, n))
+    o = out.cpu().numpy()
+    assert relerr(o[..., 0], ref.real) <= TOL_FFT and relerr(o[..., 1], ref.imag) <= TOL_FFT
