@@ -570,7 +570,7 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
         __syncthreads();
 
         // 3. row transforms: thread = (half q, row kyp, plane gB)
-        if (TMA || gB < gcount) {
+        if (TMA || (BSTG && SALIAS) || gB < gcount) {
             float ar[M], ai[M];
             const float2* rowp = sMid + gB * P + kyp * PW;
             const bool packed = (kyp == 0);
@@ -584,7 +584,7 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
                 if (q == 0) load_split<N, false, 0>(load, ar, ai);
                 else        load_split<N, false, 1>(load, ar, ai);
             }
-            if constexpr (TMA && SALIAS) __syncthreads();   // scratch consumed: it becomes the staging tile
+            if constexpr ((TMA || BSTG) && SALIAS) __syncthreads();   // scratch consumed: it becomes the staging tile
             cfft<M, false>(ar, ai);                     // ar/ai[k] = F[kx = 2k+q]
 
             if constexpr (!BARE) {
@@ -1036,6 +1036,23 @@ template <> struct FftCfg<32>  { static constexpr int G = 8;  static constexpr b
 template <> struct FftCfg<64>  { static constexpr int G = 4;  static constexpr bool ALIAS = false, SALIAS = false; static constexpr int MINB = 1, MINB_INV = 1; static constexpr bool TMA = true; };
 template <> struct FftCfg<128> { static constexpr int G = 2;  static constexpr bool ALIAS = true,  SALIAS = false; static constexpr int MINB = 1, MINB_INV = 1; static constexpr bool TMA = false; };
 
+// Bare layout staged through shared memory.  Its copies are whole planes, so a tile needs no width to move
+// long rows, and half as many planes per CTA put more planes in flight on an SM: fewer threads wait at each
+// barrier, and 4 to 8 CTAs are at different stages (three at n = 64, where the forward transform's staging
+// image has to lie over the scratch for them to fit; at n = 8 it saves the shared memory of two more CTAs).
+// B200, forward / inverse, one tile as in FftCfg -> these (us):
+//   n = 8,   400000 planes of 7 x 7     62.6 / 58.4 -> 52.0 / 48.2    (staging image apart: 55.6 / 50.4)
+//   n = 16,  131072 planes of 13 x 13   61.6 / 60.0 -> 51.1 / 50.1    (a quarter of the planes: 53 / 52)
+//   n = 32,  32768 planes of 31 x 31    57.4 / 58.6 -> 52.7 / 51.5    (a quarter: 56.5 / 52.0; shared image 62.8)
+//   n = 64,  8192 planes of 57 x 57     66.0 / 66.0 -> 57.1 / 61.2    (a quarter: 56.2 / 62.7; image apart 65)
+template <int N> struct BareCfg;
+template <> struct BareCfg<8>  : FftCfg<8>  { static constexpr int G = 16; static constexpr bool SALIAS = true;  static constexpr int MINB = 8, MINB_INV = 8; };
+template <> struct BareCfg<16> : FftCfg<16> { static constexpr int G = 8;  static constexpr bool SALIAS = false; static constexpr int MINB = 7, MINB_INV = 7; };
+template <> struct BareCfg<32> : FftCfg<32> { static constexpr int G = 4;  static constexpr bool SALIAS = false; static constexpr int MINB = 4, MINB_INV = 4; };
+template <> struct BareCfg<64> : FftCfg<64> { static constexpr int G = 2;  static constexpr bool SALIAS = true;  static constexpr int MINB = 3, MINB_INV = 3; };
+template <int N, int LAYOUT> struct LayoutCfg { using type = FftCfg<N>; };
+template <int N> struct LayoutCfg<N, LAYOUT_BARE_STAGED> { using type = BareCfg<N>; };
+
 // SM count of the current device (0 on failure); looked up once per device ordinal.
 static inline int fft_sm_count() {
     static std::atomic<int> sms[64];
@@ -1112,7 +1129,7 @@ static bool fill_tiling(FftParams& p) {
 // Forward transform of one operand, or of two operands in one launch (pb may be null).
 template <int N, int LAYOUT>
 static cudaError_t launch_r2c_layout(FftParams pa, const FftParams* pb_in, cudaStream_t st) {
-    using Cfg = FftCfg<N>;
+    using Cfg = typename LayoutCfg<N, LAYOUT>::type;
     constexpr int G = Cfg::G;
     FftParams pb{};
     if (!fill_tiling<G>(pa)) return cudaErrorInvalidValue;
@@ -1129,7 +1146,7 @@ static cudaError_t launch_r2c_layout(FftParams pa, const FftParams* pb_in, cudaS
     CUtensorMap tma, tmb;
     memset(&tma, 0, sizeof(tma));
     memset(&tmb, 0, sizeof(tmb));
-    constexpr bool SALIAS = Cfg::SALIAS && LAYOUT == LAYOUT_FREQ_TMA;
+    constexpr bool SALIAS = Cfg::SALIAS && (LAYOUT == LAYOUT_FREQ_TMA || LAYOUT == LAYOUT_BARE_STAGED);
     if (LAYOUT == LAYOUT_FREQ_TMA) {
         const size_t stage = (size_t)2 * N * (N / 2 + 1) * G * sizeof(float);
         if (SALIAS) smem = (size_t)in_bytes + (stage > mid ? stage : mid);
@@ -1137,7 +1154,11 @@ static cudaError_t launch_r2c_layout(FftParams pa, const FftParams* pb_in, cudaS
         if (!make_spec_map<N, G>(&tma, pa.spec_out, pa)) return cudaErrorInvalidValue;
         if (pb_in && !make_spec_map<N, G>(&tmb, pb.spec_out, pb)) return cudaErrorInvalidValue;
     }
-    if (LAYOUT == LAYOUT_BARE_STAGED) smem += BareGeom<N, G>::BYTES;
+    if (LAYOUT == LAYOUT_BARE_STAGED) {
+        const size_t image = BareGeom<N, G>::BYTES;
+        if (SALIAS) smem = (size_t)in_bytes + (image > mid ? image : mid);
+        else smem += image;
+    }
     // the windowed variant (spatial tiling) is a separate instantiation, so that the plain
     // kernels carry none of its code
     const bool win = pa.win || (pb_in && pb.win);
@@ -1174,7 +1195,7 @@ template <int N> struct C2rDoubleBuffer { static constexpr bool value = (N == 64
 
 template <int N, int LAYOUT>
 static cudaError_t launch_c2r_layout(FftParams p, cudaStream_t st) {
-    using Cfg = FftCfg<N>;
+    using Cfg = typename LayoutCfg<N, LAYOUT>::type;
     constexpr int G = Cfg::G;
     constexpr bool DB = C2rDoubleBuffer<N>::value && LAYOUT == LAYOUT_FREQ_TMA;
     if (!fill_tiling<G>(p)) return cudaErrorInvalidValue;
