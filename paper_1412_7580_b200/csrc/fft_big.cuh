@@ -2,9 +2,11 @@
 // that give the frequency-major rows 32 bytes, is 528 KB and does not fit shared memory), and the
 // pieces it shares with the forward transform of fft_split.cuh.
 //
-// A tile of 8 planes is transformed by a cluster of CL = 2, 4 or 8 CTAs.  The half spectrum between
+// A tile of 8 planes is transformed by a cluster of CL = 1, 2, 4 or 8 CTAs.  The half spectrum between
 // the two 1-D passes goes through a scratch area in global memory, 512 KB per tile in flight, which
-// is rewritten for every tile and therefore mostly stays in the L2.
+// is rewritten for every tile; the spectra, read once, and the result pass through the L2 as first to
+// leave, so that the scratch stays (12,288 planes of 118 x 118: 717 -> 668 us, 4,096 of 128 x 128:
+// 243 -> 227; a third of the scratch was written back to memory without).
 //   B. rows: chunks of 8 rows ky (x 8 planes = 64 rows of 128 kx) arrive through a ring of three TMA
 //      buffers; the two teams of 256 threads take them alternately.  Four threads per row run the
 //      inverse complex FFT (one radix-4 decimation-in-frequency step on the loads, 32-point register
@@ -15,7 +17,8 @@
 //      butterfly stage exchanges by shuffles, and the cropped, scaled rows go straight to the result.
 //      No shared memory and no barrier, so the next tile's chunks are loaded meanwhile.
 // The CTAs of a cluster share the chunks and the planes of a tile (see big_cluster).
-// Bound by instruction issue (46 % of the slots) and the latencies of the two phases, 2.2 TB/s.
+// Bound by the latencies of the two phases, of which the second one's reads of the scratch are the
+// longest (a third of the time), and by instruction issue (half of the slots): 2.3 TB/s.
 #pragma once
 
 #include "fft_kernels.cuh"
@@ -76,6 +79,17 @@ __device__ __forceinline__ void fk_tma_load_4d(uint32_t dst, const CUtensorMap* 
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
 }
+// The same for data that a kernel reads once: its lines are the first to leave the L2.
+__device__ __forceinline__ void fk_tma_load_4d_once(uint32_t dst, const CUtensorMap* map, int c0, int c1,
+                                                    int c2, int c3, uint32_t bar) {
+    unsigned long long once;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(once));
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(once)
+        : "memory");
+}
 template <int TEAM>
 __device__ __forceinline__ void big_team_sync(int team) {
     asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(TEAM) : "memory");
@@ -124,8 +138,8 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
         const int row = tile / tpr, c0 = (tile - row * tpr) * G;
         const uint32_t bar = fk_smem_u32(&bar_storage[s]);
         fk_mbar_expect_tx(bar, (uint32_t)(Gm::STAGE + (ci == 0 ? Gm::STAGE_NY : 0)));
-        fk_tma_load_4d(fk_smem_u32(fc_smem + s * Gm::BUF), &tmS, c0, row, ci * KC, 0, bar);
-        if (ci == 0) fk_tma_load_4d(fk_smem_u32(fc_smem + RING * Gm::BUF + s * Gm::STAGE_NY), &tmNy, c0, row, M, 0, bar);
+        fk_tma_load_4d_once(fk_smem_u32(fc_smem + s * Gm::BUF), &tmS, c0, row, ci * KC, 0, bar);
+        if (ci == 0) fk_tma_load_4d_once(fk_smem_u32(fc_smem + RING * Gm::BUF + s * Gm::STAGE_NY), &tmNy, c0, row, M, 0, bar);
         issued[s] = seq;
     };
     // Wait for chunk `seq`.  The buffer's previous chunk belongs to the other team: until that team has
@@ -236,11 +250,11 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
                 float* o = out + (2 * j) * wc;
                 if (2 * j < rows) {
                     if (acc) zr += *o;
-                    *o = zr;
+                    __stcs(o, zr);
                 }
                 if (2 * j + 1 < rows) {
                     if (acc) zi += o[wc];
-                    o[wc] = zi;
+                    __stcs(o + wc, zi);
                 }
             });
         }
@@ -248,11 +262,15 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
     }
 }
 
-// CTAs that share a tile: two when there is a tile for every pair of SMs (4,096 planes of 128 x 128: 241 us,
-// 252 with one and 471 with four, whose clusters leave SMs empty), more where SMs would be idle (14 tiles
-// of 97 x 101 planes: 57 us with one CTA per tile, 34 with two, 23 with four or eight).
+// CTAs that share a tile.  One when every tile gets an SM of its own and pairs would take a second, partly
+// empty round (128 tiles of 128 x 128 planes: 52 us, 59 with two); two when there are more (512 tiles: 241 us,
+// 252 with one and 471 with four, whose clusters leave SMs empty) or tiles for at most half of the SMs; more
+// where SMs would still be idle (14 tiles of 97 x 101 planes: 57 us with one CTA per tile, 34 with two, 23
+// with four or eight).
 static inline int big_cluster(long long tiles, int slots) {
-    return 8 * tiles <= slots ? 8 : 4 * tiles <= slots ? 4 : 2;
+    if (8 * tiles <= slots) return 8;
+    if (4 * tiles <= slots) return 4;
+    return 2 * tiles > slots && tiles <= slots ? 1 : 2;
 }
 
 static cudaError_t launch_c2r_big(FftParams p, float* scratch, size_t scratch_bytes, cudaStream_t st) {
