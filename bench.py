@@ -428,7 +428,7 @@ class Bench:
         blocks = self.timed(step, args.steps)
         t1 = time.time()
         # counted by the library.  Per pass: the forward FFTs (one launch for both operands with the
-        # one-pass kernels, one per operand with the two-pass kernels), the contraction, the inverse FFT
+        # one-pass kernels, the filters apart where they have a kernel of their own), the contraction, the inverse FFT
         counted = fc.fftconv_launch_count() - launches0
         total_steps = args.steps * len(blocks)
         assert counted % total_steps == 0, (counted, total_steps)

@@ -49,8 +49,8 @@ typedef enum {
 } fftconv_status;
 
 typedef enum {
-    FFTCONV_MATH_AUTO = 0, /* tensor cores unless a bin's result has fewer than 128 elements,
-                              where the FP32 kernel is as fast and exact                  */
+    FFTCONV_MATH_AUTO = 0, /* tensor cores unless a bin's result has fewer than 128 elements or
+                              the matrices are small enough that the FP32 kernel is as fast */
     FFTCONV_MATH_FP32 = 1, /* per-bin contraction with FP32 FFMA                  */
     FFTCONV_MATH_TF32 = 2  /* per-bin contraction on tcgen05 tensor cores, TF32
                               inputs, FP32 accumulation in tensor memory         */
@@ -81,8 +81,8 @@ int conv_plan_pass_math(const conv_plan_t* plan, int pass);
 /* Bytes of device scratch the three passes need: the frequency-domain copies of
  * the two operands and of the result (Section 6 lists the same buffers), in the
  * plan's private frequency-major layout; plans with n = 128 add the scratch
- * that the transforms of large planes pass their half spectra through between
- * the two 1-D passes (80 MiB = 83.9e6 bytes: 512 KiB for each of up to 160
+ * that the inverse transform of large planes passes its half spectra through
+ * between the two 1-D passes (80 MiB = 83.9e6 bytes: 512 KiB for each of up to 160
  * resident CTAs).  0 on a null plan. */
 size_t conv_plan_workspace_bytes(const conv_plan_t* plan);
 

@@ -186,7 +186,7 @@ size_t pass_bytes(const conv_plan_s& p, int pass) {
            align_up(d.c.spec.bytes(p.bins), kAlign);
 }
 
-// Bytes of the spectra regions (with the header); the scratch of the two-pass transforms
+// Bytes of the spectra regions (with the header); the scratch of the n = 128 inverse transform
 // (n = 128) follows them.
 size_t spectra_bytes(const conv_plan_s* plan) {
     if (plan->reuse) {
