@@ -12,7 +12,7 @@
 //
 // cfft and rfft are templates over the value type V: float, or F2 (f32x2.cuh), which carries the same
 // element of two independent transforms through packed instructions -- twice the transforms for the
-// same number of issued instructions, bit for bit the same results (forward transform of n = 128).
+// same number of issued instructions, bit for bit the same results (transforms of n = 128).
 #pragma once
 
 #include <utility>

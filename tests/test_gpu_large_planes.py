@@ -1,0 +1,48 @@
+"""Transforms of planes that need the basis 128: the kernels choose their loads by the parity of the row length
+and by the alignment of the tensor, split the rows over work items and clip ragged tiles of 8 planes."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+# (S, f, f', h, w, kh, kw), samples by which the tensors are shifted in memory
+@pytest.mark.parametrize("dims,shift", [
+    ((2, 9, 3, 128, 128, 5, 5), 0),        # pairs of columns; every row and column in use
+    ((2, 9, 3, 128, 128, 5, 5), 1),        # the same from an address that is no multiple of 8 bytes
+    ((1, 8, 10, 66, 127, 3, 4), 0),        # odd rows, the last column has no partner; dy's rows are even
+    ((3, 1, 17, 127, 66, 2, 3), 0),        # one plane in a tile, tiles of 8 + 8 + 1
+    ((1, 7, 8, 40, 101, 9, 3), 2),         # fewer rows than half the basis
+    ((2, 3, 5, 97, 20, 97, 2), 0),         # narrow planes, kernel as high as the plane
+])
+def test_passes_against_oracle(dims, shift):
+    import torch
+    import oracle
+    import paper_1412_7580_b200 as fc
+    from paper_1412_7580_b200 import workloads as wl
+    s = wl.ConvShape("large_planes", *dims, 128, cfg=9, point=sum(dims) + shift)
+    host = wl.make_x(s), wl.make_w(s), wl.make_dy(s)
+
+    def shifted(a):
+        flat = torch.empty(a.size + shift, device="cuda")
+        flat[shift:] = torch.from_numpy(a.ravel()).cuda()
+        return flat[shift:].view(a.shape)
+
+    x, w, dy = host
+    xd, wd, dyd = (shifted(a) for a in host)
+    p = fc.conv_plan(*s.args())
+    fc.conv_plan_set_math(p, fc.binding.MATH_FP32)
+    fc.conv_plan_alloc_workspace(p)
+    y, dx, dw = (shifted(np.full(shape, np.nan, np.float32)) for shape in
+                 ((s.S, s.fp, s.oh, s.ow), x.shape, w.shape))
+    fc.conv_fprop(p, xd, wd, y)
+    fc.conv_bprop(p, dyd, wd, dx)
+    fc.conv_accgrad(p, dyd, xd, dw)
+    torch.cuda.synchronize()
+    assert fc.conv_plan_status(p) == 0
+    # FP32 end to end: 2 x 14 butterfly stages and sums of at most 17 terms round at 2^-24 each; 1e-5 of the
+    # largest result is several times their worst case
+    for got, ref in ((y, oracle.fprop(x, w)), (dx, oracle.bprop(dy, w, s.h, s.w)), (dw, oracle.accgrad(dy, x, s.kh, s.kw))):
+        g = got.cpu().numpy().astype(np.float64)
+        assert np.max(np.abs(g - ref)) <= 1e-5 * np.max(np.abs(ref))
+    fc.conv_plan_destroy(p)
