@@ -2,23 +2,32 @@
 // that give the frequency-major rows 32 bytes, is 528 KB and does not fit shared memory), and the
 // pieces it shares with the forward transform of fft_split.cuh.
 //
-// A tile of 8 planes is transformed by a cluster of CL = 1, 2, 4 or 8 CTAs.  The half spectrum between
-// the two 1-D passes goes through a scratch area in global memory, 512 KB per tile in flight, which
-// is rewritten for every tile; the spectra, read once, and the result pass through the L2 as first to
-// leave, so that the scratch stays (12,288 planes of 118 x 118: 717 -> 668 us, 4,096 of 128 x 128:
-// 243 -> 227; a third of the scratch was written back to memory without).
-//   B. rows: chunks of 8 rows ky (x 8 planes = 64 rows of 128 kx) arrive through a ring of three TMA
-//      buffers; the two teams of 256 threads take them alternately.  Four threads per row run the
-//      inverse complex FFT (one radix-4 decimation-in-frequency step on the loads, 32-point register
-//      FFT); the rows are assembled in the chunk's buffer and copied to the scratch in 16-byte pieces.
-//      Rows ky = 0 and n/2 travel as one complex row (Section 5.2's border case).
-//   A. columns: a warp takes 16 columns of a plane, two adjacent lanes per column.  Each lane reads the
-//      bins of one parity straight from the scratch (irfft_half, decimation in time), the last
-//      butterfly stage exchanges by shuffles, and the cropped, scaled rows go straight to the result.
-//      No shared memory and no barrier, so the next tile's chunks are loaded meanwhile.
-// The CTAs of a cluster share the chunks and the planes of a tile (see big_cluster).
-// Bound by the latencies of the two phases, of which the second one's reads of the scratch are the
-// longest (a third of the time), and by instruction issue (half of the slots): 2.3 TB/s.
+// The mirror image of the forward transform: a work item is a tile of 8 planes and one eighth of the rows ky,
+// those congruent to +-r modulo 16 for class r = 0 .. 7.  The bins of a class add to the samples x[j + 8v]
+// (j < 8, v < 16) of a column twice the real part of w_16^{-rv} t_r[j], where t_r is ONE 8-point transform over
+// the class's rows, times w_128^{-rj}; class 0 (ky = 0 mod 8) leaves the terms r = 0 and 8 of the same sum.  So
+// each class leaves 8 complex values per column, and the last step of a tile is one 16-point real transform per
+// (column, j): no 1-D transform spans two items.  The values pass through a scratch area in global memory,
+// 512 KB per tile in flight, rewritten for every tile; the spectra, read once, and the result pass through the
+// L2 as first to leave, so that the scratch stays there.
+// A tile belongs to a cluster of CL = 1, 2, 4 or 8 CTAs, which share its classes and then its planes (big_cluster).
+//
+// Per item, 512 threads, packed fp32 pairs (f32x2.cuh) of two adjacent columns:
+//   B. the two residues of a class arrive as TMA boxes of 8 planes x 4 rows, in a ring of six; a team of 8 warps per
+//      box, eight threads per row: the first butterfly of a decimation in frequency yields the even and the odd
+//      columns, the two halves of a packed value; 8 points, a twiddle, an exchange in shared memory, 8 points,
+//      written back in place;
+//   A. thread = (plane, pair of columns): 8 rows, 8-point FFT, twiddle, coalesced 16-byte stores to the scratch.
+//   C. after the last item, thread = (pair of columns, j): 16-point transform, scale, cropped rows to the result.
+// Row ky = 0 carries ky = n/2 as (re, im) (Section 5.2).  Only the columns and rows inside the crop are computed from
+// A on, so that a filter gradient costs little more than the spectrum's loads.
+//
+// Bound by the chain of an item: at 6,500 - 8,500 cycles per 64 KB it is 1.5 - 2 times what its loads take (4,400); the
+// shared-memory pipe is busy for 2,600 of them.  Against whole rows and whole columns, with the half spectrum of a
+// tile in the scratch and two lanes of a warp per column: 4,096 planes of 128 x 128 226 -> 183 us, 12,288 of 118 x 118
+// 663 -> 545, 91 of 97 x 101 20.6 -> 15.4; 4,096 filter gradients of 5 x 5 176 -> 128.  Tried and not kept: four classes
+// with 16-point transforms (195 and 135 us: one item's loads ahead instead of two); a 17th warp for the loads (no
+// registers left for step C; 20.5 against 15.4 us for 91 planes).
 #pragma once
 
 #include "fft_kernels.cuh"
@@ -28,19 +37,18 @@ namespace fc {
 constexpr int BIG_MAX_SMS = 160;  // scratch is sized for this many tiles in flight
 
 struct BigGeom {
-    static constexpr int N = 128, M = 64, NC = 65, L = 32, H = 32, G = 8;
-    static constexpr int TEAM = 256, TEAMS = 2, THREADS = 512, RING = 3;
-    static constexpr int ROWS = 64;                              // rows per chunk (four threads per row)
-    static constexpr int KC = ROWS / G;                          // rows ky per chunk
-    static constexpr int CHUNKS = M / KC;
-    static constexpr int PITCH = N + 2;                          // float2 per row: 16-byte multiple, odd in 16-byte units
-    static constexpr size_t BUF = (size_t)ROWS * PITCH * 8;
-    static constexpr size_t STAGE = (size_t)2 * N * ROWS * 4;
+    static constexpr int N = 128, M = 64, NC = 65, G = 8, T = 512, TEAM = 256, CLASSES = 8, HI = 4, RING = 6;
+    static constexpr size_t STAGE = (size_t)2 * N * HI * G * 4;  // a box: [part*N + kx][hi][plane]
+    // the same box as rows of 64 pairs of columns in 16-byte units (re, re', im, im'); pair m = a + 8b stands at 9a + b:
+    // lanes over the planes (B) and lanes over the pairs (A) are conflict-free
+    static constexpr int RP = 72, PP = HI * RP + 1;
+    static constexpr size_t ROWS = (size_t)G * PP * 16;
+    static constexpr size_t BUF = ((ROWS > STAGE ? ROWS : STAGE) + 127) / 128 * 128;
     static constexpr size_t STAGE_NY = (size_t)2 * N * G * 4;
-    static constexpr size_t SCRATCH_PER_TILE = (size_t)G * M * N * 8;
-    static constexpr size_t SMEM = RING * (BUF + STAGE_NY);   // a chunk 0 brings its row ky = n/2 along
-    static_assert(STAGE <= BUF && BUF % 128 == 0, "a buffer holds a chunk's spectrum, then its rows");
-    static_assert(TEAM == 4 * ROWS && M % KC == 0, "thread roles");
+    static constexpr size_t SMEM = RING * BUF + STAGE_NY;
+    // scratch of a tile: [class][plane][j][pair], 16 bytes each
+    static constexpr int S_J = 64, S_PLANE = 8 * S_J, S_CLASS = G * S_PLANE;
+    static constexpr size_t SCRATCH_PER_TILE = (size_t)CLASSES * S_CLASS * 16;
 };
 
 static inline size_t big_scratch_bytes(int n) {
@@ -64,6 +72,43 @@ static bool big_make_map(CUtensorMap* map, const float* spec, const FftParams& p
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// w_64^{t k} (between the two 8-point steps of a row of 64 pairs), both components duplicated for packed
+// operations, and w_128^{t + 8r} (the butterfly between the halves of a pair)
+struct BigTwiddles { unsigned long long c[8][8], s[8][8]; float ec[8][8], es[8][8]; };
+constexpr BigTwiddles make_big_twiddles() {
+    BigTwiddles w{};
+    for (int t = 0; t < 8; ++t)
+        for (int k = 0; k < 8; ++k) {
+            w.c[t][k] = f2_const(static_cast<float>(cx_cos2pi(t * k, 64)));
+            w.s[t][k] = f2_const(static_cast<float>(cx_sin2pi(t * k, 64)));
+            w.ec[t][k] = static_cast<float>(cx_cos2pi(t + 8 * k, 128));
+            w.es[t][k] = static_cast<float>(cx_sin2pi(t + 8 * k, 128));
+        }
+    return w;
+}
+__constant__ BigTwiddles c_big_tw = make_big_twiddles();
+// (re, im) times w = (c, -s)
+__device__ __forceinline__ void big_rotate(F2& re, F2& im, unsigned long long c_, unsigned long long s_) {
+    const F2 c{c_}, s{s_};
+    const F2 x = f2_fma(s, im, f2_mul(c, re));
+    im = f2_mul(c, im) - f2_mul(s, re);
+    re = x;
+}
+// [2][N][NC][R][ld] as (col, row, lo, hi, part*N + kx) with ky = L hi + lo; boxes of all hi
+template <int L>
+static bool big_make_class_map(CUtensorMap* map, const float* spec, const FftParams& p) {
+    tc_encode_fn enc = tc_get_encode();
+    if (!enc) return false;
+    constexpr int N = BigGeom::N, NC = BigGeom::NC;
+    const cuuint64_t mat = (cuuint64_t)p.R * p.ld * 4;
+    cuuint64_t dims[5] = {(cuuint64_t)p.C, (cuuint64_t)p.R, L, 64 / L, (cuuint64_t)2 * N};
+    cuuint64_t strides[4] = {(cuuint64_t)p.ld * 4, mat, mat * L, mat * NC};
+    cuuint32_t box[5] = {8u, 1u, 1u, 64u / L, (cuuint32_t)2 * N};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float*>(spec), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 __device__ __forceinline__ void fk_tma_store_4d(const CUtensorMap* map, uint32_t src, int c0, int c1,
                                                 int c2, int c3) {
     asm volatile(
@@ -90,187 +135,282 @@ __device__ __forceinline__ void fk_tma_load_4d_once(uint32_t dst, const CUtensor
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(once)
         : "memory");
 }
-template <int TEAM>
-__device__ __forceinline__ void big_team_sync(int team) {
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(TEAM) : "memory");
+__device__ __forceinline__ void fk_tma_load_5d_once(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
+                                                    int c4, uint32_t bar) {
+    unsigned long long once;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(once));
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "l"(once)
+        : "memory");
 }
 // Barrier over the CTAs of a tile; orders their accesses to the scratch.
 __device__ __forceinline__ void big_tile_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// Barrier over the team that works on one box.
+__device__ __forceinline__ void big_team_sync(int team) {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(BigGeom::TEAM) : "memory");
+}
 
-__global__ void __launch_bounds__(BigGeom::THREADS, 1)
+// Phase A of class R: 8 rows of a pair of columns (row(box, hi) -> 16-byte unit), 8-point FFT, twiddle; put(j, value).
+// release() comes when the rows are in registers.
+template <int R, class Row, class Release, class Put>
+__device__ __forceinline__ void big_column(Row&& row, Release&& release, Put&& put) {
+    if constexpr (R == 0) {
+        F2 Xr[9], Xi[9], g[16];
+        static_for<8>([&](auto K) __attribute__((always_inline)) {              // row ky = 8k
+            constexpr int k = decltype(K)::value;
+            const ulonglong2 v = row(k & 1, k / 2);
+            Xr[k].b = v.x; Xi[k].b = v.y;
+        });
+        Xr[8] = Xi[0]; Xi[0] = Xi[8] = F2{0};
+        release();
+        irfft<16>(Xr, Xi, g);
+        static_for<8>([&](auto J) __attribute__((always_inline)) {              // terms 0 and 8 of the last step
+            constexpr int j = decltype(J)::value;
+            put(J, make_ulonglong2(vmul(0.5f, g[j] + g[j + 8]).b, vmul(0.5f, g[j] - g[j + 8]).b));
+        });
+    } else {
+        F2 ar[8], ai[8];
+        static_for<8>([&](auto Mm) __attribute__((always_inline)) {             // row ky = 16m + R, above n/2 a conjugate
+            constexpr int m = decltype(Mm)::value;
+            const ulonglong2 v = m < 4 ? row(0, m) : row(1, 7 - m);
+            ar[m].b = v.x;
+            ai[m].b = v.y;
+            if constexpr (m >= 4) ai[m] = -ai[m];
+        });
+        release();
+        cfft<8, true>(ar, ai);
+        static_for<8>([&](auto J) __attribute__((always_inline)) {
+            constexpr int j = decltype(J)::value;
+            if constexpr (j == 0) {
+                put(J, make_ulonglong2(ar[0].b, ai[0].b));
+            } else {
+                constexpr float c = Tw<128, R * j>::c, s = Tw<128, R * j>::s;
+                put(J, make_ulonglong2(vfma(-s, ai[j], vmul(c, ar[j])).b, vfma(s, ar[j], vmul(c, ai[j])).b));
+            }
+        });
+    }
+}
+
+__global__ void __launch_bounds__(BigGeom::T, 1)
 c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ CUtensorMap tmNy,
-               const FftParams p, float2* __restrict__ scratch_all, const int cl) {
+               const __grid_constant__ FftParams p, ulonglong2* __restrict__ scratch_all, const int cl) {
     using Gm = BigGeom;
-    constexpr int N = Gm::N, M = Gm::M, L = Gm::L, H = Gm::H, G = Gm::G, KC = Gm::KC, PITCH = Gm::PITCH, RING = Gm::RING;
+    constexpr int N = Gm::N, M = Gm::M, G = Gm::G, RP = Gm::RP, PP = Gm::PP, RING = Gm::RING, PITCH = Gm::HI * G;
     extern __shared__ __align__(128) unsigned char fc_smem[];
-    __shared__ __align__(8) unsigned long long bar_storage[RING];
-    __shared__ volatile int issued[RING];   // last chunk requested into each buffer
-    const int team = threadIdx.x / Gm::TEAM, tid = threadIdx.x - team * Gm::TEAM;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int q4 = tid / Gm::ROWS, rB = tid - q4 * Gm::ROWS;            // B: (quarter, row = ky_local*8 + plane)
-    const int q2 = lane & 1;                                            // A: parity of the bins / half of the rows
+    __shared__ __align__(8) unsigned long long bars[RING + 1];
+    __shared__ volatile int dead;           // a load never landed: the barriers are still walked, nothing is waited for
+    const float* sNy = reinterpret_cast<const float*>(fc_smem + RING * Gm::BUF);
+    const uint32_t bar_ny = fk_smem_u32(&bars[RING]);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int t = warp & 7, team = warp >> 3;               // B: part of the row, box
+    const int gA = tid >> 6, mA = tid & 63;                 // A: plane, pair of columns; C: j, pair of columns
     const int hc = p.h, wc = p.w, hw = hc * wc, tpr = p.tiles_per_row;
-    const float scale = p.scale;
-    const bool acc = p.accumulate != 0;
+    const int pairs = (wc + 1) >> 1, nj = min(8, hc);       // inside the crop
+    const F2 scale = f2_pack(p.scale, p.scale);
     const int rank = (int)blockIdx.x % cl, group = (int)blockIdx.x / cl, groups = (int)gridDim.x / cl;
-    const int K = Gm::CHUNKS / cl;                                      // chunks of a tile that this CTA takes
-    float2* scratch = scratch_all + (size_t)group * (G * M * N);
+    const int K = Gm::CLASSES / cl;                         // items of a tile that this CTA takes
+    ulonglong2* scratch = scratch_all + (size_t)group * (Gm::SCRATCH_PER_TILE / 16);
+    const int tiles = group < p.num_tiles ? (p.num_tiles - group + groups - 1) / groups : 0;
+    const int items = K * tiles;
 
     dep_trigger();
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < RING; ++s) {
-            fk_mbar_init(fk_smem_u32(&bar_storage[s]), 1);
-            issued[s] = -1;
-        }
+    if (tid == 0) {
+        for (int s = 0; s <= RING; ++s) fk_mbar_init(fk_smem_u32(&bars[s]), 1);
+        dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     dep_wait();                     // no global access above this line
 
-    // The chunks of this CTA over all its tiles form one sequence: chunk `seq` uses buffer seq % RING
-    // and team seq & 1.
-    auto request = [&](int seq) {   // one thread
-        const int tile = group + (seq / K) * groups, ci = rank * K + seq % K, s = seq % RING;
-        if (tile >= p.num_tiles) return;
+    // The items of this CTA over all its tiles form one sequence; item i has buffers 2i and 2i + 1 modulo RING.
+    auto request = [&](int i) {     // one thread
+        if (i >= items || dead) return;
+        const int tile = group + (i / K) * groups, cls = rank * K + i % K, s = 2 * i % RING;
         const int row = tile / tpr, c0 = (tile - row * tpr) * G;
-        const uint32_t bar = fk_smem_u32(&bar_storage[s]);
-        fk_mbar_expect_tx(bar, (uint32_t)(Gm::STAGE + (ci == 0 ? Gm::STAGE_NY : 0)));
-        fk_tma_load_4d_once(fk_smem_u32(fc_smem + s * Gm::BUF), &tmS, c0, row, ci * KC, 0, bar);
-        if (ci == 0) fk_tma_load_4d_once(fk_smem_u32(fc_smem + RING * Gm::BUF + s * Gm::STAGE_NY), &tmNy, c0, row, M, 0, bar);
-        issued[s] = seq;
-    };
-    // Wait for chunk `seq`.  The buffer's previous chunk belongs to the other team: until that team has
-    // handed the buffer on (issued), the barrier is one phase behind and its parity would mislead.
-    auto landed = [&](int seq) -> bool {
-        const int s = seq % RING;
-        const long long t0 = clock64(), limit = p.wait_cycles > 0 ? p.wait_cycles : FK_WAIT_CYCLES;
-        bool late = false;
-        while (issued[s] < seq) {
-            const long long dt = clock64() - t0;
-            if (dt > limit && !late) {                      // report, then give the other team the default limit
-                if (p.status) atomicExch(p.status, 1);
-                late = true;
-            }
-            if (dt > limit + FK_WAIT_CYCLES) return false;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const uint32_t bar = fk_smem_u32(&bars[s + b]);
+            fk_mbar_expect_tx(bar, (uint32_t)Gm::STAGE);
+            fk_tma_load_5d_once(fk_smem_u32(fc_smem + (s + b) * Gm::BUF), &tmS, c0, row, b == 0 ? cls : (cls == 0 ? 8 : 16 - cls), 0, 0, bar);
         }
-        return fk_wait_or_report(fk_smem_u32(&bar_storage[s]), (uint32_t)(seq / RING) & 1u, p.wait_cycles, p.status);
     };
-    if (threadIdx.x == 0)
-        for (int s = 0; s < RING; ++s) request(s);
-    bool dead = false;          // a load never landed: keep walking through the barriers, stop waiting
+    auto request_ny = [&](int tile) {       // row n/2, which travels with row 0; one thread
+        if (rank != 0 || tile >= p.num_tiles || dead) return;
+        const int row = tile / tpr, c0 = (tile - row * tpr) * G;
+        fk_mbar_expect_tx(bar_ny, (uint32_t)Gm::STAGE_NY);
+        fk_tma_load_4d_once(fk_smem_u32(sNy), &tmNy, c0, row, M, 0, bar_ny);
+    };
+    if (tid == 0) {
+        request(0);
+        request_ny(group);
+        request(1);
+        request(2);
+    }
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        if (!dead && !fk_wait_or_report(bar, parity, p.wait_cycles, p.status)) dead = 1;
+    };
 
-    int seq = 0;
+    int i = 0;
+    uint32_t ny_phase = 0;
     for (int tile = group; tile < p.num_tiles; tile += groups) {
         const int row = tile / tpr, c0 = (tile - row * tpr) * G;
         const int gcount = min(G, p.C - c0);
-
-        // ---- B: rows ----
 #pragma unroll 1
-        for (int k = 0; k < K; ++k, ++seq) {
-            if ((seq & 1) != team) continue;
-            const int ci = rank * K + k, s = seq % RING;
-            unsigned char* buf = fc_smem + s * Gm::BUF;
-            if (!dead && !landed(seq)) dead = true;
-            float* st = reinterpret_cast<float*>(buf);
-            if (ci == 0) {
-                const float* sNy = reinterpret_cast<const float*>(fc_smem + RING * Gm::BUF + s * Gm::STAGE_NY);
-                // row 0 becomes X_0 + i X_{N/2}: one complex row that carries both real rows
-                for (int it = tid; it < G * N; it += Gm::TEAM) {
-                    const int g = it & (G - 1), kx = it >> 3;
-                    const float a = st[kx * Gm::ROWS + g], b = st[(N + kx) * Gm::ROWS + g];
-                    const float c = sNy[kx * G + g], d = sNy[(N + kx) * G + g];
-                    st[kx * Gm::ROWS + g] = a - d;
-                    st[(N + kx) * Gm::ROWS + g] = b + c;
+        for (int k = 0; k < K; ++k, ++i) {
+            const int cls = rank * K + k, s = 2 * i % RING;
+            // ---- B: rows of one residue ----
+            {
+                unsigned char* buf = fc_smem + (s + team) * Gm::BUF;
+                wait(fk_smem_u32(&bars[s + team]), (uint32_t)(2 * i / RING) & 1u);
+                if (cls == 0 && team == 0) wait(bar_ny, ny_phase);
+                F2 zr[8], zi[8];
+                {
+                    const float* st = reinterpret_cast<const float*>(buf) + t * PITCH + lane;
+                    const bool packed = cls == 0 && team == 0 && lane < G;              // row ky = 0
+                    const float* ny = sNy + t * G + (lane & 7);
+                    static_for<8>([&](auto U) {
+                        constexpr int u = decltype(U)::value;
+                        float ar = st[(8 * u) * PITCH], ai = st[(N + 8 * u) * PITCH];
+                        float br = st[(M + 8 * u) * PITCH], bi = st[(N + M + 8 * u) * PITCH];
+                        if (packed) {       // X_0 + i X_{N/2}: one complex row that carries both real rows
+                            ar -= ny[(N + 8 * u) * G];      ai += ny[(8 * u) * G];
+                            br -= ny[(N + M + 8 * u) * G];  bi += ny[(M + 8 * u) * G];
+                        }
+                        // even columns from the sum, odd ones from the difference times w_128^{-(t + 8u)}
+                        const float c = c_big_tw.ec[t][u], sn = c_big_tw.es[t][u];
+                        const float dr = ar - br, di = ai - bi;
+                        zr[u] = f2_pack(ar + br, vfma(-sn, di, c * dr));
+                        zi[u] = f2_pack(ai + bi, vfma(sn, dr, c * di));
+                    });
                 }
-                big_team_sync<Gm::TEAM>(team);
-            }
-            float ar[L], ai[L];
-            {
-                const float* sb = st + rB;
-                auto load = [&](auto Kx) -> float2 {
-                    constexpr int kx = decltype(Kx)::value;
-                    return make_float2(sb[kx * Gm::ROWS], sb[(N + kx) * Gm::ROWS]);
-                };
-                if (q4 == 0)      load_split4<N, true, 0>(load, ar, ai);
-                else if (q4 == 1) load_split4<N, true, 1>(load, ar, ai);
-                else if (q4 == 2) load_split4<N, true, 2>(load, ar, ai);
-                else              load_split4<N, true, 3>(load, ar, ai);
-            }
-            big_team_sync<Gm::TEAM>(team);                    // spectrum in registers: the buffer takes the rows
-            cfft<L, true>(ar, ai);                            // ar/ai[m] = value at column 4m + q4
-            float2* sRows = reinterpret_cast<float2*>(buf);
-            {
-                float2* dst = sRows + rB * PITCH + q4;
-                static_for<L>([&](auto Mm) {
-                    constexpr int m = decltype(Mm)::value;
-                    dst[4 * m] = make_float2(ar[m], ai[m]);
+                cfft<8, true>(zr, zi);
+                big_team_sync(team);                        // the box is in registers: the buffer takes the rows
+                ulonglong2* rp = reinterpret_cast<ulonglong2*>(buf) + (lane & 7) * PP + (lane >> 3) * RP;
+                static_for<8>([&](auto U) {
+                    constexpr int u = decltype(U)::value;
+                    if constexpr (u > 0) {                  // w_64^{-t u}
+                        const F2 c{c_big_tw.c[t][u]}, sn{c_big_tw.s[t][u]};
+                        const F2 x = f2_mul(c, zr[u]) - f2_mul(sn, zi[u]);
+                        zi[u] = f2_fma(sn, zr[u], f2_mul(c, zi[u]));
+                        zr[u] = x;
+                    }
+                    rp[9 * u + t] = make_ulonglong2(zr[u].b, zi[u].b);
+                });
+                big_team_sync(team);
+                static_for<8>([&](auto U) {
+                    const ulonglong2 v = rp[9 * t + decltype(U)::value];
+                    zr[decltype(U)::value].b = v.x; zi[decltype(U)::value].b = v.y;
+                });
+                cfft<8, true>(zr, zi);                      // pair m = t + 8u of columns
+                static_for<8>([&](auto U) {
+                    constexpr int u = decltype(U)::value;
+                    rp[9 * t + u] = make_ulonglong2(zr[u].b, zi[u].b);
                 });
             }
-            big_team_sync<Gm::TEAM>(team);
-            constexpr int PER_ROW = N / 2;
-#pragma unroll 4
-            for (int i = tid; i < Gm::ROWS * PER_ROW; i += Gm::TEAM) {
-                const int rr = i / PER_ROW, pc = i - rr * PER_ROW;
-                const int g = rr & (G - 1), ky = ci * KC + (rr >> 3);
-                const float4 v = *reinterpret_cast<const float4*>(sRows + rr * PITCH + 2 * pc);
-                __stcg(reinterpret_cast<float4*>(scratch + ((size_t)(g * M + ky) * N + 2 * pc)), v);
+            __syncthreads();
+            // ---- A: columns ----
+            {
+                const ulonglong2* r0 = reinterpret_cast<const ulonglong2*>(fc_smem + s * Gm::BUF) + gA * PP + 9 * (mA & 7) + (mA >> 3);
+                auto rowv = [&](int box, int hi) __attribute__((always_inline)) { return r0[box * (int)(Gm::BUF / 16) + hi * RP]; };
+                auto release = [&]() __attribute__((always_inline)) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncthreads();                        // the rows are in registers: the buffers take the item after next
+                    if (tid == 0) {
+                        request(i + RING / 2);
+                        if (cls == 0) request_ny(tile + groups);
+                    }
+                };
+                ulonglong2* dst = scratch + (size_t)cls * Gm::S_CLASS + gA * Gm::S_PLANE + mA;
+                const int live = gA < gcount && mA < pairs ? nj : 0;
+                auto put = [&](auto J, ulonglong2 v) __attribute__((always_inline)) {
+                    constexpr int j = decltype(J)::value;
+                    if (j < live) __stcg(dst + j * Gm::S_J, v);
+                };
+                switch (cls) {
+                    case 0: big_column<0>(rowv, release, put); break;
+                    case 1: big_column<1>(rowv, release, put); break;
+                    case 2: big_column<2>(rowv, release, put); break;
+                    case 3: big_column<3>(rowv, release, put); break;
+                    case 4: big_column<4>(rowv, release, put); break;
+                    case 5: big_column<5>(rowv, release, put); break;
+                    case 6: big_column<6>(rowv, release, put); break;
+                    default: big_column<7>(rowv, release, put); break;
+                }
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before the buffer's next TMA fill
-            big_team_sync<Gm::TEAM>(team);
-            if (tid == 0) request(seq + RING);
         }
+        if (rank == 0) ny_phase ^= 1u;
         big_tile_sync();                                    // the scratch is complete
 
-        // ---- A: columns; 8 groups of 16 columns per plane ----
+        // ---- C: last step of the columns, crop ----
+        if (gA < nj && mA < pairs) {
+            const int j = gA, m = mA;
+            const ulonglong2* src = scratch + j * Gm::S_J + m;
 #pragma unroll 1
-        for (int task = rank * 16 + warp; task < 8 * gcount; task += 16 * cl) {
-            const int g = task >> 3, c = (task & 7) * 16 + (lane >> 1);
-            if ((task & 7) * 16 >= wc) continue;              // warp-uniform
-            float er[H], ei[H];
-            {
-                const float2* src = scratch + (size_t)g * (M * N) + c;
-                auto X = [&](auto Kk) -> float2 { return __ldcg(src + (size_t)decltype(Kk)::value * N); };
-                if (q2 == 0) irfft_half<N, 0>(X, er, ei);
-                else         irfft_half<N, 1>(X, er, ei);
+            for (int g0 = rank; g0 < gcount; g0 += 2 * cl) {
+                ulonglong2 in[2][8];                        // two planes' loads in flight
+#pragma unroll
+                for (int b = 0; b < 2; ++b)
+                    if (g0 + b * cl < gcount)
+#pragma unroll
+                        for (int r = 0; r < 8; ++r) in[b][r] = __ldcg(src + r * Gm::S_CLASS + (g0 + b * cl) * Gm::S_PLANE);
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const int g = g0 + b * cl;
+                    if (g >= gcount) break;
+                    F2 Xr[9], Xi[9], x[16];
+                    Xr[0].b = in[b][0].x; Xr[8].b = in[b][0].y; Xi[0] = Xi[8] = F2{0};
+#pragma unroll
+                    for (int r = 1; r < 8; ++r) { Xr[r].b = in[b][r].x; Xi[r].b = in[b][r].y; }
+                    irfft<16>(Xr, Xi, x);                   // row j + 8v
+                    float* const plane = p.real_out + ((size_t)row * p.C + c0 + g) * hw;
+                    float* o = plane + (size_t)j * wc + 2 * m;
+                    const int step = 8 * wc;
+                    if (((wc | ((int)(reinterpret_cast<uintptr_t>(plane) >> 2))) & 1) == 0) {
+#pragma unroll
+                        for (int v = 0; v < 16; ++v, o += step) {
+                            if (j + 8 * v >= hc) break;
+                            F2 z = f2_mul(x[v], scale);
+                            if (p.accumulate) z = z + F2{*reinterpret_cast<const unsigned long long*>(o)};
+                            float lo, hi;
+                            f2_unpack(z, lo, hi);
+                            __stcs(reinterpret_cast<float2*>(o), make_float2(lo, hi));
+                        }
+                    } else {
+                        const bool two = 2 * m + 1 < wc;
+#pragma unroll
+                        for (int v = 0; v < 16; ++v, o += step) {
+                            if (j + 8 * v >= hc) break;
+                            float lo, hi;
+                            f2_unpack(f2_mul(x[v], scale), lo, hi);
+                            if (p.accumulate) {
+                                lo += *o;
+                                if (two) hi += o[1];
+                            }
+                            __stcs(o, lo);
+                            if (two) __stcs(o + 1, hi);
+                        }
+                    }
+                }
             }
-            __syncwarp();
-            // z_j = E_j + O'_j (rows 2j, 2j+1),  z_{j+H} = E_j - O'_j (rows N/2 + 2j, ...): q2 = 0 holds E
-            // and forms the first, q2 = 1 holds O' and forms the second
-            const bool live = c < wc;
-            float* out = p.real_out + ((size_t)row * p.C + c0 + g) * hw + (size_t)(q2 * M) * wc + c;
-            const int rows = live ? hc - q2 * M : 0;          // rows of this lane's half that are kept
-            static_for<H>([&](auto J) {
-                constexpr int j = decltype(J)::value;
-                const float tr = __shfl_xor_sync(0xffffffffu, er[j], 1), ti = __shfl_xor_sync(0xffffffffu, ei[j], 1);
-                float zr = (q2 == 0 ? er[j] + tr : tr - er[j]) * scale;
-                float zi = (q2 == 0 ? ei[j] + ti : ti - ei[j]) * scale;
-                float* o = out + (2 * j) * wc;
-                if (2 * j < rows) {
-                    if (acc) zr += *o;
-                    __stcs(o, zr);
-                }
-                if (2 * j + 1 < rows) {
-                    if (acc) zi += o[wc];
-                    __stcs(o + wc, zi);
-                }
-            });
         }
         big_tile_sync();                                    // the scratch may be rewritten
     }
 }
 
-// CTAs that share a tile.  One when every tile gets an SM of its own and pairs would take a second, partly
-// empty round (128 tiles of 128 x 128 planes: 52 us, 59 with two); two when there are more (512 tiles: 241 us,
-// 252 with one and 471 with four, whose clusters leave SMs empty) or tiles for at most half of the SMs; more
-// where SMs would still be idle (14 tiles of 97 x 101 planes: 57 us with one CTA per tile, 34 with two, 23
-// with four or eight).
-static inline int big_cluster(long long tiles, int slots) {
-    if (8 * tiles <= slots) return 8;
-    if (4 * tiles <= slots) return 4;
-    return 2 * tiles > slots && tiles <= slots ? 1 : 2;
+// CTAs that share a tile: as many as find SMs (clusters of eight and four stay inside a GPC, so that not all SMs can
+// hold them), else two, whose rounds are finer than those of one; one where a round of single CTAs takes all tiles and
+// these are less than half full, so that step C, which a pair would share, is short.
+// Planes of 120 x 120, us with 1 / 2 / 4 / 8 CTAs: 3 tiles 48 / 30 / 19.5 / 15; 18 tiles 48 / 30 / 20.5 / 25.5; 36 tiles
+// 49 / 30 / 36 / 40; 144 tiles 63.5 / 58 / 102 / 141; 512 tiles 234 / 179 / 375 / 487.  96 tiles of 3 planes 36 / 40 / 46 / 77.
+static inline int big_cluster(long long tiles, int planes, int slots) {
+    if (16 * tiles <= slots) return 8;
+    if (6 * tiles <= slots) return 4;
+    return 2 * tiles > slots && tiles <= slots && 2 * planes <= BigGeom::G ? 1 : 2;
 }
 
 static cudaError_t launch_c2r_big(FftParams p, float* scratch, size_t scratch_bytes, cudaStream_t st) {
@@ -279,12 +419,12 @@ static cudaError_t launch_c2r_big(FftParams p, float* scratch, size_t scratch_by
     CUtensorMap tm, tmny;
     memset(&tm, 0, sizeof(tm));
     memset(&tmny, 0, sizeof(tmny));
-    if (!big_make_map<128>(&tm, p.spec_in, p, Gm::KC) || !big_make_map<128>(&tmny, p.spec_in, p, 1))
+    if (!big_make_class_map<16>(&tm, p.spec_in, p) || !big_make_map<128>(&tmny, p.spec_in, p, 1))
         return cudaErrorInvalidValue;
     int slots = 0;
-    const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(c2r_big_kernel), Gm::THREADS, Gm::SMEM, 1 << 20, &slots);
+    const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(c2r_big_kernel), Gm::T, Gm::SMEM, 1 << 20, &slots);
     if (e != cudaSuccess) return e;
-    const int cl = big_cluster(p.num_tiles, slots);
+    const int cl = big_cluster(p.num_tiles, p.C, slots);
     long long groups = slots / cl;
     if (groups < 1) groups = 1;
     if (groups > p.num_tiles) groups = p.num_tiles;
@@ -292,8 +432,8 @@ static cudaError_t launch_c2r_big(FftParams p, float* scratch, size_t scratch_by
     if (fit < 1) return cudaErrorInvalidValue;
     if (groups > fit) groups = fit;
     const dim3 grid((unsigned)(groups * cl));
-    float2* sc = reinterpret_cast<float2*>(scratch);
-    return dep_launch(p.overlap != 0, cl, c2r_big_kernel, grid, dim3(Gm::THREADS), Gm::SMEM, st, tm, tmny, p, sc, cl);
+    ulonglong2* sc = reinterpret_cast<ulonglong2*>(scratch);
+    return dep_launch(p.overlap != 0, cl, c2r_big_kernel, grid, dim3(Gm::T), Gm::SMEM, st, tm, tmny, p, sc, cl);
 }
 
 // Which plane sizes take the transforms of this file and fft_split.cuh.

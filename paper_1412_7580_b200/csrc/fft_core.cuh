@@ -213,10 +213,10 @@ FC_HD void rfft(const V (&x)[N], V (&Xr)[N / 2 + 1], V (&Xi)[N / 2 + 1]) {
 // Z'_k = (X_k + conj X_{M-k}) + i w_N^{-k} (X_k - conj X_{M-k}); the
 // unnormalised inverse FFT_M of Z' is N (x_2j + i x_2j+1).
 // ---------------------------------------------------------------------------
-template <int N>
-FC_HD void irfft(const float (&Xr)[N / 2 + 1], const float (&Xi)[N / 2 + 1], float (&x)[N]) {
+template <int N, class V>
+FC_HD void irfft(const V (&Xr)[N / 2 + 1], const V (&Xi)[N / 2 + 1], V (&x)[N]) {
     constexpr int M = N / 2;
-    float zr[M], zi[M];
+    V zr[M], zi[M];
     zr[0] = Xr[0] + Xr[M];
     zi[0] = Xr[0] - Xr[M];
     if constexpr (M >= 2) {
@@ -228,12 +228,12 @@ FC_HD void irfft(const float (&Xr)[N / 2 + 1], const float (&Xi)[N / 2 + 1], flo
             constexpr int k = decltype(K)::value + 1;
             constexpr float c = Tw<N, k>::c;
             constexpr float s = Tw<N, k>::s;
-            const float pr = Xr[k], pi = Xi[k], qr = Xr[M - k], qi = Xi[M - k];
-            const float er = pr + qr, ei = pi - qi;   // E = P + conj Q
-            const float dr = pr - qr, di = pi + qi;   // D = P - conj Q
+            const V pr = Xr[k], pi = Xi[k], qr = Xr[M - k], qi = Xi[M - k];
+            const V er = pr + qr, ei = pi - qi;   // E = P + conj Q
+            const V dr = pr - qr, di = pi + qi;   // D = P - conj Q
             // U = w_N^{-k} D with w^{-k} = (c, +s): U = (c dr - s di, c di + s dr)
-            const float ur = vfma(-s, di, vmul(c, dr));
-            const float ui = vfma(s, dr, vmul(c, di));
+            const V ur = vfma(-s, di, vmul(c, dr));
+            const V ui = vfma(s, dr, vmul(c, di));
             // Z'_k = E + iU = (er - ui, ei + ur); Z'_{M-k} = conj(E - iU) = (er + ui, -(ei - ur))
             zr[k] = er - ui;     zi[k] = ei + ur;
             zr[M - k] = er + ui; zi[M - k] = ur - ei;

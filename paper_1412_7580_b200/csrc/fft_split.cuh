@@ -47,28 +47,6 @@ struct SplitGeom {
     static constexpr size_t SMEM = BUF + NY;
 };
 
-// w_64^{t k} (between the two 8-point steps of a row), both components duplicated for packed operations,
-// and w_128^{t + 8r} (the last step)
-struct SplitTwiddles { unsigned long long c[8][8], s[8][8]; float ec[8][8], es[8][8]; };
-constexpr SplitTwiddles make_split_twiddles() {
-    SplitTwiddles w{};
-    for (int t = 0; t < 8; ++t)
-        for (int k = 0; k < 8; ++k) {
-            w.c[t][k] = f2_const(static_cast<float>(cx_cos2pi(t * k, 64)));
-            w.s[t][k] = f2_const(static_cast<float>(cx_sin2pi(t * k, 64)));
-            w.ec[t][k] = static_cast<float>(cx_cos2pi(t + 8 * k, 128));
-            w.es[t][k] = static_cast<float>(cx_sin2pi(t + 8 * k, 128));
-        }
-    return w;
-}
-__constant__ SplitTwiddles c_split_tw = make_split_twiddles();
-// (re, im) times w = (c, -s)
-__device__ __forceinline__ void split_rotate(F2& re, F2& im, unsigned long long c_, unsigned long long s_) {
-    const F2 c{c_}, s{s_};
-    const F2 x = f2_fma(s, im, f2_mul(c, re));
-    im = f2_mul(c, im) - f2_mul(s, re);
-    re = x;
-}
 // Last step of a row: E and O, the transforms of the even and the odd columns, are the two halves of a packed
 // value; X_q = E + w_N^q O and X_{q + N/2} = E - w_N^q O, w = (c, -s).
 __device__ __forceinline__ void split_last(F2 re, F2 im, float c, float s, float& ar, float& ai, float& br, float& bi) {
@@ -81,20 +59,6 @@ __device__ __forceinline__ void split_last(F2 re, F2 im, float c, float s, float
     bi = vfma(2.0f, ei, -ai);
 }
 
-// [2][N][NC][R][ld] as (col, row, lo, hi, part*N + kx) with ky = 8 hi + lo
-static inline bool split_make_map(CUtensorMap* map, const float* spec, const FftParams& p) {
-    tc_encode_fn enc = tc_get_encode();
-    if (!enc) return false;
-    constexpr int N = SplitGeom::N, NC = SplitGeom::NC;
-    const cuuint64_t mat = (cuuint64_t)p.R * p.ld * 4;
-    cuuint64_t dims[5] = {(cuuint64_t)p.C, (cuuint64_t)p.R, 8, 8, (cuuint64_t)2 * N};
-    cuuint64_t strides[4] = {(cuuint64_t)p.ld * 4, mat, mat * 8, mat * NC};
-    cuuint32_t box[5] = {8u, 1u, 1u, 8u, (cuuint32_t)2 * N};
-    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float*>(spec), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 __device__ __forceinline__ void fk_tma_store_5d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3, int c4) {
     asm volatile(
         "cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];"
@@ -280,7 +244,7 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
             cfft<8, false>(zr[b], zi[b]);
             static_for<8>([&](auto K) {
                 constexpr int k = decltype(K)::value;
-                if constexpr (k > 0) split_rotate(zr[b][k], zi[b][k], c_split_tw.c[t][k], c_split_tw.s[t][k]);
+                if constexpr (k > 0) big_rotate(zr[b][k], zi[b][k], c_big_tw.c[t][k], c_big_tw.s[t][k]);
                 rp[8 * k + t] = make_ulonglong2(zr[b][k].b, zi[b][k].b);
             });
         }
@@ -301,7 +265,7 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
             static_for<8>([&](auto Rr) {
                 constexpr int r = decltype(Rr)::value;
                 float ar, ai, br, bi;
-                split_last(zr[b][r], zi[b][r], c_split_tw.ec[t][r], c_split_tw.es[t][r], ar, ai, br, bi);
+                split_last(zr[b][r], zi[b][r], c_big_tw.ec[t][r], c_big_tw.es[t][r], ar, ai, br, bi);
                 o[(8 * r) * (8 * G)] = ar;           o[(N + 8 * r) * (8 * G)] = ai;
                 o[(M + 8 * r) * (8 * G)] = br;       o[(N + M + 8 * r) * (8 * G)] = bi;
             });
@@ -345,11 +309,11 @@ static cudaError_t launch_r2c_split(FftParams pa, const FftParams* pb_in, cudaSt
     CUtensorMap m[4];
     memset(m, 0, sizeof(m));
     if (!fill_tiling<Gm::G>(pa)) return cudaErrorInvalidValue;
-    if (!split_make_map(&m[0], pa.spec_out, pa) || !big_make_map<128>(&m[1], pa.spec_out, pa, 1)) return cudaErrorInvalidValue;
+    if (!big_make_class_map<8>(&m[0], pa.spec_out, pa) || !big_make_map<128>(&m[1], pa.spec_out, pa, 1)) return cudaErrorInvalidValue;
     if (pb_in) {
         pb = *pb_in;
         if (!fill_tiling<Gm::G>(pb)) return cudaErrorInvalidValue;
-        if (!split_make_map(&m[2], pb.spec_out, pb) || !big_make_map<128>(&m[3], pb.spec_out, pb, 1)) return cudaErrorInvalidValue;
+        if (!big_make_class_map<8>(&m[2], pb.spec_out, pb) || !big_make_map<128>(&m[3], pb.spec_out, pb, 1)) return cudaErrorInvalidValue;
     }
     const long long items = (long long)Gm::CLASSES * ((long long)pa.num_tiles + pb.num_tiles);
     if (items > 0x3fffffffLL) return cudaErrorInvalidValue;
