@@ -95,15 +95,15 @@ __device__ __forceinline__ void big_rotate(F2& re, F2& im, unsigned long long c_
     re = x;
 }
 // [2][N][NC][R][ld] as (col, row, lo, hi, part*N + kx) with ky = L hi + lo; boxes of all hi
-template <int L>
+template <int N, int L>
 static bool big_make_class_map(CUtensorMap* map, const float* spec, const FftParams& p) {
     tc_encode_fn enc = tc_get_encode();
     if (!enc) return false;
-    constexpr int N = BigGeom::N, NC = BigGeom::NC;
+    constexpr int NC = N / 2 + 1, HI = N / 2 / L;
     const cuuint64_t mat = (cuuint64_t)p.R * p.ld * 4;
-    cuuint64_t dims[5] = {(cuuint64_t)p.C, (cuuint64_t)p.R, L, 64 / L, (cuuint64_t)2 * N};
+    cuuint64_t dims[5] = {(cuuint64_t)p.C, (cuuint64_t)p.R, L, HI, (cuuint64_t)2 * N};
     cuuint64_t strides[4] = {(cuuint64_t)p.ld * 4, mat, mat * L, mat * NC};
-    cuuint32_t box[5] = {8u, 1u, 1u, 64u / L, (cuuint32_t)2 * N};
+    cuuint32_t box[5] = {8u, 1u, 1u, (cuuint32_t)HI, (cuuint32_t)2 * N};
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float*>(spec), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -419,7 +419,7 @@ static cudaError_t launch_c2r_big(FftParams p, float* scratch, size_t scratch_by
     CUtensorMap tm, tmny;
     memset(&tm, 0, sizeof(tm));
     memset(&tmny, 0, sizeof(tmny));
-    if (!big_make_class_map<16>(&tm, p.spec_in, p) || !big_make_map<128>(&tmny, p.spec_in, p, 1))
+    if (!big_make_class_map<128, 16>(&tm, p.spec_in, p) || !big_make_map<128>(&tmny, p.spec_in, p, 1))
         return cudaErrorInvalidValue;
     int slots = 0;
     const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(c2r_big_kernel), Gm::T, Gm::SMEM, 1 << 20, &slots);

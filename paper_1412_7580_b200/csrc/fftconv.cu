@@ -18,7 +18,6 @@
 #include "fft_big.cuh"
 #include "fft_split.cuh"
 #include "fft_small.cuh"
-#include "fft_sub.cuh"
 #include "fft1d.cuh"
 
 #define FFTCONV_API extern "C" __attribute__((visibility("default")))
@@ -277,10 +276,8 @@ int run_pass(conv_plan_s* plan, int pass, const float* a_in, const float* b_in, 
     // One forward launch: both operands in one kernel, or one operand.
     auto forward = [&](const fc::FftParams& pa, const fc::FftParams* pb) -> cudaError_t {
         g_launches.fetch_add(1, std::memory_order_relaxed);
-        if (big) return fc::launch_r2c_split(pa, pb, st);
-        // wide planes at n = 64: the sub-batched kernels (rows twice as long); else the plain ones
-        const cudaError_t es = fc::launch_r2c_sub_any(plan->n, pa, pb, st);
-        return es != cudaErrorNotSupported ? es : fc::launch_r2c<true>(plan->n, pa, pb, st);
+        if (big) return fc::launch_r2c_split<128>(pa, pb, st);
+        return fc::split_pays(plan->n, pa, pb) ? fc::launch_r2c_split<64>(pa, pb, st) : fc::launch_r2c<true>(plan->n, pa, pb, st);
     };
     // Small planes (the filters of fprop and bprop) take the pruned-DFT kernel, whose stores are
     // whole 128-byte lines; it runs after the other operand's transform, as its programmatic

@@ -1,4 +1,4 @@
-"""Transforms of planes that need the basis 128: the kernels choose their loads by the parity of the row length
+"""Transforms of planes that need the bases 64 and 128: the kernels choose their loads by the parity of the row length
 and by the alignment of the tensor, split the rows over work items and clip ragged tiles of 8 planes."""
 import numpy as np
 import pytest
@@ -6,21 +6,26 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-# (S, f, f', h, w, kh, kw), samples by which the tensors are shifted in memory
+# (S, f, f', h, w, kh, kw, n), samples by which the tensors are shifted in memory
 @pytest.mark.parametrize("dims,shift", [
-    ((2, 9, 3, 128, 128, 5, 5), 0),        # pairs of columns; every row and column in use
-    ((2, 9, 3, 128, 128, 5, 5), 1),        # the same from an address that is no multiple of 8 bytes
-    ((1, 8, 10, 66, 127, 3, 4), 0),        # odd rows, the last column has no partner; dy's rows are even
-    ((3, 1, 17, 127, 66, 2, 3), 0),        # one plane in a tile, tiles of 8 + 8 + 1
-    ((1, 7, 8, 40, 101, 9, 3), 2),         # fewer rows than half the basis
-    ((2, 3, 5, 97, 20, 97, 2), 0),         # narrow planes, kernel as high as the plane
+    ((2, 9, 3, 128, 128, 5, 5, 128), 0),   # pairs of columns; every row and column in use
+    ((2, 9, 3, 128, 128, 5, 5, 128), 1),   # the same from an address that is no multiple of 8 bytes
+    ((1, 8, 10, 66, 127, 3, 4, 128), 0),   # odd rows, the last column has no partner; dy's rows are even
+    ((3, 1, 17, 127, 66, 2, 3, 128), 0),   # one plane in a tile, tiles of 8 + 8 + 1
+    ((1, 7, 8, 40, 101, 9, 3, 128), 2),    # fewer rows than half the basis
+    ((2, 3, 5, 97, 20, 97, 2, 128), 0),    # narrow planes, kernel as high as the plane
+    ((2, 9, 12, 64, 64, 14, 5, 64), 0),
+    ((2, 9, 12, 64, 64, 5, 14, 64), 1),
+    ((1, 8, 10, 33, 63, 3, 4, 64), 0),
+    ((3, 5, 17, 61, 20, 15, 3, 64), 3),    # narrow planes and filters too high for the small-plane kernel
+    ((2, 4, 3, 57, 58, 3, 3, 64), 0),      # no tile more than half full
 ])
 def test_passes_against_oracle(dims, shift):
     import torch
     import oracle
     import paper_1412_7580_b200 as fc
     from paper_1412_7580_b200 import workloads as wl
-    s = wl.ConvShape("large_planes", *dims, 128, cfg=9, point=sum(dims) + shift)
+    s = wl.ConvShape("large_planes", *dims, cfg=9, point=sum(dims) + shift)
     host = wl.make_x(s), wl.make_w(s), wl.make_dy(s)
 
     def shifted(a):
