@@ -58,14 +58,14 @@ static inline size_t big_scratch_bytes(int n) {
 // Planar spectrum [2][N][NC][R][ld] seen as a 4-D tensor (col, row, ky, part*N + kx):
 // bin = kx*NC + ky and the parts are N*NC bins apart, so the last stride is uniform.
 template <int N>
-static bool big_make_map(CUtensorMap* map, const float* spec, const FftParams& p, int box_ky) {
+static bool big_make_map(CUtensorMap* map, const float* spec, const FftParams& p, int box_ky, int planes = 8) {
     tc_encode_fn enc = tc_get_encode();
     if (!enc) return false;
     constexpr int NC = N / 2 + 1;
     const cuuint64_t mat = (cuuint64_t)p.R * p.ld * 4;
     cuuint64_t dims[4] = {(cuuint64_t)p.C, (cuuint64_t)p.R, (cuuint64_t)NC, (cuuint64_t)2 * N};
     cuuint64_t strides[3] = {(cuuint64_t)p.ld * 4, mat, mat * NC};
-    cuuint32_t box[4] = {8u, 1u, (cuuint32_t)box_ky, (cuuint32_t)2 * N};
+    cuuint32_t box[4] = {(cuuint32_t)planes, 1u, (cuuint32_t)box_ky, (cuuint32_t)2 * N};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(spec), dims, strides, box,
                estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -96,14 +96,14 @@ __device__ __forceinline__ void big_rotate(F2& re, F2& im, unsigned long long c_
 }
 // [2][N][NC][R][ld] as (col, row, lo, hi, part*N + kx) with ky = L hi + lo; boxes of all hi
 template <int N, int L>
-static bool big_make_class_map(CUtensorMap* map, const float* spec, const FftParams& p) {
+static bool big_make_class_map(CUtensorMap* map, const float* spec, const FftParams& p, int planes = 8) {
     tc_encode_fn enc = tc_get_encode();
     if (!enc) return false;
     constexpr int NC = N / 2 + 1, HI = N / 2 / L;
     const cuuint64_t mat = (cuuint64_t)p.R * p.ld * 4;
     cuuint64_t dims[5] = {(cuuint64_t)p.C, (cuuint64_t)p.R, L, HI, (cuuint64_t)2 * N};
     cuuint64_t strides[4] = {(cuuint64_t)p.ld * 4, mat, mat * L, mat * NC};
-    cuuint32_t box[5] = {8u, 1u, 1u, (cuuint32_t)HI, (cuuint32_t)2 * N};
+    cuuint32_t box[5] = {(cuuint32_t)planes, 1u, 1u, (cuuint32_t)HI, (cuuint32_t)2 * N};
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float*>(spec), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

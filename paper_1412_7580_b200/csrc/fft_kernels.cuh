@@ -52,12 +52,11 @@
 
 namespace fc {
 
-// LAYOUT_FREQ_TMA / _DIRECT: planar frequency-major spectra, moved by the TMA or
-// by plain per-thread accesses; LAYOUT_BARE: [plane][n][n/2+1] interleaved pairs, accessed
-// by the threads directly; LAYOUT_BARE_STAGED: the same layout, but a tile's planes (which
+// LAYOUT_FREQ_TMA: planar frequency-major spectra, moved by the TMA; LAYOUT_BARE:
+// [plane][n][n/2+1] interleaved pairs, accessed by the threads directly; LAYOUT_BARE_STAGED: the same layout, but a tile's planes (which
 // are contiguous in memory) travel between global and shared memory as one bulk
 // asynchronous copy per plane and the threads only touch the shared-memory image.
-enum { LAYOUT_FREQ_TMA = 0, LAYOUT_BARE = 1, LAYOUT_FREQ_DIRECT = 2, LAYOUT_BARE_STAGED = 3 };
+enum { LAYOUT_FREQ_TMA = 0, LAYOUT_BARE = 1, LAYOUT_BARE_STAGED = 2 };
 
 // Pitch (in complex elements) of one plane of the bare layout in shared memory: the plane
 // itself, rounded up so that every plane starts on a 16-byte boundary, plus a few elements so
@@ -595,18 +594,9 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
             cfft<M, false>(ar, ai);                     // ar/ai[k] = F[kx = 2k+q]
 
             if constexpr (!BARE) {
-                // element (part, bin = kx*NC + ky, plane g): staging offset (part*B + bin)*G + g,
-                // global offset ((part*B + bin)*R + row)*ld + col
-                float* o;
-                size_t sb, sp;      // strides of one bin and of one part
-                if constexpr (TMA) {
-                    o = sStage + (q * NC + kyp) * G + gB;
-                    sb = G; sp = (size_t)B * G;
-                } else {
-                    const size_t mat = (size_t)p.R * p.ld;
-                    o = p.spec_out + (size_t)(q * NC + kyp) * mat + (size_t)row * p.ld + c0 + gB;
-                    sb = mat; sp = (size_t)B * mat;
-                }
+                // element (part, bin = kx*NC + ky, plane g): staging offset (part*B + bin)*G + g
+                float* o = sStage + (q * NC + kyp) * G + gB;
+                constexpr size_t sb = G, sp = (size_t)B * G;        // strides of one bin and of one part
                 // With the TMA staging the packed row is written like any other row and taken
                 // apart afterwards by the whole CTA (below): the lanes that hold it then do no
                 // more work than the rest.
@@ -839,11 +829,10 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
                 phase ^= 1u;
             }
             // Rows ky = 0 and ky = N/2 are real after the column pass, so they travel through
-            // the row pass as one complex row Z = X_0 + i X_{N/2}.  For N <= 32 the whole CTA
+            // the row pass as one complex row Z = X_0 + i X_{N/2}.  The whole CTA
             // forms Z in the staging tile first (one element per thread, one more barrier), so
             // that the two warps holding the packed rows do no more work than the others.
-            constexpr bool WIDE_COMBINE = (N <= 64);
-            if constexpr (WIDE_COMBINE) {
+            {
                 // The two rows are Hermitian in kx, and their bins kx > N/2 are never read: the
                 // thread of kx <= N/2 also forms Z[N - kx] = conj X_0[kx] + i conj X_{N/2}[kx]
                 // (the contraction leaves those bins out, see GemmParams::herm_n).
@@ -865,12 +854,7 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
             const float* sb = sStage + kyp * G + gB;
             auto load = [&](auto Kx) -> float2 {
                 constexpr int kx = decltype(Kx)::value;
-                float2 v = make_float2(sb[kx * NC * G], sb[(B + kx * NC) * G]);
-                if (!WIDE_COMBINE && packed) {       // row ky = N/2 rides as i times itself
-                    v.x -= sb[(B + kx * NC + M) * G];
-                    v.y += sb[(kx * NC + M) * G];
-                }
-                return v;
+                return make_float2(sb[kx * NC * G], sb[(B + kx * NC) * G]);
             };
             if (q == 0) load_split<N, true, 0>(load, ar, ai);
             else        load_split<N, true, 1>(load, ar, ai);
@@ -915,33 +899,21 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
             if (is_fetcher && tile + (int)gridDim.x < p.num_tiles) fetch_bare(row_n, tcol_n);
         } else {
             if (gB < gcount) {
-                const size_t mat = (size_t)p.R * p.ld;
-                const float* fbase = p.spec_in + (size_t)kyp * mat + (size_t)row * p.ld + c0 + gB;
                 const float2* bbase = reinterpret_cast<const float2*>(p.spec_in) +
                                       ((size_t)row * p.C + c0 + gB) * (size_t)(N * NC);
                 auto load = [&](auto Kx) -> float2 {
                     constexpr int kx = decltype(Kx)::value;
-                    float2 v;
-                    if constexpr (LAYOUT == LAYOUT_FREQ_DIRECT) {
-                        const float* a = fbase + (size_t)(kx * NC) * mat;
-                        v = make_float2(__ldg(a), __ldg(a + (size_t)B * mat));
-                        if (packed) {
-                            v.x -= __ldg(a + (size_t)(B + M) * mat);
-                            v.y += __ldg(a + (size_t)M * mat);
-                        }
-                    } else {
-                        auto fetch = [&](int ky) -> float2 {
-                            if (kx <= M) return __ldg(bbase + ky * NC + kx);
-                            float2 t = __ldg(bbase + ((N - ky) & (N - 1)) * NC + (N - kx));
-                            t.y = -t.y;
-                            return t;
-                        };
-                        v = fetch(kyp);
-                        if (packed) {
-                            const float2 nq = fetch(M);
-                            v.x -= nq.y;
-                            v.y += nq.x;
-                        }
+                    auto fetch = [&](int ky) -> float2 {
+                        if (kx <= M) return __ldg(bbase + ky * NC + kx);
+                        float2 t = __ldg(bbase + ((N - ky) & (N - 1)) * NC + (N - kx));
+                        t.y = -t.y;
+                        return t;
+                    };
+                    float2 v = fetch(kyp);
+                    if (packed) {
+                        const float2 nq = fetch(M);
+                        v.x -= nq.y;
+                        v.y += nq.x;
                     }
                     return v;
                 };
@@ -1059,11 +1031,11 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
 // Host-side launchers.
 // ---------------------------------------------------------------------------
 template <int N> struct FftCfg;   // planes per CTA, buffer aliasing, min CTAs per SM, TMA staging
-template <> struct FftCfg<8>   { static constexpr int G = 32; static constexpr bool ALIAS = false, SALIAS = true;  static constexpr int MINB = 4, MINB_INV = 4; static constexpr bool TMA = true; };
-template <> struct FftCfg<16>  { static constexpr int G = 16; static constexpr bool ALIAS = false, SALIAS = false;  static constexpr int MINB = 4, MINB_INV = 4; static constexpr bool TMA = true; };
-template <> struct FftCfg<32>  { static constexpr int G = 8;  static constexpr bool ALIAS = false, SALIAS = false;  static constexpr int MINB = 2, MINB_INV = 3; static constexpr bool TMA = true; };
-template <> struct FftCfg<64>  { static constexpr int G = 4;  static constexpr bool ALIAS = false, SALIAS = false; static constexpr int MINB = 1, MINB_INV = 1; static constexpr bool TMA = true; };
-template <> struct FftCfg<128> { static constexpr int G = 2;  static constexpr bool ALIAS = true,  SALIAS = false; static constexpr int MINB = 1, MINB_INV = 1; static constexpr bool TMA = false; };
+template <> struct FftCfg<8>   { static constexpr int G = 32; static constexpr bool ALIAS = false, SALIAS = true;  static constexpr int MINB = 4, MINB_INV = 4; };
+template <> struct FftCfg<16>  { static constexpr int G = 16; static constexpr bool ALIAS = false, SALIAS = false;  static constexpr int MINB = 4, MINB_INV = 4; };
+template <> struct FftCfg<32>  { static constexpr int G = 8;  static constexpr bool ALIAS = false, SALIAS = false;  static constexpr int MINB = 2, MINB_INV = 3; };
+template <> struct FftCfg<64>  { static constexpr int G = 4;  static constexpr bool ALIAS = false, SALIAS = false; static constexpr int MINB = 1, MINB_INV = 1; };
+template <> struct FftCfg<128> { static constexpr int G = 2;  static constexpr bool ALIAS = true,  SALIAS = false; static constexpr int MINB = 1, MINB_INV = 1; };
 
 // Bare layout staged through shared memory.  Its copies are whole planes, so a tile needs no width to move
 // long rows, and half as many planes per CTA put more planes in flight on an SM: fewer threads wait at each
@@ -1191,9 +1163,10 @@ static cudaError_t launch_r2c_layout(FftParams pa, const FftParams* pb_in, cudaS
     // the windowed variant (spatial tiling) is a separate instantiation, so that the plain
     // kernels carry none of its code
     const bool win = pa.win || (pb_in && pb.win);
-    auto kern = (win && LAYOUT == LAYOUT_FREQ_TMA) ? r2c_kernel<N, G, LAYOUT, Cfg::ALIAS, SALIAS, Cfg::MINB, LAYOUT == LAYOUT_FREQ_TMA>
+    constexpr bool WIN = LAYOUT == LAYOUT_FREQ_TMA && N <= 32;     // (windows of n = 64 have the kernel of fft_split.cuh)
+    auto kern = (win && WIN) ? r2c_kernel<N, G, LAYOUT, Cfg::ALIAS, SALIAS, Cfg::MINB, WIN>
                                                    : r2c_kernel<N, G, LAYOUT, Cfg::ALIAS, SALIAS, Cfg::MINB, false>;
-    if (win && LAYOUT != LAYOUT_FREQ_TMA) return cudaErrorInvalidValue;
+    if (win && !WIN) return cudaErrorInvalidValue;
     int grid = 0;
     cudaError_t e = persistent_grid(reinterpret_cast<const void*>(kern), N * G, smem,
                                     (long long)pa.num_tiles + pb.num_tiles, &grid);
@@ -1205,9 +1178,8 @@ static cudaError_t launch_r2c_layout(FftParams pa, const FftParams* pb_in, cudaS
 // image fits (n <= 64) and the spectrum is 16-byte aligned, else accessed by the threads.
 template <int N, bool FREQ>
 static cudaError_t launch_r2c_n(const FftParams& pa, const FftParams* pb_in, cudaStream_t st) {
-    using Cfg = FftCfg<N>;
     if constexpr (FREQ) {
-        return launch_r2c_layout<N, Cfg::TMA ? LAYOUT_FREQ_TMA : LAYOUT_FREQ_DIRECT>(pa, pb_in, st);
+        return launch_r2c_layout<N, LAYOUT_FREQ_TMA>(pa, pb_in, st);
     } else {
         if constexpr (N <= 64) {
             if ((reinterpret_cast<uintptr_t>(pa.spec_out) & 15) == 0)
@@ -1249,9 +1221,8 @@ static cudaError_t launch_c2r_layout(FftParams p, cudaStream_t st) {
 
 template <int N, bool FREQ>
 static cudaError_t launch_c2r_n(const FftParams& p, cudaStream_t st) {
-    using Cfg = FftCfg<N>;
     if constexpr (FREQ) {
-        return launch_c2r_layout<N, Cfg::TMA ? LAYOUT_FREQ_TMA : LAYOUT_FREQ_DIRECT>(p, st);
+        return launch_c2r_layout<N, LAYOUT_FREQ_TMA>(p, st);
     } else {
         if constexpr (N <= 64) {
             if ((reinterpret_cast<uintptr_t>(p.spec_in) & 15) == 0)
@@ -1268,7 +1239,7 @@ static cudaError_t launch_r2c(int n, const FftParams& p, const FftParams* second
         case 16:  return launch_r2c_n<16, FREQ>(p, second, st);
         case 32:  return launch_r2c_n<32, FREQ>(p, second, st);
         case 64:  return launch_r2c_n<64, FREQ>(p, second, st);
-        case 128: return launch_r2c_n<128, FREQ>(p, second, st);
+        case 128: if constexpr (!FREQ) return launch_r2c_n<128, FREQ>(p, second, st); else break;
     }
     return cudaErrorInvalidValue;
 }
@@ -1279,7 +1250,8 @@ static cudaError_t launch_c2r(int n, const FftParams& p, cudaStream_t st) {
         case 16:  return launch_c2r_n<16, FREQ>(p, st);
         case 32:  return launch_c2r_n<32, FREQ>(p, st);
         case 64:  return launch_c2r_n<64, FREQ>(p, st);
-        case 128: return launch_c2r_n<128, FREQ>(p, st);
+        // n = 128 has kernels of its own for the passes
+        case 128: if constexpr (!FREQ) return launch_c2r_n<128, FREQ>(p, st); else break;
     }
     return cudaErrorInvalidValue;
 }

@@ -77,25 +77,28 @@ __device__ __forceinline__ void fk_tma_store_5d(const CUtensorMap* map, uint32_t
 // bytes else; rows and columns past the plane are zeros.  The loads are volatile, so that they are issued in
 // program order, well ahead of their use (split_column): left to itself the compiler puts each load right
 // before its use and a thread has a few in flight.
-template <bool PAIR>
+// LOW (windows): the rows below `low` do not exist either.
+template <bool PAIR, bool LOW>
 struct SplitLoad {
     const float* s0;
     int pitch;                      // bytes from row to row
     int rows, rows2;                // rows that exist in the first and in the second column
+    int low;
     template <int r>
     __device__ __forceinline__ F2 get() const {
         const char* q = reinterpret_cast<const char*>(s0) + (long long)pitch * r;
+        const unsigned at = LOW ? (unsigned)(r - low) : (unsigned)r;
         if constexpr (PAIR) {
             F2 v;
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %2, %3;\n\tmov.b64 %0, 0;\n\t@p ld.global.nc.b64 %0, [%1];\n\t}"
-                         : "=l"(v.b) : "l"(q), "r"(rows), "n"(r));
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.u32 p, %2, %3;\n\tmov.b64 %0, 0;\n\t@p ld.global.nc.b64 %0, [%1];\n\t}"
+                         : "=l"(v.b) : "l"(q), "r"(rows), "r"(at));
             return v;
         } else {
             float u, v;
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1];\n\t}"
-                         : "=f"(u) : "l"(q), "r"(rows), "n"(r));
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1+4];\n\t}"
-                         : "=f"(v) : "l"(q), "r"(rows2), "n"(r));
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.u32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1];\n\t}"
+                         : "=f"(u) : "l"(q), "r"(rows), "r"(at));
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.u32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1+4];\n\t}"
+                         : "=f"(v) : "l"(q), "r"(rows2), "r"(at));
             return f2_pack(u, v);
         }
     }
@@ -104,8 +107,8 @@ struct SplitLoad {
 // Phase A of class R: first butterflies of a column, twiddles, 16-point FFT; put(row, re, im) with row = 8 *
 // (second residue) + hi; release() comes before the first put.  The samples of the next AHEAD butterflies are on
 // their way.
-template <int N, int R, bool PAIR, class Release>
-__device__ __forceinline__ void split_column(const SplitLoad<PAIR>& x, ulonglong2* dst, Release&& release) {
+template <int N, int R, class Load, class Release>
+__device__ __forceinline__ void split_column(const Load& x, ulonglong2* dst, Release&& release) {
     constexpr int V = N / 16, AHEAD = 24 / V;
     auto put = [&](auto K, F2 re, F2 im) __attribute__((always_inline)) { dst[decltype(K)::value * SplitGeom<N>::RP] = make_ulonglong2(re.b, im.b); };
     F2 ring[AHEAD][V];
@@ -174,8 +177,8 @@ __device__ __forceinline__ void split_column(const SplitLoad<PAIR>& x, ulonglong
         });
     }
 }
-template <int N, bool PAIR, class Release>
-__device__ __forceinline__ void split_class(int cls, const SplitLoad<PAIR>& x, ulonglong2* dst, Release&& release) {
+template <int N, class Load, class Release>
+__device__ __forceinline__ void split_class(int cls, const Load& x, ulonglong2* dst, Release&& release) {
     if (cls == 0)                 split_column<N, 0>(x, dst, release);
     else if (N == 64 || cls == 1) split_column<N, 1>(x, dst, release);
     else if constexpr (N == 128) {
@@ -190,6 +193,7 @@ __device__ __forceinline__ void split_prefetch(int item, int items0, const FftPa
     using Gm = SplitGeom<N>;
     const bool second = item >= items0;
     const FftParams& p = second ? p1 : p0;
+    if (p.win) return;              // the windows of a plane share its samples, which are in the L2 already for the most part
     const int it = second ? item - items0 : item;
     const int tile = it / Gm::CLASSES, cls = it - tile * Gm::CLASSES;
     const int row = tile / p.tiles_per_row, c0 = (tile - row * p.tiles_per_row) * Gm::G;
@@ -202,7 +206,7 @@ __device__ __forceinline__ void split_prefetch(int item, int items0, const FftPa
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((uint32_t)(hi - lo)) : "memory");
 }
 
-template <int N>
+template <int N, bool WIN>
 __global__ void __launch_bounds__(SplitGeom<N>::T, SplitGeom<N>::MINB)
 r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUtensorMap tmNy0,
                  const __grid_constant__ CUtensorMap tmS1, const __grid_constant__ CUtensorMap tmNy1,
@@ -231,19 +235,32 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
 
         // ---- A: columns; a pair of columns past the plane reads no sample and writes zeros ----
         {
-            const float* planes = p.real_in + ((size_t)row * p.C + c0) * (size_t)(h * w);
-            const bool live = gA < p.C - c0 && cA < w;
-            const float* s0 = planes + (live ? gA * (h * w) + cA : 0);
-            const int rows = live ? h : 0, rows2 = live && cA + 1 < w ? h : 0;
+            // a window of a larger plane: its origin (y0, x0) may lie outside, samples there read as zero
+            int pitch = w, size = h * w, s = row, y0 = 0, x0 = 0, low = 0, high = h, left = 0, right = w;
+            if (WIN && p.win) {
+                const int nt = p.nty * p.ntx;
+                s = row / nt;
+                const int t = row - s * nt, ty = t / p.ntx, tx = t - ty * p.ntx;
+                pitch = p.W; size = p.H * p.W;
+                y0 = ty * p.step_y + p.oy; x0 = tx * p.step_x + p.ox;
+                low = max(0, -y0); high = min(h, p.H - y0);
+                left = max(0, -x0); right = min(w, p.W - x0);
+            }
+            const float* planes = p.real_in + ((size_t)s * p.C + c0) * (size_t)size;
+            const bool plane = gA < p.C - c0 && high > low;
+            const bool live = plane && cA >= left && cA < right, live2 = plane && cA + 1 >= left && cA + 1 < right;
+            const float* s0 = planes + (plane ? gA * size + y0 * pitch + x0 + cA : 0);
+            const int rows = live ? high - low : 0, rows2 = live2 ? high - low : 0;
             ulonglong2* dst = sMid + gA * PP + (cA >> 1);
             auto release = [&]() __attribute__((always_inline)) {  // the previous item's store has read the buffer
                 if (tid == 0) fk_bulk_wait_read();
                 __syncthreads();
             };
-            if (((w & 1) | ((int)(reinterpret_cast<uintptr_t>(planes) >> 2) & 1)) == 0)
-                split_class<N>(cls, SplitLoad<true>{s0, 4 * w, rows, rows2}, dst, release);
+            // pairs that start at multiples of 8 bytes are inside or outside as a whole
+            if (((w | pitch | x0 | (int)(reinterpret_cast<uintptr_t>(planes) >> 2)) & 1) == 0)
+                split_class<N>(cls, SplitLoad<true, WIN>{s0, 4 * pitch, rows, rows2, low}, dst, release);
             else
-                split_class<N>(cls, SplitLoad<false>{s0, 4 * w, rows, rows2}, dst, release);
+                split_class<N>(cls, SplitLoad<false, WIN>{s0, 4 * pitch, rows, rows2, low}, dst, release);
         }
         __syncthreads();
 
@@ -362,11 +379,11 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
     if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// At n = 64 the plain kernel, whose tiles are 4 planes, is the better one where no tile is more than half full: 300 rows of
+// At n = 64 (without windows) the plain kernel, whose tiles are 4 planes, is the better one where no tile is more than half full: 300 rows of
 // 4 planes 20.9 -> 18.8 us (25 x 25), of 6 planes 18.8 against 26.9.
 static inline bool split_pays(int n, const FftParams& pa, const FftParams* pb) {
-    if (n != 64 || pa.win || (pb && pb->win)) return false;
-    return 2 * pa.C > SplitGeom<64>::G || (pb && 2 * pb->C > SplitGeom<64>::G);
+    if (n != 64) return false;
+    return pa.win || (pb && pb->win) || 2 * pa.C > SplitGeom<64>::G || (pb && 2 * pb->C > SplitGeom<64>::G);
 }
 
 // Forward transform of one operand, or of two in one launch (pb may be null).
@@ -386,9 +403,12 @@ static cudaError_t launch_r2c_split(FftParams pa, const FftParams* pb_in, cudaSt
     const long long items = (long long)Gm::CLASSES * ((long long)pa.num_tiles + pb.num_tiles);
     if (items > 0x3fffffffLL) return cudaErrorInvalidValue;
     int grid = 0;
-    const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(r2c_split_kernel<N>), Gm::T, Gm::SMEM, items, &grid);
+    // the windowed variant is an instantiation of its own, so that the plain one carries none of its tests
+    auto kern = N == 64 && (pa.win || pb.win) ? r2c_split_kernel<N, N == 64> : r2c_split_kernel<N, false>;
+    if (N != 64 && (pa.win || pb.win)) return cudaErrorInvalidValue;
+    const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(kern), Gm::T, Gm::SMEM, items, &grid);
     if (e != cudaSuccess) return e;
-    return dep_launch(false, r2c_split_kernel<N>, dim3(grid), dim3(Gm::T), Gm::SMEM, st, m[0], m[1], m[2], m[3], pa, pb);
+    return dep_launch(false, kern, dim3(grid), dim3(Gm::T), Gm::SMEM, st, m[0], m[1], m[2], m[3], pa, pb);
 }
 
 }  // namespace fc

@@ -17,6 +17,7 @@
 #include "fft_kernels.cuh"
 #include "fft_big.cuh"
 #include "fft_split.cuh"
+#include "fft_inv64.cuh"
 #include "fft_small.cuh"
 #include "fft1d.cuh"
 
@@ -397,8 +398,9 @@ int run_pass(conv_plan_s* plan, int pass, const float* a_in, const float* b_in, 
     // whose loads are whole 128-byte lines; everything else the butterfly kernels
     cudaError_t ie = plan->small_planes ? fc::launch_c2r_small(plan->n, ip, st) : cudaErrorNotSupported;
     if (ie == cudaErrorNotSupported)
-        ie = big ? fc::launch_c2r_big(ip, scratch, scratch_bytes, st)
-                 : fc::launch_c2r<true>(plan->n, ip, st);
+        ie = big                            ? fc::launch_c2r_big(ip, scratch, scratch_bytes, st)
+             : fc::inv64_pays(plan->n, ip) ? fc::launch_c2r_inv64(ip, st)
+                                            : fc::launch_c2r<true>(plan->n, ip, st);
     if (ie != cudaSuccess) return FFTCONV_ECUDA;
     mark(4);
     if (timing) plan->timed = true;

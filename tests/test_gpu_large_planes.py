@@ -6,21 +6,27 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-# (S, f, f', h, w, kh, kw, n), samples by which the tensors are shifted in memory
-@pytest.mark.parametrize("dims,shift", [
-    ((2, 9, 3, 128, 128, 5, 5, 128), 0),   # pairs of columns; every row and column in use
-    ((2, 9, 3, 128, 128, 5, 5, 128), 1),   # the same from an address that is no multiple of 8 bytes
-    ((1, 8, 10, 66, 127, 3, 4, 128), 0),   # odd rows, the last column has no partner; dy's rows are even
-    ((3, 1, 17, 127, 66, 2, 3, 128), 0),   # one plane in a tile, tiles of 8 + 8 + 1
-    ((1, 7, 8, 40, 101, 9, 3, 128), 2),    # fewer rows than half the basis
-    ((2, 3, 5, 97, 20, 97, 2, 128), 0),    # narrow planes, kernel as high as the plane
-    ((2, 9, 12, 64, 64, 14, 5, 64), 0),
-    ((2, 9, 12, 64, 64, 5, 14, 64), 1),
-    ((1, 8, 10, 33, 63, 3, 4, 64), 0),
-    ((3, 5, 17, 61, 20, 15, 3, 64), 3),    # narrow planes and filters too high for the small-plane kernel
-    ((2, 4, 3, 57, 58, 3, 3, 64), 0),      # no tile more than half full
+# (S, f, f', h, w, kh, kw, n), samples by which the tensors are shifted in memory, tile basis
+@pytest.mark.parametrize("dims,shift,tile", [
+    ((2, 9, 3, 128, 128, 5, 5, 128), 0, 0),   # pairs of columns; every row and column in use
+    ((2, 9, 3, 128, 128, 5, 5, 128), 1, 0),   # the same from an address that is no multiple of 8 bytes
+    ((1, 8, 10, 66, 127, 3, 4, 128), 0, 0),   # odd rows, the last column has no partner; dy's rows are even
+    ((3, 1, 17, 127, 66, 2, 3, 128), 0, 0),   # one plane in a tile, tiles of 8 + 8 + 1
+    ((1, 7, 8, 40, 101, 9, 3, 128), 2, 0),    # fewer rows than half the basis
+    ((2, 3, 5, 97, 20, 97, 2, 128), 0, 0),    # narrow planes, kernel as high as the plane
+    ((2, 9, 12, 64, 64, 14, 5, 64), 0, 0),
+    ((2, 9, 12, 64, 64, 5, 14, 64), 1, 0),
+    ((1, 8, 10, 33, 63, 3, 4, 64), 0, 0),
+    ((3, 5, 17, 61, 20, 15, 3, 64), 3, 0),    # narrow planes and filters too high for the small-plane kernel
+    ((2, 4, 3, 57, 58, 3, 3, 64), 0, 0),      # no tile more than half full
+    ((19, 33, 30, 64, 63, 14, 2, 64), 0, 0),  # more tiles of 4 planes than SMs, the last of a row not full
+    ((19, 30, 33, 57, 64, 2, 13, 64), 1, 0),
+    ((2, 9, 6, 128, 128, 5, 7, 128), 0, 64),  # windows of 64 x 64: pairs inside or outside as a whole,
+    ((2, 9, 6, 128, 128, 7, 6, 128), 1, 64),  # odd origins and addresses,
+    ((9, 17, 18, 100, 128, 5, 7, 128), 0, 64),
+    ((1, 3, 9, 97, 125, 13, 2, 128), 0, 64),  # odd planes, windows that hang over the edge
 ])
-def test_passes_against_oracle(dims, shift):
+def test_passes_against_oracle(dims, shift, tile):
     import torch
     import oracle
     import paper_1412_7580_b200 as fc
@@ -37,6 +43,7 @@ def test_passes_against_oracle(dims, shift):
     xd, wd, dyd = (shifted(a) for a in host)
     p = fc.conv_plan(*s.args())
     fc.conv_plan_set_math(p, fc.binding.MATH_FP32)
+    fc.conv_plan_set_tiling(p, tile)
     fc.conv_plan_alloc_workspace(p)
     y, dx, dw = (shifted(np.full(shape, np.nan, np.float32)) for shape in
                  ((s.S, s.fp, s.oh, s.ow), x.shape, w.shape))
@@ -45,8 +52,8 @@ def test_passes_against_oracle(dims, shift):
     fc.conv_accgrad(p, dyd, xd, dw)
     torch.cuda.synchronize()
     assert fc.conv_plan_status(p) == 0
-    # FP32 end to end: 2 x 14 butterfly stages and sums of at most 17 terms round at 2^-24 each; 1e-5 of the
-    # largest result is several times their worst case
+    # FP32 end to end: 2 x 14 butterfly stages and sums of at most 4 x 54 products (9 planes x 6 windows), each rounded at
+    # 2^-24 of its value, signs at random: 2^-24 (28 + sqrt(216)) = 2.5e-6 of the largest result; four times that
     for got, ref in ((y, oracle.fprop(x, w)), (dx, oracle.bprop(dy, w, s.h, s.w)), (dw, oracle.accgrad(dy, x, s.kh, s.kw))):
         g = got.cpu().numpy().astype(np.float64)
         assert np.max(np.abs(g - ref)) <= 1e-5 * np.max(np.abs(ref))
