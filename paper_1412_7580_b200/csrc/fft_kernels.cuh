@@ -269,7 +269,7 @@ __device__ __forceinline__ void load_split_narrow(Load&& load, int live, float (
 template <int N, int G, int LAYOUT, bool ALIAS, bool SALIAS, int MINB, bool WIN = false>
 __global__ void __launch_bounds__(N* G, MINB)
 r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUtensorMap tmS1,
-           const FftParams p0, const FftParams p1) {
+           const __grid_constant__ FftParams p0, const __grid_constant__ FftParams p1) {
     // Two operands can share one launch (both forward transforms of a pass): tiles
     // [0, p0.num_tiles) belong to the first, the rest to the second.
     constexpr int T = N * G, NC = N / 2 + 1, M = N / 2, HALF = T / 2, B = N * NC;
@@ -316,7 +316,7 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
         opC = second ? p1.C : p0.C;
         tpr = second ? p1.tiles_per_row : p0.tiles_per_row;
         hw = h * w;
-        split4 = (4 * w <= N);
+        split4 = (4 * w <= N) && !(WIN && (second ? p1.win : p0.win));
         narrow = (2 * w <= N);
         step_rows = gridDim.x / tpr; step_cols = gridDim.x - step_rows * tpr;
     };
@@ -351,7 +351,27 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
 
     // Stage the planes of a tile.  Returns true if the copy is asynchronous (wait on the
     // barrier before reading), false if it was done with plain loads by all threads.
-    bool win_pending = false;       // windowed tile on its way in through cp.async
+    // Window of a larger plane: clipped loads (Section 5.1) of the column that this thread transforms, straight into
+    // registers, where they wait while the rows of the tile before are transformed.  The loads are volatile: they are
+    // issued together, where they stand.  (B200, 16 x 256 planes of 128 x 128, 3 x 3 kernels, 16 x 16 windows: x 224 ->
+    // 170 us, dy of bprop 276 -> 195, both operands of accGrad 429 -> 299 against 4-byte asynchronous copies through
+    // shared memory, which cost an access more per sample and a wait and a barrier more per tile.)
+    float nv[WIN ? N : 1];
+    auto fetch_window = [&](const FftParams& pw, int row, int tcol) __attribute__((always_inline)) {
+        const int nt = pw.nty * pw.ntx;
+        const int s = row / nt, t = row - s * nt;
+        const int ty = t / pw.ntx, tx = t - ty * pw.ntx;
+        const int y0 = ty * pw.step_y + pw.oy, xx = tx * pw.step_x + pw.ox + cA;
+        const int low = max(0, -y0);
+        const int rows = gA < pw.C - tcol * G && cA < pw.w && xx >= 0 && xx < pw.W ? max(0, min(pw.h, pw.H - y0) - low) : 0;
+        const float* src = pw.real_in + ((size_t)s * pw.C + tcol * G + gA) * ((size_t)pw.H * pw.W) + (long long)y0 * pw.W + xx;
+        const int pitch = 4 * pw.W;
+        static_for<N>([&](auto Rr) __attribute__((always_inline)) {
+            constexpr int r = decltype(Rr)::value;
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1];\n\t}"
+                         : "=f"(nv[r]) : "l"(reinterpret_cast<const char*>(src) + (long long)pitch * r), "r"(r - low), "r"(rows));
+        });
+    };
     int off = 0, off_n = 0;         // first sample of the tile in sIn: this tile, the one on its way
     auto stage = [&](bool second, int row, int tcol) -> bool {
         const int sh = second ? p1.h : p0.h, sw = second ? p1.w : p0.w;
@@ -359,43 +379,11 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
         const float* base = second ? p1.real_in : p0.real_in;
         const int c0 = tcol * G;
         const int gcount = min(G, sC - c0);
-        if (WIN && (second ? p1.win : p0.win)) {
-            // window of a larger plane: clipped loads (Section 5.1), one plane row per N lanes
-            const FftParams& pw = second ? p1 : p0;
-            const int nt = pw.nty * pw.ntx;
-            const int s = row / nt, t = row - s * nt;
-            const int ty = t / pw.ntx, tx = t - ty * pw.ntx;
-            const int y0 = ty * pw.step_y + pw.oy, x0 = tx * pw.step_x + pw.ox;
-            const int rr = tid / N, cc = tid - rr * N;
-            const int xx = x0 + cc;
-            const bool col_ok = (cc < sw) && xx >= 0 && xx < pw.W;
-            // 4-byte asynchronous copies; a sample outside the plane is a copy of zero bytes,
-            // which writes a zero.  Completion: every thread waits for its own copies, then a
-            // barrier (win_pending, at the top of the tile loop).  The row test and the address
-            // are formed once per row sweep; the planes of the tile only advance pointers.
-            if (cc < sw) {
-                const int r_lo = max(0, -y0), r_hi = min(sh, pw.H - y0);    // window rows inside the plane
-                const size_t plane = (size_t)pw.H * pw.W;
-                const float* pl0 = base + ((size_t)s * sC + c0) * plane;
-                const long long off0 = (long long)y0 * pw.W + xx;
-                const uint32_t tile_stride = 4u * (uint32_t)(sh * sw);
-                const uint32_t dst0 = fk_smem_u32(sIn + cc);
-                for (int r = rr; r < sh; r += G) {
-                    const bool ok = col_ok && r >= r_lo && r < r_hi;
-                    const float* src = ok ? pl0 + (off0 + (long long)r * pw.W) : pl0;
-                    const size_t step = ok ? plane : 0;
-                    const int nbytes = ok ? 4 : 0;
-                    uint32_t dstp = dst0 + 4u * (uint32_t)(r * sw);
-                    for (int g = 0; g < gcount; ++g) {
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
-                                     ::"r"(dstp), "l"(src), "r"(nbytes) : "memory");
-                        dstp += tile_stride;
-                        src += step;
-                    }
-                }
+        if constexpr (WIN) {
+            if (second ? p1.win : p0.win) {
+                fetch_window(second ? p1 : p0, row, tcol);
+                return false;
             }
-            win_pending = true;
-            return false;
         }
         const float* src = base + ((size_t)row * sC + c0) * (sh * sw);
         // One bulk copy of the 16-byte units inside the tile, up to three samples before and
@@ -408,7 +396,7 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
         if (WIN && mis != 0) {
             // The windowed kernel loads the odd filter tile by the threads: with the misalignment
             // kept per tile its windows took longer (16 x 256 planes of 128 x 128, 3 x 3 kernels:
-            // a step 2125 us without, 2149 us with).
+            // a step 2125 us without, 2149 us with, when the windows still passed through shared memory).
             for (int i = tid; i < total; i += T) sIn[i] = __ldg(src + i);
             return false;
         }
@@ -465,12 +453,6 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
             }
             phase ^= 1u;
         }
-        if (WIN && win_pending) {
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            __syncthreads();
-            win_pending = false;
-        }
-
         // 2. column transforms.  Wide planes: thread = (plane gA, column cA), cA < w, one real
         //    FFT of length N each.  Narrow planes (filters): four threads per column, thread
         //    q4 computing the outputs ky = 4k + q4 through one radix-4 decimation-in-frequency
@@ -485,6 +467,9 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
                 if (act) {
                     float v[N];
                     const float* src = sIn + off + gA * hw + cA;
+                    if (WIN && p.win) {
+                        static_for<N>([&](auto Rr) { v[decltype(Rr)::value] = nv[WIN ? decltype(Rr)::value : 0]; });
+                    } else
                     // Zero-padding below the plane.  Rows r < N/2 exist whenever h > N/2 (the
                     // usual case: N is the next power of two), so they are plain loads; the
                     // others are loaded unconditionally (clamped) and zeroed by a select --
@@ -970,17 +955,21 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
             const float scale = p.scale;
             if (WIN && p.win) {
                 // rows [oy, oy + win_hc) of the transform go to the tile's place in the plane
-                dst = p.real_out + win_base + (cA - p.ox);
                 const bool acc = p.accumulate != 0;
-                const int r0 = p.oy, r1 = p.oy + win_hc, pitch = p.W;
+                const int r0 = p.oy, pitch = p.W;
+                dst = p.real_out + win_base + (cA - p.ox) - (long long)r0 * pitch;
                 static_for<N>([&](auto Rr) {
                     constexpr int r = decltype(Rr)::value;
-                    if (r >= r0 && r < r1) {
-                        float o = v[r] * scale;
-                        if (acc) o += *dst;
-                        *dst = o;
-                        dst += pitch;
+                    if (!acc) {
+                        asm volatile(
+                            "{\n\t.reg .pred p;\n\t"
+                            "setp.lt.u32 p, %2, %3;\n\t"
+                            "@p st.global.f32 [%0], %1;\n\t}"
+                            ::"l"(dst), "f"(v[r] * scale), "r"(r - r0), "r"(win_hc) : "memory");
+                    } else if ((unsigned)(r - r0) < (unsigned)win_hc) {
+                        *dst += v[r] * scale;
                     }
+                    dst += pitch;
                 });
             } else if (!ACC && !p.accumulate && 2 * hc > N) {
                 static_for<N>([&](auto Rr) {
@@ -1134,11 +1123,11 @@ static cudaError_t launch_r2c_layout(FftParams pa, const FftParams* pb_in, cudaS
     constexpr int G = Cfg::G;
     FftParams pb{};
     if (!fill_tiling<G>(pa)) return cudaErrorInvalidValue;
-    int in_bytes = real_tile_bytes(G, pa.real_in, pa.h, pa.w);
+    int in_bytes = pa.win ? 0 : real_tile_bytes(G, pa.real_in, pa.h, pa.w);     // (windows go straight to registers)
     if (pb_in) {
         pb = *pb_in;
         if (!fill_tiling<G>(pb)) return cudaErrorInvalidValue;
-        const int b = real_tile_bytes(G, pb.real_in, pb.h, pb.w);
+        const int b = pb.win ? 0 : real_tile_bytes(G, pb.real_in, pb.h, pb.w);
         if (b > in_bytes) in_bytes = b;
     }
     pa.in_bytes = pb.in_bytes = in_bytes;
