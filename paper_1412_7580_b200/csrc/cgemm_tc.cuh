@@ -13,7 +13,7 @@
 // the minus sign coming from the instruction descriptor's negate-A bit, so no
 // expanded or interleaved copy of an operand is ever built.
 //
-// One persistent CTA per SM, warp-specialised:
+// One persistent CTA per SM (up to four for narrow matrices), warp-specialised:
 //   warp 0      TMA producer: 128-byte-swizzled boxes of 32 k-values x 128 rows
 //               of A_re, A_im, B_re, B_im per stage (64 KB), 3 stages in flight;
 //   warp 1      issues tcgen05.mma (one lane), owns the TMEM allocation;
@@ -27,7 +27,8 @@
 // than a tile are fetched and multiplied only as far as they go (rows of the
 // boxes, N of the instructions, k-steps), which also makes room for a fourth stage:
 // M, N, K = 50, 90, 67 over the bins of n = 32 22.0 -> 18.5 us, 24, 100, 200 (n = 64)
-// 96 -> 83 us, 100, 10, 200 (n = 64) 88-120 -> 75-95 us; full tiles unchanged.
+// 96 -> 83 us, 100, 10, 200 (n = 64) 88-120 -> 75-95 us; full tiles unchanged.  Narrow ones (N <= 64) share an SM among
+// two to four CTAs, where their loads, MMAs and stores fit (see the launcher).
 //
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises the
 // caller's status word, drains what it issued, frees its tensor memory and
@@ -57,11 +58,9 @@ constexpr uint32_t TC_EPI_BYTES = 4 * 2 * TC_EPI_BUF_BYTES;      // 4 warps x 2 
 // n = 64: 62 us with three, 59 with four, 65 with six).
 constexpr int TC_MAX_STAGES = 4;
 constexpr uint32_t tc_smem_bytes(int stages) { return 1024 + stages * TC_STAGE_BYTES + TC_EPI_BYTES + 512; }
-constexpr uint32_t TC_SMEM_BYTES = tc_smem_bytes(TC_STAGES);
 // A launch that shares the SMs with a transform kernel (the filter spectrum produced range by range
 // beside the contraction) runs a ring of two stages and leaves 64 KB of shared memory to that kernel.
 constexpr int TC_STAGES_SHARED = 2;
-constexpr uint32_t TC_TMEM_COLS = 512;
 constexpr long long TC_WAIT_CYCLES = 2000000000LL;               // about one second
 
 struct TcParams {
@@ -80,6 +79,8 @@ struct TcParams {
     int rows_a, rows_b;         // K-major: rows of a TMA box; MN-major: a multiple of 32, one box each
     int mma_n;                  // N of the instructions (multiple of 16)
     int stages;                 // stages of the ring: as many as its shared memory holds, at most TC_MAX_STAGES
+    uint32_t ring_bytes, epi_bytes;     // shared memory of the ring and of the epilogue's staging tiles
+    uint32_t acc_cols;          // TMEM columns from one accumulator to the next: 128, or 64 or 32 where N allows
 };
 
 static inline bool tc_shape_supported(int M, int N, int K) {
@@ -217,9 +218,11 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     extern __shared__ uint8_t tc_raw[];
     const uint32_t raw_addr = smem_u32(tc_raw);
     const uint32_t tiles = (raw_addr + 1023u) & ~1023u;             // stage buffers, 1024-aligned
-    const uint32_t epi = tiles + ST * TC_STAGE_BYTES;        // epilogue staging, 1024-aligned
-    uint8_t* ctl = tc_raw + (tiles - raw_addr) + ST * TC_STAGE_BYTES + TC_EPI_BYTES;
-    const uint32_t bars = epi + TC_EPI_BYTES;
+    const uint32_t ring_bytes = FULL ? ST * TC_STAGE_BYTES : p.ring_bytes, epi_bytes = FULL ? TC_EPI_BYTES : p.epi_bytes;
+    const uint32_t acc_cols = FULL ? (uint32_t)TC_BN : p.acc_cols, tmem_cols = 4u * acc_cols;
+    const uint32_t epi = tiles + ring_bytes;                 // epilogue staging, 1024-aligned
+    uint8_t* ctl = tc_raw + (tiles - raw_addr) + ring_bytes + epi_bytes;
+    const uint32_t bars = epi + epi_bytes;
     // barrier slots (8 bytes each): full[4] empty[4] tfull[2] tempty[2] drain
     auto full = [&](int s) { return bars + 8u * s; };
     auto empty = [&](int s) { return bars + 8u * (TC_MAX_STAGES + s); };
@@ -245,7 +248,7 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(tmem_slot)), "r"(TC_TMEM_COLS) : "memory");
+                     ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before_sync();
@@ -338,8 +341,8 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int buf = tl & 1;
                 if (!mbar_wait(tempty(buf), ((uint32_t)(tl >> 1) & 1u) ^ 1u, abort_flag, p.wait_cycles)) { ok = false; break; }
                 tc_fence_after_sync();
-                const uint32_t d_re = tmem_base + (uint32_t)buf * 256u;
-                const uint32_t d_im = d_re + 128u;
+                const uint32_t d_re = tmem_base + (uint32_t)buf * 2u * acc_cols;
+                const uint32_t d_im = d_re + acc_cols;
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
                     if (!mbar_wait(full(s), ph, abort_flag, p.wait_cycles)) { ok = false; break; }
                     tc_fence_after_sync();
@@ -391,7 +394,7 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             tc_fence_after_sync();
             const int row0 = m_t * TC_BM + q * 32;
             const int col0 = n_t * TC_BN;
-            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * 256u;
+            const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * 2u * acc_cols;
             if (row0 < p.M) {                                           // warp-uniform
 #pragma unroll 1
                 for (int part = 0; part < 2; ++part) {
@@ -399,7 +402,7 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     for (int c = 0; c < TC_BN; c += 32) {
                         if (col0 + c >= p.N) break;                     // warp-uniform
                         uint32_t v[32];
-                        tc_ld32(t_row + (uint32_t)(part * 128 + c), v);
+                        tc_ld32(t_row + (uint32_t)part * acc_cols + (uint32_t)c, v);
                         // the staging buffer used two stores ago must have been read out
                         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                         __syncwarp();
@@ -436,7 +439,7 @@ cgemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     tc_fence_after_sync();
     if (warp == 1) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                     ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
+                     ::"r"(tmem_base), "r"(tmem_cols) : "memory");
     }
 }
 
@@ -462,8 +465,36 @@ static cudaError_t launch_cgemm_tc_f(const GemmParams& g, int* status, cudaStrea
     p.rows_a = cover(g.M, TA ? 32 : 8, TC_BM);
     p.rows_b = cover(g.N, TB ? 32 : 16, TC_BN);
     p.mma_n = cover(g.N, 16, TC_BN);
-    const int fit = (int)(ST * TC_STAGE_BYTES / (256u * (uint32_t)(p.rows_a + p.rows_b)));
+    // CTAs per SM.  The tiles of narrow matrices are short chains of a load, a few MMAs and a store, which one CTA's ring
+    // and two accumulators do not hide.  Where the accumulators leave tensor memory for more CTAs (N <= 64: two, N <= 32:
+    // four) as many run as find two stages of the ring in shared memory (not beside a transform kernel, which needs the
+    // space).  M, N, K = 55, 12, 15 over the bins of n = 64 18.7 -> 12.8 us, 18, 6, 33 21.0 -> 12.9, 19, 34, 4 22.8 -> 16.0,
+    // n = 128: 9, 18, 20 55.6 -> 27, 40, 20, 60 88 -> 58-67, 96, 3, 128 158 -> 132-140; 300, 20, 20 (n = 64) unchanged.
+    const uint32_t stage = 256u * (uint32_t)(p.rows_a + p.rows_b);
+    int per_sm = 1;
+    p.acc_cols = TC_BN;
+    p.epi_bytes = TC_EPI_BYTES;
+    uint32_t ring = ST * TC_STAGE_BYTES;
+    if (!FULL && ST == TC_STAGES && g.N <= 64) {
+        // the staging tiles of the warps that have rows; at least 16 KB, because an MMA reads 128 rows of A whatever rows_a
+        // is, and what lies behind the last stage's has to be shared memory of this CTA
+        const uint32_t warps = (uint32_t)((p.rows_a + 31) / 32), epi = (warps < 2 ? 2 : warps) * 2 * TC_EPI_BUF_BYTES;
+        constexpr uint32_t SM_BYTES = 227 * 1024, RESERVED = 1024;      // per SM; per CTA, by the system
+        for (int c = g.N <= 32 ? 4 : 2; c > 1; --c) {
+            const uint32_t room = SM_BYTES / c / 1024 * 1024 - RESERVED, fixed = tc_smem_bytes(0) - TC_EPI_BYTES + epi;
+            if (room < fixed + 2 * stage) continue;
+            per_sm = c;
+            p.acc_cols = g.N <= 32 ? 32 : 64;
+            p.epi_bytes = epi;
+            ring = (room - fixed) / 1024 * 1024;
+            break;
+        }
+    }
+    p.ring_bytes = ring;
+    const int fit = (int)(ring / stage);
     p.stages = fit < TC_MAX_STAGES ? fit : TC_MAX_STAGES;
+    if (per_sm > 1) p.ring_bytes = (uint32_t)p.stages * stage;
+    const size_t smem = tc_smem_bytes(0) - TC_EPI_BYTES + p.epi_bytes + p.ring_bytes;
     const bool okA = TA ? tc_make_map(&tmA, g.A, g.bins, g.K, g.M, g.lda, 32, TC_BK,
                                       CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)
                         : tc_make_map(&tmA, g.A, g.bins, g.M, g.K, g.lda, TC_BK, p.rows_a);
@@ -494,8 +525,9 @@ static cudaError_t launch_cgemm_tc_f(const GemmParams& g, int* status, cudaStrea
     }
     const long long tiles = (long long)p.bins_run * p.m_tiles * p.n_tiles;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const int grid = (int)(tiles < sm_count ? tiles : sm_count);
-    return dep_launch(g.overlap != 0, kern, dim3(grid), dim3(TC_THREADS), tc_smem_bytes(ST), st, tmA, tmB, tmC, p);
+    const long long slots = (long long)sm_count * per_sm;
+    const int grid = (int)(tiles < slots ? tiles : slots);
+    return dep_launch(g.overlap != 0, kern, dim3(grid), dim3(TC_THREADS), smem, st, tmA, tmB, tmC, p);
 }
 
 template <bool TA, bool TB, int ST>

@@ -116,3 +116,12 @@ def test_tf32_tiles_used_in_part(shape, flags):
 def test_the_arithmetic_asked_for_is_the_one_that_runs(shape, flags):
     assert run(*shape, math=1, seed=17, **flags) <= 1.2e-5
     assert 2e-5 <= run(*shape, math=2, seed=17, **flags) <= TOL[2]
+
+
+# narrow matrices run several CTAs per SM (N <= 32: up to four, N <= 64: two), as many as find shared memory for their
+# rows: both lines, rows that fill one to four staging tiles, one and several k-blocks, more tiles than all CTAs
+@pytest.mark.parametrize("flags", FLAGS[:3])
+@pytest.mark.parametrize("shape", [(1300, 8, 16, 4), (1300, 16, 8, 33), (700, 55, 12, 15), (700, 97, 32, 40), (700, 128, 33, 33),
+                                   (400, 130, 64, 16), (400, 64, 65, 8), (650, 121, 5, 130), (1300, 1, 130, 3)])
+def test_tf32_several_ctas_per_sm(shape, flags):
+    assert run(*shape, math=2, seed=19, **flags) <= TOL[2]
