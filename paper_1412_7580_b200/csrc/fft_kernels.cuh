@@ -369,7 +369,7 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
         static_for<N>([&](auto Rr) __attribute__((always_inline)) {
             constexpr int r = decltype(Rr)::value;
             asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1];\n\t}"
-                         : "=f"(nv[r]) : "l"(reinterpret_cast<const char*>(src) + (long long)pitch * r), "r"(r - low), "r"(rows));
+                         : "=&f"(nv[r]) : "l"(reinterpret_cast<const char*>(src) + (long long)pitch * r), "r"(r - low), "r"(rows));
         });
     };
     int off = 0, off_n = 0;         // first sample of the tile in sIn: this tile, the one on its way

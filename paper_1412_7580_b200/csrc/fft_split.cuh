@@ -76,7 +76,8 @@ __device__ __forceinline__ void fk_tma_store_5d(const CUtensorMap* map, uint32_t
 // The samples of two adjacent columns, row by row: one 8-byte load where the pair is so aligned, two of 4
 // bytes else; rows and columns past the plane are zeros.  The loads are volatile, so that they are issued in
 // program order, well ahead of their use (split_column): left to itself the compiler puts each load right
-// before its use and a thread has a few in flight.
+// before its use and a thread has a few in flight.  The output is written before the address is read
+// (early-clobber constraint).
 // LOW (windows): the rows below `low` do not exist either.
 template <bool PAIR, bool LOW>
 struct SplitLoad {
@@ -91,14 +92,14 @@ struct SplitLoad {
         if constexpr (PAIR) {
             F2 v;
             asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.u32 p, %2, %3;\n\tmov.b64 %0, 0;\n\t@p ld.global.nc.b64 %0, [%1];\n\t}"
-                         : "=l"(v.b) : "l"(q), "r"(rows), "r"(at));
+                         : "=&l"(v.b) : "l"(q), "r"(rows), "r"(at));
             return v;
         } else {
             float u, v;
             asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.u32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1];\n\t}"
-                         : "=f"(u) : "l"(q), "r"(rows), "r"(at));
+                         : "=&f"(u) : "l"(q), "r"(rows), "r"(at));
             asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.u32 p, %2, %3;\n\tmov.b32 %0, 0;\n\t@p ld.global.nc.b32 %0, [%1+4];\n\t}"
-                         : "=f"(v) : "l"(q), "r"(rows2), "r"(at));
+                         : "=&f"(v) : "l"(q), "r"(rows2), "r"(at));
             return f2_pack(u, v);
         }
     }

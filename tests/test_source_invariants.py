@@ -84,3 +84,18 @@ def test_no_wait_runs_out_in_silence():
             code = re.sub(r"//[^\n]*", "", text)
             assert "status" not in code and "mbar" not in code
     assert bare == 1
+
+
+def test_outputs_written_before_the_last_input_is_read_are_early_clobbers():
+    """A predicated load that zeroes its destination first (mov, then @p ld from an address operand) may only have an
+    output that shares no register with the address: "=&"."""
+    checked = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = open(os.path.join(CSRC, name)).read()
+        for m in re.finditer(r'asm volatile\("([^;]|;(?!\s*$))*?;\s*$', text, re.M):
+            stmt = m.group(0)
+            first = re.search(r"mov\.b(?:32|64) %0, 0;", stmt)
+            if first and re.search(r"ld\.[a-z.]+b?\d+ %0, \[%[1-9]", stmt[first.end():]):
+                assert re.search(r':\s*"=&[a-z]"', stmt), f"{name}: {stmt}"
+                checked += 1
+    assert checked >= 4
