@@ -314,9 +314,9 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
             const int rg = warp >> 1;
             const ulonglong2* rp = rowp + rg * 4 * RP;
             float* o = sStage + (size_t)((rg >> 1) * 2 * N) * (8 * G) + (rg & 1) * 32 + lane;
-            auto half = [&](auto Q) __attribute__((always_inline)) {
+            F2 zr[16], zi[16];
+            auto load = [&](auto Q) __attribute__((always_inline)) {
                 constexpr int q = decltype(Q)::value;
-                F2 zr[16], zi[16];
                 static_for<16>([&](auto J) __attribute__((always_inline)) {
                     constexpr int j = decltype(J)::value;
                     const ulonglong2 a = rp[j], b = rp[j + 16];
@@ -335,18 +335,24 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
                         }
                     }
                 });
-                __syncthreads();                            // the rows are in registers: the buffer becomes the staging tile
-                cfft<16, false>(zr, zi);                    // E, O at 2k + q
+            };
+            auto store = [&](auto Q) __attribute__((always_inline)) {
                 static_for<16>([&](auto K) __attribute__((always_inline)) {
-                    constexpr int k = decltype(K)::value, kx = 2 * k + q;
+                    constexpr int k = decltype(K)::value, kx = 2 * k + decltype(Q)::value;
                     float ar, ai, br, bi;
                     split_last(zr[k], zi[k], Tw<64, kx>::c, Tw<64, kx>::s, ar, ai, br, bi);
                     o[kx * (8 * G)] = ar;        o[(N + kx) * (8 * G)] = ai;
                     o[(M + kx) * (8 * G)] = br;  o[(N + M + kx) * (8 * G)] = bi;
                 });
             };
-            if ((warp & 1) == 0) half(std::integral_constant<int, 0>{});
-            else                 half(std::integral_constant<int, 1>{});
+            constexpr std::integral_constant<int, 0> even{};
+            constexpr std::integral_constant<int, 1> odd{};
+            if ((warp & 1) == 0) load(even);
+            else                 load(odd);
+            __syncthreads();                                // the rows are in registers: the buffer becomes the staging tile
+            cfft<16, false>(zr, zi);                        // E, O at 2k + q
+            if ((warp & 1) == 0) store(even);
+            else                 store(odd);
         }
         if (cls == 0) {
             // row ky = 0 of every plane holds Z = FFT(X_0 + i X_{N/2}):

@@ -99,3 +99,29 @@ def test_outputs_written_before_the_last_input_is_read_are_early_clobbers():
                 assert re.search(r':\s*"=&[a-z]"', stmt), f"{name}: {stmt}"
                 checked += 1
     assert checked >= 4
+
+
+def lambdas_of(text):
+    """(name, body) of every named lambda."""
+    for m in re.finditer(r"\bauto\s+(\w+)\s*=\s*\[&\][^{;]*\{", text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[i], 0)
+            i += 1
+        yield m.group(1), text[m.end():i]
+
+
+def test_no_block_barrier_under_a_condition_that_differs_between_warps():
+    """__syncthreads() is defined only where the whole block takes the same path to it; a step that some warps run in
+    another form than the others has to meet at a barrier outside the branch (or at a numbered one)."""
+    branches = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        bodies = {}
+        for lam, body in lambdas_of(text):
+            bodies.setdefault(lam, []).append(body)
+        for m in re.finditer(r"if \(\(?(?:warp|lane|tid|team|q4?)\b[^)]*\)?[^)]*\)\s*(\w+)\(", text):
+            for body in bodies.get(m.group(1), []):
+                branches += 1
+                assert "__syncthreads" not in body, f"{name}: {m.group(0)}...) reaches a block barrier"
+    assert branches >= 6
