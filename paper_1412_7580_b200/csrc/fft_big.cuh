@@ -203,7 +203,8 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
     constexpr int N = Gm::N, M = Gm::M, G = Gm::G, RP = Gm::RP, PP = Gm::PP, RING = Gm::RING, PITCH = Gm::HI * G;
     extern __shared__ __align__(128) unsigned char fc_smem[];
     __shared__ __align__(8) unsigned long long bars[RING + 1];
-    __shared__ volatile int dead;           // a load never landed: the barriers are still walked, nothing is waited for
+    __shared__ volatile int dead;           // a load never landed: the tile is walked to its end, nothing more is stored
+    __shared__ int asked, asked_ny;         // boxes and rows n/2 requested so far (written by thread 0)
     const float* sNy = reinterpret_cast<const float*>(fc_smem + RING * Gm::BUF);
     const uint32_t bar_ny = fk_smem_u32(&bars[RING]);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -221,7 +222,7 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
     dep_trigger();
     if (tid == 0) {
         for (int s = 0; s <= RING; ++s) fk_mbar_init(fk_smem_u32(&bars[s]), 1);
-        dead = 0;
+        dead = asked = asked_ny = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -238,12 +239,14 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
             fk_mbar_expect_tx(bar, (uint32_t)Gm::STAGE);
             fk_tma_load_5d_once(fk_smem_u32(fc_smem + (s + b) * Gm::BUF), &tmS, c0, row, b == 0 ? cls : (cls == 0 ? 8 : 16 - cls), 0, 0, bar);
         }
+        asked += 2;
     };
     auto request_ny = [&](int tile) {       // row n/2, which travels with row 0; one thread
         if (rank != 0 || tile >= p.num_tiles || dead) return;
         const int row = tile / tpr, c0 = (tile - row * tpr) * G;
         fk_mbar_expect_tx(bar_ny, (uint32_t)Gm::STAGE_NY);
         fk_tma_load_4d_once(fk_smem_u32(sNy), &tmNy, c0, row, M, 0, bar_ny);
+        ++asked_ny;
     };
     if (tid == 0) {
         request(0);
@@ -257,11 +260,12 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
 
     int i = 0;
     uint32_t ny_phase = 0;
+    bool gone = false;              // from then on only the cluster's barriers are walked
     for (int tile = group; tile < p.num_tiles; tile += groups) {
         const int row = tile / tpr, c0 = (tile - row * tpr) * G;
         const int gcount = min(G, p.C - c0);
 #pragma unroll 1
-        for (int k = 0; k < K; ++k, ++i) {
+        for (int k = 0; k < K && !gone; ++k, ++i) {
             const int cls = rank * K + k, s = 2 * i % RING;
             // ---- B: rows of one residue ----
             {
@@ -345,9 +349,10 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
         }
         if (rank == 0) ny_phase ^= 1u;
         big_tile_sync();                                    // the scratch is complete
+        gone = dead;
 
         // ---- C: last step of the columns, crop ----
-        if (gA < nj && mA < pairs) {
+        if (!gone && gA < nj && mA < pairs) {
             const int j = gA, m = mA;
             const ulonglong2* src = scratch + j * Gm::S_J + m;
 #pragma unroll 1
@@ -399,6 +404,10 @@ c2r_big_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant__ 
             }
         }
         big_tile_sync();                                    // the scratch may be rewritten
+    }
+    if (tid == 0 && dead) {
+        fk_ring_drain(fk_smem_u32(&bars[0]), RING, asked);
+        fk_ring_drain(bar_ny, 1, asked_ny);
     }
 }
 

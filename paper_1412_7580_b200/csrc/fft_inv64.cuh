@@ -55,7 +55,8 @@ c2r_inv64_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
     constexpr int N = Gm::N, M = Gm::M, G = Gm::G, RP = Gm::RP, PP = Gm::PP, RING = Gm::RING, PITCH = Gm::HI * G;
     extern __shared__ __align__(128) unsigned char fc_smem[];
     __shared__ __align__(8) unsigned long long bars[RING + 1];
-    __shared__ volatile int dead;           // a load never landed: the barriers are still walked, nothing is waited for
+    __shared__ volatile int dead;           // a load never landed: the tile is walked to its end, nothing more is stored
+    __shared__ int asked, asked_ny;         // boxes and rows n/2 requested so far (written by thread 0)
     const float* sNy = reinterpret_cast<const float*>(fc_smem + RING * Gm::BUF);
     const uint32_t bar_ny = fk_smem_u32(&bars[RING]);
     const int team = threadIdx.x / Gm::TEAM, tid = threadIdx.x - team * Gm::TEAM, warp = tid >> 5, lane = tid & 31;
@@ -67,7 +68,7 @@ c2r_inv64_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
     dep_trigger();
     if (threadIdx.x == 0) {
         for (int s = 0; s <= RING; ++s) fk_mbar_init(fk_smem_u32(&bars[s]), 1);
-        dead = 0;
+        dead = asked = asked_ny = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -81,6 +82,7 @@ c2r_inv64_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
         const uint32_t bar = fk_smem_u32(&bars[rq_s]);
         fk_mbar_expect_tx(bar, (uint32_t)Gm::STAGE);
         fk_tma_load_5d(fk_smem_u32(fc_smem + rq_s * Gm::BUF), &tmS, c0, row, rq_box, 0, 0, bar);
+        ++asked;
         if (++rq_s == RING) rq_s = 0;
         rq_box ^= 1;
         if (rq_box == 0) rq_tile += gridDim.x;
@@ -90,6 +92,7 @@ c2r_inv64_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
         const int row = tile / tpr, c0 = (tile - row * tpr) * G;
         fk_mbar_expect_tx(bar_ny, (uint32_t)Gm::STAGE_NY);
         fk_tma_load_4d(fk_smem_u32(sNy), &tmNy, c0, row, M, 0, bar_ny);
+        ++asked_ny;
     };
     if (threadIdx.x == 0) {
         request();
@@ -220,6 +223,7 @@ c2r_inv64_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
             if (team == 1) { u[i] = u[i + 8]; v[i] = v[i + 8]; }
         });
         __syncthreads();
+        const bool gone = dead;                             // (the waits of this tile are over, those of the next not begun)
         F2 e[8], f[8], tr[8], ti[8];
         static_for<8>([&](auto I) __attribute__((always_inline)) {
             constexpr int i = decltype(I)::value;
@@ -230,6 +234,7 @@ c2r_inv64_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
         });
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();                                    // the buffer may take another box
+        if (gone) break;
         if (threadIdx.x == 0) request();
         {
             // crop: rows [r0, r0 + hc) and columns [x0, x0 + wc) of the transform
@@ -274,6 +279,10 @@ c2r_inv64_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
             }
         }
         if ((s0 += 2) >= RING) { s0 -= RING; lap ^= 1u; }
+    }
+    if (threadIdx.x == 0 && dead) {
+        fk_ring_drain(fk_smem_u32(&bars[0]), RING, asked);
+        fk_ring_drain(bar_ny, 1, asked_ny);
     }
 }
 

@@ -47,6 +47,7 @@
 #include <mutex>
 
 #include "fft_core.cuh"
+#include "launch_rules.h"
 #include "tma_util.cuh"
 #include "dep_launch.cuh"
 
@@ -181,6 +182,14 @@ __device__ __forceinline__ void fk_bulk_g2s(uint32_t dst, const void* src, uint3
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
         ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+// After a give-up: a ring's boxes still in flight must land (or have had the default limit to) before the CTA's shared
+// memory is released.  One thread; `requested` boxes were asked for in order, and none after that.
+__device__ __forceinline__ void fk_ring_drain(uint32_t bars, int slots, long long requested) {
+    for (int s = 0; s < slots; ++s) {
+        const int uses = ring_uses(requested, s, slots);
+        if (uses > 0) (void)fk_mbar_wait(bars + 8u * (uint32_t)s, (uint32_t)(uses - 1) & 1u, FK_WAIT_CYCLES);
+    }
 }
 __device__ __forceinline__ void fk_bulk_s2g(void* dst, uint32_t src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"

@@ -353,6 +353,7 @@ c2r_small_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
 
     uint32_t phase = 0;             // bit s: phase of this warp's stage s
     bool ok = true;
+    int asked = 0;                  // set when a load never came: boxes requested until then
     float acc[K][K];
     long long blk = first;
     int i = 0, s = 0;
@@ -364,7 +365,10 @@ c2r_small_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
 #pragma unroll
                 for (int v = 0; v < K; ++v) acc[u][v] = 0.0f;
         }
-        if (ok && !fk_wait_or_report(bars + 8u * s, (phase >> s) & 1u, p.wait_cycles, p.status)) ok = false;
+        if (ok && !fk_wait_or_report(bars + 8u * s, (phase >> s) & 1u, p.wait_cycles, p.status)) {
+            ok = false;
+            asked = (int)min(items, j + NST);
+        }
         phase ^= (1u << s);
         if (ok) {
             if (ky == 0 || ky == N / 2) {
@@ -418,7 +422,7 @@ c2r_small_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
             }
         }
         __syncwarp();                                   // the row is consumed by every lane
-        if (j + NST < items) issue();
+        if (ok && j + NST < items) issue();
         if (++s == NST) s = 0;
         if (++i != my_rows) continue;
 
@@ -439,7 +443,10 @@ c2r_small_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
             // the four warps' accumulators are added in a fixed order
             if (!ok) failed = 1;
             __syncthreads();
-            if (failed) return;                         // a load never came: status raised, leave
+            if (failed) {                               // a load never came: status raised, leave when the others have
+                if (lane == 0) fk_ring_drain(bars, NST, ok ? min(items, j + 1 + NST) : asked);
+                return;
+            }
             for (int e = threadIdx.x; e < count * KSQ; e += SMALLINV_WARPS * 32) {
                 const int pl = e / KSQ, idx = e - pl * KSQ;
                 float sum = 0.0f;
@@ -451,7 +458,10 @@ c2r_small_kernel(const __grid_constant__ CUtensorMap tmS, const __grid_constant_
             }
             __syncthreads();                            // before the accumulators are written again
         } else {
-            if (!ok) return;
+            if (!ok) {
+                if (lane == 0) fk_ring_drain(bars, NST, asked);
+                return;
+            }
             __syncwarp();
             const float* mine = red + (size_t)warp * KSQ * 33;
             for (int e = lane; e < count * KSQ; e += 32) {

@@ -30,6 +30,7 @@ def _run(fc, torch, plan, s, xd, wd, dyd):
 @pytest.mark.parametrize("dims", [(8, 24, 40, 13, 13, 3, 3, 16),      # double-buffered inverse transform
                                   (4, 24, 40, 31, 31, 5, 5, 32),
                                   (2, 12, 10, 64, 64, 7, 7, 64),
+                                  (19, 33, 30, 64, 63, 14, 2, 64),    # more tiles than SMs: two teams per tile
                                   (1, 9, 10, 120, 120, 5, 5, 128)])   # transforms of large planes
 @pytest.mark.parametrize("math", [1, 2])
 def test_wait_limit_runs_out_and_the_plan_recovers(dims, math):

@@ -125,3 +125,22 @@ def test_no_block_barrier_under_a_condition_that_differs_between_warps():
                 branches += 1
                 assert "__syncthreads" not in body, f"{name}: {m.group(0)}...) reaches a block barrier"
     assert branches >= 6
+
+
+def test_kernels_with_a_ring_of_boxes_drain_it_when_they_give_up():
+    """A kernel that stops waiting after a load that never landed may have further boxes in flight; it must wait for
+    them before its shared memory is released, ask for no more, and store nothing formed without the data."""
+    def kernel(name, kern):
+        body = dict(kernels_of(open(os.path.join(CSRC, name)).read()))[kern]
+        return re.sub(r"//[^\n]*", "", body)
+    for name, kern in (("fft_inv64.cuh", "c2r_inv64_kernel"), ("fft_big.cuh", "c2r_big_kernel")):
+        body = kernel(name, kern)
+        tail = body[body.rindex("if ("):]
+        assert "dead" in tail.split("{")[0] and tail.count("fk_ring_drain(") == 2, kern
+        assert body.count("|| dead) return;") == 2, f"{kern}: a request after the give-up"
+        gone = body.index("gone = dead;")
+        assert re.search(r"if \((gone\) break|!gone &&)", body[gone:]), f"{kern}: results without data are stored"
+    body = kernel("fft_small.cuh", "c2r_small_kernel")
+    assert "if (ok && j + NST < items) issue();" in body
+    for leave in re.finditer(r"return;", body):
+        assert "fk_ring_drain(" in body[max(0, leave.start() - 160):leave.start()]
