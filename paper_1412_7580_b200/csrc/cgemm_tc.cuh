@@ -28,7 +28,7 @@
 // boxes, N of the instructions, k-steps), which also makes room for a fourth stage:
 // M, N, K = 50, 90, 67 over the bins of n = 32 22.0 -> 18.5 us, 24, 100, 200 (n = 64)
 // 96 -> 83 us, 100, 10, 200 (n = 64) 88-120 -> 75-95 us; full tiles unchanged.  Narrow ones (N <= 64) share an SM among
-// two to four CTAs, where their loads, MMAs and stores fit (see the launcher).
+// two to four CTAs, where their loads, MMAs and stores fit (tc_share).
 //
 // Every wait on an mbarrier is bounded; when one runs out the kernel raises the
 // caller's status word, drains what it issued, frees its tensor memory and
@@ -44,20 +44,13 @@
 #include "cgemm_ffma.cuh"
 #include "tma_util.cuh"
 #include "dep_launch.cuh"
+#include "launch_rules.h"
 #include "fft_kernels.cuh"
 
 namespace fc {
 
-constexpr int TC_BM = 128, TC_BN = 128, TC_BK = 32, TC_STAGES = 3;
 constexpr int TC_THREADS = 192;
-constexpr uint32_t TC_TILE_BYTES = TC_BM * TC_BK * 4;            // one 128 x 32 fp32 box: 16 KB
-constexpr uint32_t TC_STAGE_BYTES = 4 * TC_TILE_BYTES;           // A_re, A_im, B_re, B_im
-constexpr uint32_t TC_EPI_BUF_BYTES = 32 * 128;                  // 32 rows x 32 fp32, one TMA store box
-constexpr uint32_t TC_EPI_BYTES = 4 * 2 * TC_EPI_BUF_BYTES;      // 4 warps x 2 buffers
-// Narrow matrices leave room for more stages than three, but more than four do not pay (S64 f64 f'128,
-// n = 64: 62 us with three, 59 with four, 65 with six).
-constexpr int TC_MAX_STAGES = 4;
-constexpr uint32_t tc_smem_bytes(int stages) { return 1024 + stages * TC_STAGE_BYTES + TC_EPI_BYTES + 512; }
+constexpr uint32_t tc_smem_bytes(int stages) { return TC_FIXED_BYTES + stages * TC_STAGE_BYTES + TC_EPI_BYTES; }
 // A launch that shares the SMs with a transform kernel (the filter spectrum produced range by range
 // beside the contraction) runs a ring of two stages and leaves 64 KB of shared memory to that kernel.
 constexpr int TC_STAGES_SHARED = 2;
@@ -465,36 +458,6 @@ static cudaError_t launch_cgemm_tc_f(const GemmParams& g, int* status, cudaStrea
     p.rows_a = cover(g.M, TA ? 32 : 8, TC_BM);
     p.rows_b = cover(g.N, TB ? 32 : 16, TC_BN);
     p.mma_n = cover(g.N, 16, TC_BN);
-    // CTAs per SM.  The tiles of narrow matrices are short chains of a load, a few MMAs and a store, which one CTA's ring
-    // and two accumulators do not hide.  Where the accumulators leave tensor memory for more CTAs (N <= 64: two, N <= 32:
-    // four) as many run as find two stages of the ring in shared memory (not beside a transform kernel, which needs the
-    // space).  M, N, K = 55, 12, 15 over the bins of n = 64 18.7 -> 12.8 us, 18, 6, 33 21.0 -> 12.9, 19, 34, 4 22.8 -> 16.0,
-    // n = 128: 9, 18, 20 55.6 -> 27, 40, 20, 60 88 -> 58-67, 96, 3, 128 158 -> 132-140; 300, 20, 20 (n = 64) unchanged.
-    const uint32_t stage = 256u * (uint32_t)(p.rows_a + p.rows_b);
-    int per_sm = 1;
-    p.acc_cols = TC_BN;
-    p.epi_bytes = TC_EPI_BYTES;
-    uint32_t ring = ST * TC_STAGE_BYTES;
-    if (!FULL && ST == TC_STAGES && g.N <= 64) {
-        // the staging tiles of the warps that have rows; at least 16 KB, because an MMA reads 128 rows of A whatever rows_a
-        // is, and what lies behind the last stage's has to be shared memory of this CTA
-        const uint32_t warps = (uint32_t)((p.rows_a + 31) / 32), epi = (warps < 2 ? 2 : warps) * 2 * TC_EPI_BUF_BYTES;
-        constexpr uint32_t SM_BYTES = 227 * 1024, RESERVED = 1024;      // per SM; per CTA, by the system
-        for (int c = g.N <= 32 ? 4 : 2; c > 1; --c) {
-            const uint32_t room = SM_BYTES / c / 1024 * 1024 - RESERVED, fixed = tc_smem_bytes(0) - TC_EPI_BYTES + epi;
-            if (room < fixed + 2 * stage) continue;
-            per_sm = c;
-            p.acc_cols = g.N <= 32 ? 32 : 64;
-            p.epi_bytes = epi;
-            ring = (room - fixed) / 1024 * 1024;
-            break;
-        }
-    }
-    p.ring_bytes = ring;
-    const int fit = (int)(ring / stage);
-    p.stages = fit < TC_MAX_STAGES ? fit : TC_MAX_STAGES;
-    if (per_sm > 1) p.ring_bytes = (uint32_t)p.stages * stage;
-    const size_t smem = tc_smem_bytes(0) - TC_EPI_BYTES + p.epi_bytes + p.ring_bytes;
     const bool okA = TA ? tc_make_map(&tmA, g.A, g.bins, g.K, g.M, g.lda, 32, TC_BK,
                                       CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)
                         : tc_make_map(&tmA, g.A, g.bins, g.M, g.K, g.lda, TC_BK, p.rows_a);
@@ -525,9 +488,18 @@ static cudaError_t launch_cgemm_tc_f(const GemmParams& g, int* status, cudaStrea
     }
     const long long tiles = (long long)p.bins_run * p.m_tiles * p.n_tiles;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const long long slots = (long long)sm_count * per_sm;
+    // several CTAs per SM: not beside a transform kernel, which needs the space
+    const TcShare s = tc_share(p.rows_a, p.rows_b, !FULL && ST == TC_STAGES ? g.N : TC_BN, tiles, sm_count);
+    p.ring_bytes = ST == TC_STAGES ? s.ring_bytes : ST * TC_STAGE_BYTES;
+    const int fit = (int)(p.ring_bytes / (256u * (uint32_t)(p.rows_a + p.rows_b)));
+    p.stages = fit < TC_MAX_STAGES ? fit : TC_MAX_STAGES;
+    p.epi_bytes = s.epi_bytes;
+    p.acc_cols = s.acc_cols;
+    const size_t smem = ST == TC_STAGES ? s.smem : tc_smem_bytes(ST);
+    const long long slots = (long long)sm_count * s.per_sm;
     const int grid = (int)(tiles < slots ? tiles : slots);
-    return dep_launch(g.overlap != 0, kern, dim3(grid), dim3(TC_THREADS), smem, st, tmA, tmB, tmC, p);
+    // the whole L1 as shared memory, as full tiles have it anyway
+    return dep_launch({g.overlap != 0, 1, ST == TC_STAGES ? 100 : -1}, kern, dim3(grid), dim3(TC_THREADS), smem, st, tmA, tmB, tmC, p);
 }
 
 template <bool TA, bool TB, int ST>

@@ -42,34 +42,43 @@ __device__ __forceinline__ void dep_wait() {
 //    same, most of them with sums of 32 to 64;
 //  * the inverse transform after an FP32 contraction, whatever its sum: 1-3 us shorter passes.
 // The callers set the flag accordingly; everything else is launched the plain way.
+struct DepConfig {
+    bool overlap;
+    int cluster;                // CTAs per cluster
+    // Percentage of an SM's L1 asked for as shared memory, -1: as the kernel's footprint has it.  An SM changes that division
+    // only when it is idle, so a kernel with a small footprint between kernels with a large one starts late and ends
+    // the overlap with its neighbours: 1 - 4 us per pass of 12 - 25 us.  (Not for every kernel: the forward transforms
+    // read their samples through the L1, wide planes 1713 -> 1923 us with all of it shared memory.)
+    int carveout;
+    DepConfig(bool overlap_, int cluster_ = 1, int carveout_ = -1) : overlap(overlap_), cluster(cluster_), carveout(carveout_) {}
+};
 template <typename... KArgs, typename... Args>
-static cudaError_t dep_launch(bool overlap, int cluster, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                      cudaStream_t st, Args&&... args) {
+static cudaError_t dep_launch(DepConfig c, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     int n = 0;
-    if (overlap) {
+    if (c.overlap) {
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n++].val.programmaticStreamSerializationAllowed = 1;
     }
-    if (cluster > 1) {
+    if (c.cluster > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
-        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.x = (unsigned)c.cluster;
         attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
         ++n;
+    }
+    if (c.carveout >= 0) {
+        attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[n++].val.sharedMemCarveout = (unsigned)c.carveout;
     }
     cfg.attrs = attr;
     cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-}
-template <typename... KArgs, typename... Args>
-static cudaError_t dep_launch(bool overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                              cudaStream_t st, Args&&... args) {
-    return dep_launch(overlap, 1, kern, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 }  // namespace fc

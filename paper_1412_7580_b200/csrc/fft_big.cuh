@@ -442,7 +442,7 @@ static cudaError_t launch_c2r_big(FftParams p, float* scratch, size_t scratch_by
     if (groups > fit) groups = fit;
     const dim3 grid((unsigned)(groups * cl));
     ulonglong2* sc = reinterpret_cast<ulonglong2*>(scratch);
-    return dep_launch(p.overlap != 0, cl, c2r_big_kernel, grid, dim3(Gm::T), Gm::SMEM, st, tm, tmny, p, sc, cl);
+    return dep_launch({p.overlap != 0, cl}, c2r_big_kernel, grid, dim3(Gm::T), Gm::SMEM, st, tm, tmny, p, sc, cl);
 }
 
 // Which plane sizes take the transforms of this file and fft_split.cuh.

@@ -125,3 +125,11 @@ def test_the_arithmetic_asked_for_is_the_one_that_runs(shape, flags):
                                    (400, 130, 64, 16), (400, 64, 65, 8), (650, 121, 5, 130), (1300, 1, 130, 3)])
 def test_tf32_several_ctas_per_sm(shape, flags):
     assert run(*shape, math=2, seed=19, **flags) <= TOL[2]
+
+
+# as many CTAs per SM as there are tiles for: both sides of 1, 2 and 3 tiles per SM, a sum of many k-blocks
+@pytest.mark.parametrize("flags", FLAGS[:3])
+@pytest.mark.parametrize("shape", [(148, 9, 14, 40), (149, 9, 14, 40), (296, 30, 33, 9), (297, 30, 33, 9), (445, 12, 20, 7),
+                                   (34, 45, 10, 700), (130, 130, 12, 100)])
+def test_tf32_ctas_per_sm_follow_the_tiles(shape, flags):
+    assert run(*shape, math=2, seed=23, **flags) <= TOL[2]
