@@ -489,7 +489,7 @@ static cudaError_t launch_cgemm_tc_f(const GemmParams& g, int* status, cudaStrea
     const long long tiles = (long long)p.bins_run * p.m_tiles * p.n_tiles;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     // several CTAs per SM: not beside a transform kernel, which needs the space
-    const TcShare s = tc_share(p.rows_a, p.rows_b, !FULL && ST == TC_STAGES ? g.N : TC_BN, tiles, sm_count);
+    const TcShare s = tc_share(p.rows_a, p.rows_b, !FULL && ST == TC_STAGES ? g.N : TC_BN, p.k_blocks, tiles, sm_count);
     p.ring_bytes = ST == TC_STAGES ? s.ring_bytes : ST * TC_STAGE_BYTES;
     const int fit = (int)(p.ring_bytes / (256u * (uint32_t)(p.rows_a + p.rows_b)));
     p.stages = fit < TC_MAX_STAGES ? fit : TC_MAX_STAGES;

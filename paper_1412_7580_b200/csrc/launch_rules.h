@@ -34,7 +34,8 @@ struct TcShare {
 };
 // The tiles of narrow matrices (N <= 64) are short chains of a load, a few MMAs and a store, which one CTA's ring and two
 // accumulators do not hide.  Where the accumulators leave tensor memory for more CTAs (N <= 64: two, N <= 32: four) as
-// many run as find two stages of the ring in shared memory, and as there are tiles for.  M, N, K = 55, 12, 15 over the
+// many run as find two stages of the ring in shared memory (three, where N > 32 and the sum is longer than a stage: M, N, K = 64,
+// 64, 64 over the bins of n = 64 38.6 us with four stages in one CTA, 41.5 with two in each of two), and as there are tiles for.  M, N, K = 55, 12, 15 over the
 // bins of n = 64 18.7 -> 12.8 us, 18, 6, 33 21.0 -> 12.9, 19, 34, 4 22.8 -> 16.0, n = 128: 9, 18, 20 55.6 -> 27, 40, 20, 60
 // 88 -> 58-67, 96, 3, 128 158 -> 132-140; 300, 20, 20 (n = 64) unchanged.
 // * Tiles for one CTA per SM or fewer: as many stages as one CTA can have, because a long sum lives on the loads in flight
@@ -44,7 +45,7 @@ struct TcShare {
 //   (a dependent's CTAs are placed early): fprop of S4 f1 f'39 60 x 23, n = 64, 38.2 us without the padding, 27.7 with it,
 //   36.2 with one CTA per SM.
 // rows_a, rows_b: rows of a stage's boxes.
-FC_RULE TcShare tc_share(int rows_a, int rows_b, int N, long long tiles, int sms) {
+FC_RULE TcShare tc_share(int rows_a, int rows_b, int N, int k_blocks, long long tiles, int sms) {
     const unsigned stage = 256u * (unsigned)(rows_a + rows_b);
     const int most = N > 64 ? 1 : (N > 32 ? 2 : 4);             // by tensor memory
     TcShare s{1, 0, TC_STAGES * TC_STAGE_BYTES, TC_EPI_BYTES, 0, (unsigned)TC_BN};
@@ -54,10 +55,10 @@ FC_RULE TcShare tc_share(int rows_a, int rows_b, int N, long long tiles, int sms
         const unsigned warps = (unsigned)((rows_a + 31) / 32);
         s.epi_bytes = (warps < 2 ? 2 : warps) * 2 * TC_EPI_BUF_BYTES;
         s.acc_cols = 128 / (unsigned)most;
-        const unsigned fixed = TC_FIXED_BYTES + s.epi_bytes;
+        const unsigned fixed = TC_FIXED_BYTES + s.epi_bytes, needed = N > 32 && k_blocks > 1 ? 3 : 2;
         for (int c = most; c >= 1; --c) {
             const unsigned room = (SM_SHARED_BYTES - 1024) / (unsigned)c / 1024 * 1024 - (c > 1 ? CTA_RESERVED_BYTES : 0);
-            if (c > 1 && (tiles <= (long long)(c - 1) * sms || room < fixed + 2 * stage)) continue;
+            if (c > 1 && (tiles <= (long long)(c - 1) * sms || room < fixed + needed * stage)) continue;
             s.per_sm = c;
             s.ring_bytes = (room - fixed) / 1024 * 1024;
             break;

@@ -1,5 +1,6 @@
 """The arithmetic that kernels and launchers share (csrc/launch_rules.h), compiled by itself for the host."""
 import ctypes
+import itertools
 import os
 import subprocess
 
@@ -9,8 +10,8 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_1412_7580_b200", "csrc")
 EXPORTS = """
 #include "launch_rules.h"
-extern "C" void tc_share(int rows_a, int rows_b, int N, long long tiles, int sms, long long* out) {
-    const fc::TcShare s = fc::tc_share(rows_a, rows_b, N, tiles, sms);
+extern "C" void tc_share(int rows_a, int rows_b, int N, int k_blocks, long long tiles, int sms, long long* out) {
+    const fc::TcShare s = fc::tc_share(rows_a, rows_b, N, k_blocks, tiles, sms);
     const long long v[6] = {s.per_sm, s.stages, s.ring_bytes, s.epi_bytes, s.smem, s.acc_cols};
     for (int i = 0; i < 6; ++i) out[i] = v[i];
 }
@@ -52,15 +53,15 @@ def test_contraction_ctas_per_sm(rules):
     seen = set()
     for rows_a in range(8, 129, 8):
         for rows_b, N in ((r, n) for r in range(16, 129, 16) for n in (r - 15, r)):
-            for tiles in (1, SMS, SMS + 1, 2 * SMS, 2 * SMS + 1, 3 * SMS + 1, 10 ** 6):
-                rules.tc_share(rows_a, rows_b, N, ctypes.c_longlong(tiles), SMS, out)
+            for k_blocks, tiles in itertools.product((1, 2), (1, SMS, SMS + 1, 2 * SMS, 2 * SMS + 1, 3 * SMS + 1, 10 ** 6)):
+                rules.tc_share(rows_a, rows_b, N, k_blocks, ctypes.c_longlong(tiles), SMS, out)
                 per_sm, stages, ring, epi, smem, acc = out
                 a, b = 128 * rows_a, 128 * rows_b
                 assert per_sm * (smem + RESERVED) <= SM and smem <= 227 * KB
                 fit = SM // (smem + RESERVED)
                 assert fit * 4 * acc <= TMEM and N <= acc           # not one that would wait for tensor memory
                 assert per_sm == 1 or (fit == per_sm and (per_sm - 1) * SMS < tiles)
-                assert stages == 4 or (per_sm > 1 and stages >= 2) or (stages == 3 and 5 * 2 * (a + b) > smem)
+                assert stages == 4 or (per_sm > 1 and stages >= (3 if N > 32 and k_blocks > 1 else 2)) or (stages == 3 and 5 * 2 * (a + b) > smem)
                 assert stages * 2 * (a + b) <= ring and ring + epi + 1536 <= smem
                 # an MMA reads 128 rows of A_im of the last stage, and N rounded up to 16 rows of B_im
                 assert (stages - 1) * 2 * (a + b) + a + 16 * KB <= ring + epi
