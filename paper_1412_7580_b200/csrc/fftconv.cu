@@ -306,7 +306,13 @@ int run_pass(conv_plan_s* plan, int pass, const float* a_in, const float* b_in, 
     const int herm_n = kept_herm_n(*plan);
     auto forward_small = [&](const fc::FftParams& f, bool dep) -> cudaError_t {
         g_launches.fetch_add(1, std::memory_order_relaxed);
-        const bool conc = dep && !big && !timing;
+        // At n = 64 many filters wait for the other operand, where that fills the SMs: its kernel leaves room for some of
+        // their CTAs on every SM, the rest start late and end last.  Passes beside / after it: S9 f69 f'98 k13 150 / 135 us,
+        // S12 f288 f'124 k13 386 / 350, S23 f208 f'88 k11 235 / 209, S8 f64 f'118 k11 106 / 91; fewer filters or a smaller
+        // operand the other way round: S6 f13 f'18 k13 25 / 30, S34 f17 f'16 k3 31 / 34, S1 f82 f'286 k3 288 / 307.
+        const bool wait = plan->n == 64 && (long long)f.R * f.C >= 4000 &&
+                          2LL * d.a.spec.R * ((d.a.spec.C + 7) / 8) > fc::fft_sm_count();
+        const bool conc = dep && !big && !timing && !wait;
         return fc::launch_r2c_small(plan->n, f, 0, plan->n / 2 + 1, st, conc, conc, herm_n != 0);
     };
     mark(0);
