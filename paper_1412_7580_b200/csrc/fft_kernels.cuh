@@ -713,6 +713,7 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
 // on the others.  With a load before every store the column of a thread was a chain of n round trips to memory, which
 // tiles of half as many planes hide less well: 16,385 planes of 32 x 32 113 us with the wide tiles, 143 with these,
 // 45 in batches; 65,537 of 16 x 16 70, 73 and 41; 262,145 of 8 x 8 69, 59 and 44; 4,097 of 64 x 64 232, 168 and 164.
+// In windows: accumulation and crops of at most half the basis.
 template <int N, int G, int LAYOUT, int MINB, bool WIN = false, bool DB = false, bool ACC = false>
 __global__ void __launch_bounds__(N* G, MINB)
 c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
@@ -966,20 +967,30 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
                 // rows [oy, oy + win_hc) of the transform go to the tile's place in the plane
                 const bool acc = p.accumulate != 0;
                 const int r0 = p.oy, pitch = p.W;
-                dst = p.real_out + win_base + (cA - p.ox) - (long long)r0 * pitch;
-                static_for<N>([&](auto Rr) {
-                    constexpr int r = decltype(Rr)::value;
-                    if (!acc) {
+                dst = p.real_out + win_base + (cA - p.ox);
+                if constexpr (!ACC) {
+                    dst -= (long long)r0 * pitch;
+                    static_for<N>([&](auto Rr) {
+                        constexpr int r = decltype(Rr)::value;
                         asm volatile(
                             "{\n\t.reg .pred p;\n\t"
                             "setp.lt.u32 p, %2, %3;\n\t"
                             "@p st.global.f32 [%0], %1;\n\t}"
                             ::"l"(dst), "f"(v[r] * scale), "r"(r - r0), "r"(win_hc) : "memory");
-                    } else if ((unsigned)(r - r0) < (unsigned)win_hc) {
-                        *dst += v[r] * scale;
-                    }
-                    dst += pitch;
-                });
+                        dst += pitch;
+                    });
+                } else {
+                    // a uniform branch per row: 32 x 32 windows, k27, S9 f22 f'4 43 x 103 bprop 86 us with predicates, 83 so
+                    static_for<N>([&](auto Rr) {
+                        constexpr int r = decltype(Rr)::value;
+                        if (r >= r0 && r < r0 + win_hc) {
+                            float o = v[r] * scale;
+                            if (acc) o += *dst;
+                            *dst = o;
+                            dst += pitch;
+                        }
+                    });
+                }
             } else if (!ACC && !p.accumulate && 2 * hc > N) {
                 static_for<N>([&](auto Rr) {
                     constexpr int r = decltype(Rr)::value;
@@ -1169,7 +1180,11 @@ static cudaError_t launch_r2c_layout(FftParams pa, const FftParams* pb_in, cudaS
     cudaError_t e = persistent_grid(reinterpret_cast<const void*>(kern), N * G, smem,
                                     (long long)pa.num_tiles + pb.num_tiles, &grid);
     if (e != cudaSuccess) return e;
-    return dep_launch(false, kern, dim3(grid), dim3(N * G), smem, st, tma, tmb, pa, pb);
+    // Windows, one round of tiles: no sample is read twice from an L1, and the contraction that is launched early behind this
+    // kernel finds the SMs divided as it needs them (S6 f1 f'1 103 x 65 k11 in 32 x 32 windows 19.7 -> 15.4 us, 16 x 16
+    // windows of 68 x 37 12.1 -> 10.6).  Larger launches read their overlaps from the L1 (8 x 8 windows 48 -> 61 us without).
+    const bool one_round = (long long)pa.num_tiles + pb.num_tiles <= grid;
+    return dep_launch({false, 1, win && one_round ? 100 : -1}, kern, dim3(grid), dim3(N * G), smem, st, tma, tmb, pa, pb);
 }
 
 // Bare layout: staged through shared memory with bulk copies where a tile with its staging
@@ -1208,7 +1223,9 @@ static cudaError_t launch_c2r_layout(FftParams p, cudaStream_t st) {
     }
     if (LAYOUT == LAYOUT_BARE_STAGED) smem += BareGeom<N, G>::BYTES;
     if (p.win && LAYOUT != LAYOUT_FREQ_TMA) return cudaErrorInvalidValue;
-    auto kern = (p.win && LAYOUT == LAYOUT_FREQ_TMA) ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, LAYOUT == LAYOUT_FREQ_TMA, DB>
+    constexpr bool FREQ = LAYOUT == LAYOUT_FREQ_TMA;
+    auto kern = (p.win && FREQ)  ? (p.accumulate || 2 * p.h <= N ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB, true>
+                                                                 : c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB>)
                 : p.accumulate                       ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, false, DB, LAYOUT == LAYOUT_BARE_STAGED>
                                                      : c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, false, DB>;
     int grid = 0;
