@@ -93,6 +93,7 @@ struct FftParams {
     int nty, ntx;
     int step_y, step_x;
     int oy, ox;
+    int in_step;            // forward, n = 64: the CTAs of a cluster begin each item together (fft_split.cuh)
     int overlap;            // host only: launch as a programmatic dependent of the previous kernel
     int* status;            // device status word raised when a bounded wait runs out (may be null)
     long long wait_cycles;  // limit of one wait in SM clock cycles; <= 0 selects FK_WAIT_CYCLES
@@ -1117,6 +1118,40 @@ static cudaError_t persistent_grid(const void* kern, int threads, size_t smem, l
     if (sms < 1) return cudaErrorInvalidConfiguration;
     const long long slots = (long long)per_sm * sms;
     *grid = (int)(tiles < slots ? tiles : slots);
+    return cudaSuccess;
+}
+
+// Clusters of `size` CTAs that are resident at a time: they stay inside a GPC, whose SMs they need not fill.  Remembered like
+// the grids above (persistent_grid has raised the kernel's shared-memory limit).
+static cudaError_t resident_clusters(const void* kern, int threads, size_t smem, int size, int* clusters) {
+    struct Entry { const void* kern; int size, dev, clusters; };
+    static Entry cache[32];
+    static int cached = 0;
+    static std::mutex mu;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    for (int i = 0; i < cached; ++i)
+        if (cache[i].kern == kern && cache[i].size == size && cache[i].dev == dev) {
+            *clusters = cache[i].clusters;
+            return cudaSuccess;
+        }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    if (e != cudaSuccess) return e;
+    if (n < 1) return cudaErrorInvalidConfiguration;
+    if (cached < 32) cache[cached++] = Entry{kern, size, dev, n};
+    *clusters = n;
     return cudaSuccess;
 }
 

@@ -234,6 +234,11 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
         const int h = p.h, w = p.w;
         if (tid == 32 && item + (int)gridDim.x < items) split_prefetch<N>(item + gridDim.x, items0, p0, p1);
 
+        if (N == 64 && p0.in_step) {
+            asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+            asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        }
+
         // ---- A: columns; a pair of columns past the plane reads no sample and writes zeros ----
         {
             // a window of a larger plane: its origin (y0, x0) may lie outside, samples there read as zero
@@ -388,9 +393,50 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
 
 // At n = 64 (without windows) the plain kernel, whose tiles are 4 planes, is the better one where no tile is more than half full: 300 rows of
 // 4 planes 20.9 -> 18.8 us (25 x 25), of 6 planes 18.8 against 26.9.
+// Spectra whose rows are no whole sectors (ld = 4 mod 8), from about the size of the L2 on.  Every other row starts in the
+// middle of a sector, so a tile shares its sectors with the tiles before and after it, and parts of a sector that SMs
+// of different dies write cost more than everything else.
+// * The plain kernel's tiles share sectors in pairs (2j, 2j + 1), which adjacent CTAs write, if the tiles of every matrix and
+//   those launched before it come in even numbers: SECTORS_PLAIN.  Plain / this kernel in single CTAs (passes, planes of 50 x 50):
+//   1,332 rows of 9 planes 389 / 570 us, 1,000 of 12 298 / 371, 1,332 of 18 496 / 700, 352 of 34 209 / 236, 240 of 50 187 / 200, 134 of
+//   178 323 / 406.  With odd numbers the plain kernel is the one that loses (353 of 34 288 / 230, 135 of 178 608 / 418; 160 rows of
+//   90 filters behind 115 tiles 351 / 252, behind 92 210 / 249), and where rows of planes start off a 16-byte boundary it waits for
+//   the odd samples of every tile (298 rows of 134 planes of 49 x 49 759 / 298).
+// * Otherwise SECTORS_NEAR: clusters of eight CTAs, which share a die, take four adjacent tiles and begin their items together.  Single
+//   CTAs / clusters (transform alone): 3,333 rows of 12 planes of 62 x 62 1064 / 586 us, 1,176 of 34 737 / 528, 800 of 50 planes
+//   of 49 x 49 612 / 474; clusters of four 769, 647, 565.
+// Smaller spectra are better off in single CTAs (160 rows of 50 89 / 93), longer rows turn over later (666 of 12 134 / 119 at
+// 135 MB; plain / single CTAs 160 of 50 147 / 144 at 135 MB, 52 of 201 225 / 203 at 176).
+enum { SECTORS_WHOLE = 0, SECTORS_NEAR = 1, SECTORS_PLAIN = 2 };
+static inline int split_sectors(const FftParams& pa, const FftParams* pb) {
+    const FftParams* ops[2] = {&pa, pb};
+    double bytes[2] = {0, 0}, partial = 0;
+    int widest = 0;
+    long long before = 0;
+    bool pairs = true;
+    for (int i = 0; i < (pb ? 2 : 1); ++i) bytes[i] = 8.0 * 64 * 33 * (double)ops[i]->R * ops[i]->C;
+    const double total = bytes[0] + bytes[1];
+    for (int i = 0; i < (pb ? 2 : 1); ++i) {
+        const FftParams& p = *ops[i];
+        const long long tiles = (long long)p.R * ((p.C + 3) / 4);
+        if (10 * bytes[i] > total) {
+            const bool rows_aligned = (reinterpret_cast<uintptr_t>(p.real_in) & 15) == 0 && (long long)p.C * p.h * p.w % 4 == 0;
+            pairs = pairs && rows_aligned && before % 2 == 0 && tiles % 2 == 0;
+            if (p.ld % 8 != 0) {
+                partial += bytes[i];
+                if (p.C > widest) widest = p.C;
+            }
+        }
+        before += tiles;
+    }
+    if (3 * partial <= total || total <= 120e6 + 450e3 * widest) return SECTORS_WHOLE;
+    return pairs ? SECTORS_PLAIN : SECTORS_NEAR;
+}
 static inline bool split_pays(int n, const FftParams& pa, const FftParams* pb) {
     if (n != 64) return false;
-    return pa.win || (pb && pb->win) || 2 * pa.C > SplitGeom<64>::G || (pb && 2 * pb->C > SplitGeom<64>::G);
+    if (pa.win || (pb && pb->win)) return true;
+    if (split_sectors(pa, pb) == SECTORS_PLAIN) return false;
+    return 2 * pa.C > SplitGeom<64>::G || (pb && 2 * pb->C > SplitGeom<64>::G);
 }
 
 // Forward transform of one operand, or of two in one launch (pb may be null).
@@ -415,9 +461,24 @@ static cudaError_t launch_r2c_split(FftParams pa, const FftParams* pb_in, cudaSt
     if (N != 64 && (pa.win || pb.win)) return cudaErrorInvalidValue;
     const cudaError_t e = persistent_grid(reinterpret_cast<const void*>(kern), Gm::T, Gm::SMEM, items, &grid);
     if (e != cudaSuccess) return e;
+    // n = 64: the CTAs of a launch drift apart, and in a long one the second of a tile's two items no longer finds the samples in
+    // the L2 (40,200 planes of 62 x 62: 764 MB read from memory instead of 618).  From about 400 MB of spectra on the two
+    // are a cluster whose CTAs begin each item together: 40,000 planes of 62 x 62 373 -> 311 us, 49 x 49 300 -> 278; 24,000
+    // 172 / 173 and 170 / 166, 8,000 60 / 64.
+    int cluster = 1;
+    if (N == 64 && !pa.win && !pb.win && items > grid)
+        cluster = split_sectors(pa, pb_in ? &pb : nullptr) == SECTORS_NEAR ? 8 : (items >= 8000 ? 2 : 1);
+    if (cluster > 1) {
+        int fit = 0;
+        const cudaError_t ce = resident_clusters(reinterpret_cast<const void*>(kern), Gm::T, Gm::SMEM, cluster, &fit);
+        if (ce != cudaSuccess) return ce;
+        if (fit * cluster < grid) grid = fit * cluster;
+        grid -= grid % cluster;
+    }
+    pa.in_step = cluster > 1;
     // One round of items: no L1 is of use, and the filters' transform, launched early behind this one, finds the SMs divided as it
     // needs them (S9 f58 f'6 36 x 44 k9 43.9 -> 37.7 us, S17 f34 f'6 50 x 57 k13 38.1 -> 34.3).
-    return dep_launch({false, 1, items <= grid ? 100 : -1}, kern, dim3(grid), dim3(Gm::T), Gm::SMEM, st, m[0], m[1], m[2], m[3], pa, pb);
+    return dep_launch({false, cluster, items <= grid ? 100 : -1}, kern, dim3(grid), dim3(Gm::T), Gm::SMEM, st, m[0], m[1], m[2], m[3], pa, pb);
 }
 
 }  // namespace fc

@@ -58,3 +58,30 @@ def test_passes_against_oracle(dims, shift, tile):
         g = got.cpu().numpy().astype(np.float64)
         assert np.max(np.abs(g - ref)) <= 1e-5 * np.max(np.abs(ref))
     fc.conv_plan_destroy(p)
+
+
+# Spectra beyond the L2 whose rows are no whole sectors (12 planes), by tiles in even numbers (the plain kernel) and in odd ones
+# (clusters of eight, the last one not full), and ones so large that two CTAs keep step
+@pytest.mark.parametrize("dims", [(668, 12, 2, 33, 34, 14, 2, 64), (667, 12, 2, 33, 34, 14, 2, 64), (4003, 7, 1, 33, 35, 14, 2, 64)])
+def test_forward_transform_of_spectra_beyond_the_l2(dims):
+    import torch
+    import oracle
+    import paper_1412_7580_b200 as fc
+    from paper_1412_7580_b200 import workloads as wl
+    s = wl.ConvShape("beyond_l2", *dims, cfg=9, point=sum(dims))
+    x, w, dy = wl.make_x(s), wl.make_w(s), wl.make_dy(s)
+    p = fc.conv_plan(*s.args())
+    fc.conv_plan_set_math(p, fc.binding.MATH_FP32)
+    fc.conv_plan_alloc_workspace(p)
+    y = torch.full((s.S, s.fp, s.oh, s.ow), float("nan"), device="cuda")
+    dw = torch.full(w.shape, float("nan"), device="cuda")
+    xd = torch.from_numpy(x).cuda()
+    fc.conv_fprop(p, xd, torch.from_numpy(w).cuda(), y)
+    fc.conv_accgrad(p, torch.from_numpy(dy).cuda(), xd, dw)
+    torch.cuda.synchronize()
+    assert fc.conv_plan_status(p) == 0
+    # 2 x 12 butterfly stages and sums of 12 (y) or at most 4,003 products (dw), each rounded at 2^-24 of its value, signs at
+    # random: 2^-24 (24 + sqrt(4003)) = 5.2e-6 of the largest result; four times that
+    for got, ref in ((y, oracle.fprop(x, w)), (dw, oracle.accgrad(dy, x, s.kh, s.kw))):
+        assert np.max(np.abs(got.cpu().numpy().astype(np.float64) - ref)) <= 2.1e-5 * np.max(np.abs(ref))
+    fc.conv_plan_destroy(p)
