@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <new>
@@ -506,16 +507,19 @@ FFTCONV_API size_t conv_plan_workspace_bytes(const conv_plan_t* plan) {
 }
 
 namespace {
-// Plan-time estimate of one training step (three passes) in microseconds, from the bytes each
-// kernel family moves and the rates measured for it on B200 (TB/s = bytes per picosecond):
-// transforms 4.4 (n <= 32), 3.0 (n = 64), 2.2 (n = 128: of earlier kernels; the present ones reach 2.4 - 2.5 on
-// full layers, so the ranking leans towards tiling there), windowed forward transforms 3.4
-// (2.4 at n = 8: the fixed cost per window weighs more),
-// contraction 5.5; plus a fixed cost per launch.  Only used to rank tile bases against each other.
+// Plan-time estimate of one training step (three passes) in microseconds: the bytes that each kernel moves over the rates
+// measured for it on B200 (bytes per us; medians of the launches over 40 us of 220 layers in all their bases), the chain of
+// k-blocks where a contraction has few tiles and a long sum (windows of accGrad: S128 f3 f'1 120 x 120 in 8 x 8 windows
+// 5.9 ms, its bytes 0.03), and a fixed cost per pass.  Only used to rank tile bases against each other.  Over 317 layers in two
+// or more bases (S 1 .. 128, f and f' 1 .. 384, planes of 13 .. 256, k 3 .. 13) a step in the chosen basis takes 1.5 % longer than in the
+// best one, 41 are more than 5 % behind it and one more than 5 % behind the untiled plan; with the rates of earlier
+// kernels and without the chain 4.7 %, 62 and 4.  (A third of the layers, kept out of the fit: 1.4 against 7.1 %.)
 double estimate_step_us(const conv_plan_s& p) {
-    const bool tiled = p.n != p.n_full;
-    const double fft_rate = p.n <= 32 ? 4.4e6 : (p.n == 64 ? 3.0e6 : 2.2e6);     // bytes per us
-    const double win_rate = p.n >= 16 ? 3.4e6 : 2.4e6;
+    // n = 8, 16, 32, 64, 128
+    const double fwd[5] = {4.4e6, 4.4e6, 4.4e6, 4.0e6, 3.0e6}, fwd_win[5] = {4.0e6, 4.2e6, 3.9e6, 4.2e6, 0};
+    const double inv[5] = {4.4e6, 4.4e6, 4.4e6, 4.3e6, 2.5e6}, inv_win[5] = {3.3e6, 3.2e6, 4.2e6, 4.2e6, 0};
+    const int at = p.n <= 8 ? 0 : (p.n <= 16 ? 1 : (p.n <= 32 ? 2 : (p.n <= 64 ? 3 : 4)));
+    constexpr double kSms = 148.0;
     double us = 0.0;
     for (int pass = 0; pass < 3; ++pass) {
         const PassDesc d = describe(p, pass);
@@ -525,11 +529,16 @@ double estimate_step_us(const conv_plan_s& p) {
             const OperandDesc& o = *ops[i];
             const double spec = (double)o.spec.bytes(p.bins);
             const double real = 4.0 * o.spec.R * o.spec.C * o.h * o.w;
-            const bool windowed_load = tiled && o.win && i < 2;
-            us += (spec + real) / (windowed_load ? win_rate : fft_rate);
+            us += (spec + real) / (i < 2 ? (o.win ? fwd_win[at] : fwd[at]) : (o.win ? inv_win[at] : inv[at]));
             spectra += spec;
         }
-        us += spectra / 5.5e6 + 3 * 4.0;
+        // rounds of tiles, each a chain of k-blocks: 0.8 us per 32 k on the tensor cores, 1.85 per 16 k of FP32 (four CTAs per SM)
+        const bool tensor = fc::tc_shape_profitable(d.M, d.N, d.K);
+        const int tile = tensor ? 128 : 64, block = tensor ? 32 : 16;
+        const double tiles = (double)p.bins * ((d.M + tile - 1) / tile) * ((d.N + tile - 1) / tile);
+        const double rounds = std::ceil(tiles / (tensor ? kSms : 4 * kSms));
+        const double chain = rounds * ((d.K + block - 1) / block) * (tensor ? 0.8 : 1.85), moved = spectra / 5.5e6;
+        us += (moved > chain ? moved : chain) + 3 * 4.0;
     }
     return us;
 }
