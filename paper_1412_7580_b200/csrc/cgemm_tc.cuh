@@ -498,8 +498,9 @@ static cudaError_t launch_cgemm_tc_f(const GemmParams& g, int* status, cudaStrea
     const size_t smem = ST == TC_STAGES ? s.smem : tc_smem_bytes(ST);
     const long long slots = (long long)sm_count * s.per_sm;
     const int grid = (int)(tiles < slots ? tiles : slots);
-    // the whole L1 as shared memory, as full tiles have it anyway
-    return dep_launch({g.overlap != 0, 1, ST == TC_STAGES ? 100 : -1}, kern, dim3(grid), dim3(TC_THREADS), smem, st, tmA, tmB, tmC, p);
+    // narrow matrices: the whole L1 as shared memory, as the footprint of the others has it anyway
+    const int carveout = !FULL && ST == TC_STAGES && g.N <= 64 ? 100 : -1;
+    return dep_launch({g.overlap != 0, 1, carveout}, kern, dim3(grid), dim3(TC_THREADS), smem, st, tmA, tmB, tmC, p);
 }
 
 template <bool TA, bool TB, int ST>

@@ -3,7 +3,7 @@
 // A packed instruction does two fp32 operations with the rounding of the scalar ones, from one
 // issue slot.  The fp32 pipe itself is no faster (measured on B200: 128 lane-operations per clock
 // and SM either way), so the packed form pays where a kernel is held by instruction issue: the
-// forward transform of n = 128, and the FP32 contraction, which keeps its multiply-adds at half of the issue
+// transforms of n = 64 and 128 on pairs of columns, and the FP32 contraction, which keeps its multiply-adds at half of the issue
 // slots and has the other half for loads and address arithmetic.
 #pragma once
 

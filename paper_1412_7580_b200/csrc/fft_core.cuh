@@ -10,9 +10,9 @@
 // X_k = sum_j x_j exp(-2 pi i jk/N), unnormalised; the inverse uses the
 // conjugate roots and is unnormalised as well (the caller applies 1/n^2).
 //
-// cfft and rfft are templates over the value type V: float, or F2 (f32x2.cuh), which carries the same
+// cfft, rfft and irfft are templates over the value type V: float, or F2 (f32x2.cuh), which carries the same
 // element of two independent transforms through packed instructions -- twice the transforms for the
-// same number of issued instructions, bit for bit the same results (transforms of n = 128).
+// same number of issued instructions, bit for bit the same results (transforms of n = 64 and 128).
 #pragma once
 
 #include <utility>
@@ -245,100 +245,6 @@ FC_HD void irfft(const V (&Xr)[N / 2 + 1], const V (&Xi)[N / 2 + 1], V (&x)[N]) 
         x[2 * j] = zr[j];
         x[2 * j + 1] = zi[j];
     });
-}
-
-// ---------------------------------------------------------------------------
-// One radix-4 decimation-in-frequency step of an N-point complex transform split
-// over four cooperating threads.  All threads see the N inputs through load(j)
-// (a float2); thread Q in {0..3} forms the N/4 inputs of the quarter-size
-// transform whose outputs are X_{4m+Q}:
-//   a_j = (x_j + u^Q x_{j+L} + u^2Q x_{j+2L} + u^3Q x_{j+3L}) w_N^{+-Qj},  L = N/4,
-// with u = -i forward and +i inverse.
-// ---------------------------------------------------------------------------
-template <int N, bool INV, int Q, int J>
-FC_HD void split4_elem(const float2 x0, const float2 x1, const float2 x2, const float2 x3, float& outr, float& outi) {
-    float tr, ti;
-    if constexpr (Q == 0) {
-        tr = (x0.x + x2.x) + (x1.x + x3.x); ti = (x0.y + x2.y) + (x1.y + x3.y);
-    } else if constexpr (Q == 2) {
-        tr = (x0.x + x2.x) - (x1.x + x3.x); ti = (x0.y + x2.y) - (x1.y + x3.y);
-    } else {
-        const float dr = x0.x - x2.x, di = x0.y - x2.y;     // x_j - x_{j+2L}
-        const float er = x1.x - x3.x, ei = x1.y - x3.y;     // x_{j+L} - x_{j+3L}
-        // forward Q = 1 (inverse Q = 3): d - i e;   forward Q = 3 (inverse Q = 1): d + i e
-        if constexpr ((Q == 1) != INV) { tr = dr + ei; ti = di - er; }
-        else                           { tr = dr - ei; ti = di + er; }
-    }
-    if constexpr (Q == 0 || J == 0) {
-        outr = tr; outi = ti;
-    } else {
-        constexpr float c = Tw<N, Q * J>::c;
-        constexpr float s = INV ? -Tw<N, Q * J>::s : Tw<N, Q * J>::s;
-        // w = (c, -s): w t = (c tr + s ti, c ti - s tr)
-        outr = vfma(s, ti, vmul(c, tr));
-        outi = vfma(-s, tr, vmul(c, ti));
-    }
-}
-template <int N, bool INV, int Q, class Load>
-FC_HD void load_split4(Load&& load, float (&ar)[N / 4], float (&ai)[N / 4]) {
-    constexpr int L = N / 4;
-    static_for<L>([&](auto J) {
-        constexpr int j = decltype(J)::value;
-        const float2 x0 = load(J), x1 = load(std::integral_constant<int, j + L>{});
-        const float2 x2 = load(std::integral_constant<int, j + 2 * L>{});
-        const float2 x3 = load(std::integral_constant<int, j + 3 * L>{});
-        split4_elem<N, INV, Q, j>(x0, x1, x2, x3, ar[j], ai[j]);
-    });
-}
-
-// ---------------------------------------------------------------------------
-// Inverse of the real-input FFT split over two cooperating threads (decimation
-// in time).  Thread Q in {0,1} reads the bins k = Q (mod 2) of the Hermitian half
-// through X(k) (a float2; X(0) must return (Re X_0, Re X_{N/2}) -- both bins are
-// real), forms Z'_{2m+Q} with the pre-pass of irfft (k and M-k have the same
-// parity) and runs an M/2-point inverse FFT.  Result: Q = 0 returns E_j, Q = 1
-// returns w_M^{-j} O_j (j < M/2); then z_j = E_j + w^{-j} O_j and
-// z_{j+M/2} = E_j - w^{-j} O_j, with x_2j = Re z_j, x_2j+1 = Im z_j (times N).
-// ---------------------------------------------------------------------------
-template <int N, int Q, class LoadX>
-FC_HD void irfft_half(LoadX&& X, float (&er)[N / 4], float (&ei)[N / 4]) {
-    static_assert(N >= 8, "needs an even quarter length");
-    constexpr int M = N / 2, H = M / 2;
-    auto pair = [&](auto K) {
-        constexpr int k = decltype(K)::value;
-        constexpr int m = (k - Q) / 2, mp = (M - k - Q) / 2;
-        constexpr float c = Tw<N, k>::c, s = Tw<N, k>::s;
-        const float2 P = X(K), Qv = X(std::integral_constant<int, M - k>{});
-        const float sr = P.x + Qv.x, si = P.y - Qv.y;   // P + conj Q
-        const float dr = P.x - Qv.x, di = P.y + Qv.y;   // P - conj Q
-        const float ur = vfma(-s, di, vmul(c, dr));        // w_N^{-k} D
-        const float ui = vfma(s, dr, vmul(c, di));
-        er[m] = sr - ui;  ei[m] = si + ur;
-        er[mp] = sr + ui; ei[mp] = ur - si;
-    };
-    if constexpr (Q == 0) {
-        const float2 dc = X(std::integral_constant<int, 0>{});
-        er[0] = dc.x + dc.y; ei[0] = dc.x - dc.y;
-        const float2 mid = X(std::integral_constant<int, H>{});
-        er[H / 2] = vmul(2.0f, mid.x); ei[H / 2] = vmul(-2.0f, mid.y);
-        static_for<H / 2 - 1>([&](auto I) {
-            pair(std::integral_constant<int, 2 * (decltype(I)::value + 1)>{});
-        });
-    } else {
-        static_for<H / 2>([&](auto I) {
-            pair(std::integral_constant<int, 2 * decltype(I)::value + 1>{});
-        });
-    }
-    cfft<H, true>(er, ei);
-    if constexpr (Q == 1) {
-        static_for<H - 1>([&](auto J) {
-            constexpr int j = decltype(J)::value + 1;
-            constexpr float c = Tw<M, j>::c, s = Tw<M, j>::s;
-            const float a = er[j], b = ei[j];
-            er[j] = vfma(-s, b, vmul(c, a));
-            ei[j] = vfma(s, a, vmul(c, b));
-        });
-    }
 }
 
 }  // namespace fc

@@ -359,8 +359,6 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
     const bool is_loader = (tid == T / 2);
     const bool is_storer = (tid >= T - 32) && ((tid & 31) < NB);
 
-    // Stage the planes of a tile.  Returns true if the copy is asynchronous (wait on the
-    // barrier before reading), false if it was done with plain loads by all threads.
     // Window of a larger plane: clipped loads (Section 5.1) of the column that this thread transforms, straight into
     // registers, where they wait while the rows of the tile before are transformed.  The loads are volatile: they are
     // issued together, where they stand.  (B200, 16 x 256 planes of 128 x 128, 3 x 3 kernels, 16 x 16 windows: x 224 ->
@@ -383,6 +381,9 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
         });
     };
     int off = 0, off_n = 0;         // first sample of the tile in sIn: this tile, the one on its way
+    // Stage the planes of a tile.  Returns true if the copy is asynchronous (wait on the
+    // barrier before reading), false if it was done with plain loads by all threads (filters beside
+    // windows) or into registers (windows).
     auto stage = [&](bool second, int row, int tcol) -> bool {
         const int sh = second ? p1.h : p0.h, sw = second ? p1.w : p0.w;
         const int sC = second ? p1.C : p0.C;

@@ -85,3 +85,9 @@ def test_bit_identical_reruns_and_untouched_canaries(dims, math):
     assert bool((ws_buf[:off] == 777.25).all())
     assert bool((ws_buf[off + need // 4:] == 777.25).all())
     fc.conv_plan_destroy(p)
+
+
+# n = 64 with more tiles than SMs in all three inverse transforms (two teams per tile)
+@pytest.mark.parametrize("math", [1, 2])
+def test_bit_identical_reruns_of_many_tiles(math):
+    test_bit_identical_reruns_and_untouched_canaries((19, 33, 30, 64, 63, 14, 2, 64), math)

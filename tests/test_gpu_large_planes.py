@@ -85,3 +85,55 @@ def test_forward_transform_of_spectra_beyond_the_l2(dims):
     for got, ref in ((y, oracle.fprop(x, w)), (dw, oracle.accgrad(dy, x, s.kh, s.kw))):
         assert np.max(np.abs(got.cpu().numpy().astype(np.float64) - ref)) <= 2.1e-5 * np.max(np.abs(ref))
     fc.conv_plan_destroy(p)
+
+
+# The gradient that is added to: pairs of columns (even crop, even address) and single samples, n = 64 with more tiles than SMs
+# (no square crop that the small-crop kernel takes) and n = 128
+@pytest.mark.parametrize("dims,shift", [
+    ((2, 33, 30, 64, 63, 14, 2, 64), 0),
+    ((2, 33, 30, 64, 63, 14, 2, 64), 1),
+    ((2, 30, 33, 57, 64, 2, 13, 64), 0),
+    ((2, 33, 30, 40, 40, 13, 13, 64), 0),
+    ((2, 9, 11, 120, 120, 7, 6, 128), 0),
+    ((2, 9, 11, 120, 120, 7, 6, 128), 1),
+])
+def test_accumulated_filter_gradient(dims, shift):
+    import torch
+    import oracle
+    import paper_1412_7580_b200 as fc
+    from paper_1412_7580_b200 import workloads as wl
+    s = wl.ConvShape("accumulate", *dims, cfg=9, point=sum(dims) + shift)
+    x, dy, before = wl.make_x(s), wl.make_dy(s), wl.make_w(s)
+    p = fc.conv_plan(*s.args())
+    fc.conv_plan_set_math(p, fc.binding.MATH_FP32)
+    fc.conv_plan_alloc_workspace(p)
+    flat = torch.empty(before.size + shift, device="cuda")
+    flat[shift:] = torch.from_numpy(before.ravel()).cuda()
+    dw = flat[shift:].view(before.shape)
+    fc.conv_accgrad(p, torch.from_numpy(dy).cuda(), torch.from_numpy(x).cuda(), dw, accumulate=True)
+    torch.cuda.synchronize()
+    assert fc.conv_plan_status(p) == 0
+    # the bound of test_passes_against_oracle and one rounding more
+    ref = before.astype(np.float64) + oracle.accgrad(dy, x, s.kh, s.kw)
+    assert np.max(np.abs(dw.cpu().numpy().astype(np.float64) - ref)) <= 1e-5 * np.max(np.abs(ref))
+    fc.conv_plan_destroy(p)
+
+
+# one tile of 4 planes for every SM (the plain inverse kernel) and one more (two teams per tile)
+@pytest.mark.parametrize("dims", [(37, 2, 16, 33, 40, 5, 7, 64), (149, 2, 3, 34, 33, 6, 5, 64)])
+def test_inverse_of_as_many_tiles_as_sms(dims):
+    import torch
+    import oracle
+    import paper_1412_7580_b200 as fc
+    from paper_1412_7580_b200 import workloads as wl
+    s = wl.ConvShape("sms", *dims, cfg=9, point=sum(dims))
+    x, w = wl.make_x(s), wl.make_w(s)
+    p = fc.conv_plan(*s.args())
+    fc.conv_plan_set_math(p, fc.binding.MATH_FP32)
+    fc.conv_plan_alloc_workspace(p)
+    y = torch.full((s.S, s.fp, s.oh, s.ow), float("nan"), device="cuda")
+    fc.conv_fprop(p, torch.from_numpy(x).cuda(), torch.from_numpy(w).cuda(), y)
+    torch.cuda.synchronize()
+    ref = oracle.fprop(x, w)
+    assert np.max(np.abs(y.cpu().numpy().astype(np.float64) - ref)) <= 1e-5 * np.max(np.abs(ref))
+    fc.conv_plan_destroy(p)

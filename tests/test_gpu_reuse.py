@@ -83,3 +83,39 @@ def test_reuse_matches_plain_passes_and_oracle(dims, small):
     assert relerr(dw1.cpu().numpy().astype(np.float64), oracle.accgrad(dy2, x3, s.kh, s.kw)) <= TOL[eff[2]]
     fc.conv_plan_destroy(p)
     fc.conv_plan_destroy(plain)
+
+
+@pytest.mark.parametrize("dims", [(5, 9, 7, 57, 60, 5, 4, 64), (19, 33, 30, 64, 63, 14, 2, 64), (2, 9, 10, 100, 97, 5, 3, 128)])
+def test_reuse_of_large_planes(dims):
+    """The spectra of n = 64 and 128 come from and go to kernels of their own; filters that the small-plane kernel
+    transforms (5 x 4, 5 x 3) and filters that share a launch (14 x 2)."""
+    import torch
+    import oracle
+    import paper_1412_7580_b200 as fc
+    from paper_1412_7580_b200 import workloads as wl
+    s = wl.ConvShape("reuse", *dims, cfg=10, point=sum(dims))
+    x, w, dy = wl.make_x(s), wl.make_w(s), wl.make_dy(s)
+    xd, wd, dyd = (torch.from_numpy(a).cuda() for a in (x, w, dy))
+    plans, outs = [], []
+    for reuse in (False, True):
+        p = fc.conv_plan(*s.args())
+        fc.conv_plan_set_spectrum_reuse(p, reuse)
+        fc.conv_plan_alloc_workspace(p).view(torch.float32)[64:].fill_(float("nan"))
+        o = [torch.full(shape, float("nan"), device="cuda") for shape in ((s.S, s.fp, s.oh, s.ow), x.shape, w.shape)]
+        fc.conv_fprop(p, xd, wd, o[0]); fc.conv_bprop(p, dyd, wd, o[1]); fc.conv_accgrad(p, dyd, xd, o[2])
+        plans.append(p)
+        outs.append(o)
+    torch.cuda.synchronize()
+    eff = [fc.conv_plan_pass_math(plans[1], k) for k in range(3)]
+    refs = (oracle.fprop(x, w), oracle.bprop(dy, w, s.h, s.w), oracle.accgrad(dy, x, s.kh, s.kw))
+    for a, b, ref, e in zip(*outs, refs, eff):
+        assert torch.equal(a, b)                                  # more than 4 planes in every row: the same kernels
+        assert relerr(b.cpu().numpy().astype(np.float64), ref) <= TOL[e]
+    wd.mul_(-0.5)                                                 # next step: new weights at the same address
+    fc.conv_fprop(plans[1], xd, wd, outs[1][0]); fc.conv_bprop(plans[1], dyd, wd, outs[1][1])
+    torch.cuda.synchronize()
+    for got, ref, e in zip(outs[1], refs, eff[:2]):
+        assert relerr(got.cpu().numpy().astype(np.float64), -0.5 * ref) <= TOL[e]
+    for p in plans:
+        assert fc.conv_plan_status(p) == 0
+        fc.conv_plan_destroy(p)
