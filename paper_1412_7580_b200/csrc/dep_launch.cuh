@@ -29,7 +29,8 @@ __device__ __forceinline__ void dep_wait() {
 // `overlap` = false launches the plain way.  Where overlapping pays was measured on B200
 // (three layer configurations and a 1,000-point sweep of the parameter grid):
 //  * contraction after one-pass forward transforms, inverse transform after the contraction:
-//    1-7 % shorter passes at n <= 64 with the tensor-core contraction;
+//    1-7 % shorter passes at n <= 64 with the tensor-core contraction (the two-team inverse of n = 64 excepted, see
+//    fft_inv64.cuh: a dependent's CTAs lose the placement that lets neighbours share sectors);
 //  * the forward transforms as dependents of the previous pass's inverse transform gain
 //    nothing at n <= 32, and at n = 64 a training step took 1.14 ms instead of 0.74;
 //  * at n = 128 a pass is 0.5 % longer with the contraction as a

@@ -93,7 +93,6 @@ struct FftParams {
     int nty, ntx;
     int step_y, step_x;
     int oy, ox;
-    int in_step;            // forward, n = 64: the CTAs of a cluster begin each item together (fft_split.cuh)
     int overlap;            // host only: launch as a programmatic dependent of the previous kernel
     int* status;            // device status word raised when a bounded wait runs out (may be null)
     long long wait_cycles;  // limit of one wait in SM clock cycles; <= 0 selects FK_WAIT_CYCLES
@@ -965,7 +964,7 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
             // otherwise builds a branch and fresh 64-bit address arithmetic per row)
             float* dst = p.real_out + ((size_t)row * p.C + c0 + gA) * hw + cA;
             const float scale = p.scale;
-            if (WIN && p.win) {
+            if constexpr (WIN) {
                 // rows [oy, oy + win_hc) of the transform go to the tile's place in the plane
                 const bool acc = p.accumulate != 0;
                 const int r0 = p.oy, pitch = p.W;
@@ -1260,7 +1259,7 @@ static cudaError_t launch_c2r_layout(FftParams p, cudaStream_t st) {
     if (LAYOUT == LAYOUT_BARE_STAGED) smem += BareGeom<N, G>::BYTES;
     if (p.win && LAYOUT != LAYOUT_FREQ_TMA) return cudaErrorInvalidValue;
     constexpr bool FREQ = LAYOUT == LAYOUT_FREQ_TMA;
-    auto kern = (p.win && FREQ)  ? (p.accumulate || 2 * p.h <= N ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB, true>
+    auto kern = (p.win && FREQ)  ? (p.accumulate || 2 * p.h <= N ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB, FREQ>
                                                                  : c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB>)
                 : p.accumulate                       ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, false, DB, LAYOUT == LAYOUT_BARE_STAGED>
                                                      : c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, false, DB>;

@@ -211,7 +211,7 @@ template <int N, bool WIN>
 __global__ void __launch_bounds__(SplitGeom<N>::T, SplitGeom<N>::MINB)
 r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUtensorMap tmNy0,
                  const __grid_constant__ CUtensorMap tmS1, const __grid_constant__ CUtensorMap tmNy1,
-                 const __grid_constant__ FftParams p0, const __grid_constant__ FftParams p1) {
+                 const __grid_constant__ FftParams p0, const __grid_constant__ FftParams p1, const int in_step) {
     using Gm = SplitGeom<N>;
     constexpr int M = Gm::M, G = Gm::G, CP = Gm::CP, RP = Gm::RP, PP = Gm::PP, T = Gm::T;
     extern __shared__ __align__(128) unsigned char fc_smem[];
@@ -234,7 +234,7 @@ r2c_split_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant
         const int h = p.h, w = p.w;
         if (tid == 32 && item + (int)gridDim.x < items) split_prefetch<N>(item + gridDim.x, items0, p0, p1);
 
-        if (N == 64 && p0.in_step) {
+        if (N == 64 && in_step) {                   // the CTAs of a cluster begin each item together
             asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
             asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         }
@@ -475,10 +475,9 @@ static cudaError_t launch_r2c_split(FftParams pa, const FftParams* pb_in, cudaSt
         if (fit * cluster < grid) grid = fit * cluster;
         grid -= grid % cluster;
     }
-    pa.in_step = cluster > 1;
     // One round of items: no L1 is of use, and the filters' transform, launched early behind this one, finds the SMs divided as it
     // needs them (S9 f58 f'6 36 x 44 k9 43.9 -> 37.7 us, S17 f34 f'6 50 x 57 k13 38.1 -> 34.3).
-    return dep_launch({false, cluster, items <= grid ? 100 : -1}, kern, dim3(grid), dim3(Gm::T), Gm::SMEM, st, m[0], m[1], m[2], m[3], pa, pb);
+    return dep_launch({false, cluster, items <= grid ? 100 : -1}, kern, dim3(grid), dim3(Gm::T), Gm::SMEM, st, m[0], m[1], m[2], m[3], pa, pb, cluster > 1 ? 1 : 0);
 }
 
 }  // namespace fc
