@@ -714,7 +714,7 @@ r2c_kernel(const __grid_constant__ CUtensorMap tmS0, const __grid_constant__ CUt
 // on the others.  With a load before every store the column of a thread was a chain of n round trips to memory, which
 // tiles of half as many planes hide less well: 16,385 planes of 32 x 32 113 us with the wide tiles, 143 with these,
 // 45 in batches; 65,537 of 16 x 16 70, 73 and 41; 262,145 of 8 x 8 69, 59 and 44; 4,097 of 64 x 64 232, 168 and 164.
-// In windows: accumulation and crops of at most half the basis.
+// In windows: crops of at most half the basis.
 template <int N, int G, int LAYOUT, int MINB, bool WIN = false, bool DB = false, bool ACC = false>
 __global__ void __launch_bounds__(N* G, MINB)
 c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
@@ -964,7 +964,7 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
             // otherwise builds a branch and fresh 64-bit address arithmetic per row)
             float* dst = p.real_out + ((size_t)row * p.C + c0 + gA) * hw + cA;
             const float scale = p.scale;
-            if constexpr (WIN) {
+            if (WIN && p.win) {
                 // rows [oy, oy + win_hc) of the transform go to the tile's place in the plane
                 const bool acc = p.accumulate != 0;
                 const int r0 = p.oy, pitch = p.W;
@@ -973,11 +973,15 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
                     dst -= (long long)r0 * pitch;
                     static_for<N>([&](auto Rr) {
                         constexpr int r = decltype(Rr)::value;
-                        asm volatile(
-                            "{\n\t.reg .pred p;\n\t"
-                            "setp.lt.u32 p, %2, %3;\n\t"
-                            "@p st.global.f32 [%0], %1;\n\t}"
-                            ::"l"(dst), "f"(v[r] * scale), "r"(r - r0), "r"(win_hc) : "memory");
+                        if (!acc) {
+                            asm volatile(
+                                "{\n\t.reg .pred p;\n\t"
+                                "setp.lt.u32 p, %2, %3;\n\t"
+                                "@p st.global.f32 [%0], %1;\n\t}"
+                                ::"l"(dst), "f"(v[r] * scale), "r"(r - r0), "r"(win_hc) : "memory");
+                        } else if ((unsigned)(r - r0) < (unsigned)win_hc) {
+                            *dst += v[r] * scale;
+                        }
                         dst += pitch;
                     });
                 } else {
@@ -1002,7 +1006,7 @@ c2r_kernel(const __grid_constant__ CUtensorMap tmS, const FftParams p) {
                         ::"l"(dst), "f"(v[r] * scale), "r"(r), "r"(hc) : "memory");
                     dst += wc;
                 });
-            } else if constexpr (ACC) {
+            } else if constexpr (ACC && !WIN) {
                 // rows in batches: what a batch adds to is loaded before the first of it is stored
                 constexpr int BATCH = 8;
                 static_for<N / BATCH>([&](auto Bb) {
@@ -1259,7 +1263,7 @@ static cudaError_t launch_c2r_layout(FftParams p, cudaStream_t st) {
     if (LAYOUT == LAYOUT_BARE_STAGED) smem += BareGeom<N, G>::BYTES;
     if (p.win && LAYOUT != LAYOUT_FREQ_TMA) return cudaErrorInvalidValue;
     constexpr bool FREQ = LAYOUT == LAYOUT_FREQ_TMA;
-    auto kern = (p.win && FREQ)  ? (p.accumulate || 2 * p.h <= N ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB, FREQ>
+    auto kern = (p.win && FREQ)  ? (2 * p.h <= N ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB, FREQ>
                                                                  : c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, FREQ, DB>)
                 : p.accumulate                       ? c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, false, DB, LAYOUT == LAYOUT_BARE_STAGED>
                                                      : c2r_kernel<N, G, LAYOUT, Cfg::MINB_INV, false, DB>;
