@@ -1125,21 +1125,18 @@ static cudaError_t persistent_grid(const void* kern, int threads, size_t smem, l
     return cudaSuccess;
 }
 
-// Clusters of `size` CTAs that are resident at a time: they stay inside a GPC, whose SMs they need not fill.  Remembered like
-// the grids above (persistent_grid has raised the kernel's shared-memory limit).
-static cudaError_t resident_clusters(const void* kern, int threads, size_t smem, int size, int* clusters) {
+// Clusters of `size` CTAs that are resident at a time (they stay inside a GPC, whose SMs they need not fill); 0 where none is.
+// Remembered like the grids above (persistent_grid has raised the kernel's shared-memory limit).
+static int resident_clusters(const void* kern, int threads, size_t smem, int size) {
     struct Entry { const void* kern; int size, dev, clusters; };
     static Entry cache[32];
     static int cached = 0;
     static std::mutex mu;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     std::lock_guard<std::mutex> lock(mu);
     for (int i = 0; i < cached; ++i)
-        if (cache[i].kern == kern && cache[i].size == size && cache[i].dev == dev) {
-            *clusters = cache[i].clusters;
-            return cudaSuccess;
-        }
+        if (cache[i].kern == kern && cache[i].size == size && cache[i].dev == dev) return cache[i].clusters;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)size);
     cfg.blockDim = dim3((unsigned)threads);
@@ -1151,12 +1148,12 @@ static cudaError_t resident_clusters(const void* kern, int threads, size_t smem,
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (n < 1) return cudaErrorInvalidConfiguration;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();   // the caller goes on without clusters
+        n = 0;
+    }
     if (cached < 32) cache[cached++] = Entry{kern, size, dev, n};
-    *clusters = n;
-    return cudaSuccess;
+    return n;
 }
 
 // Tensor map of a planar spectrum for the staging tiles: box = G columns x 1 row x D bins.

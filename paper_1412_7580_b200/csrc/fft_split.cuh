@@ -469,11 +469,10 @@ static cudaError_t launch_r2c_split(FftParams pa, const FftParams* pb_in, cudaSt
     if (N == 64 && !pa.win && !pb.win && items > grid)
         cluster = split_sectors(pa, pb_in ? &pb : nullptr) == SECTORS_NEAR ? 8 : (items >= 8000 ? 2 : 1);
     if (cluster > 1) {
-        int fit = 0;
-        const cudaError_t ce = resident_clusters(reinterpret_cast<const void*>(kern), Gm::T, Gm::SMEM, cluster, &fit);
-        if (ce != cudaSuccess) return ce;
-        if (fit * cluster < grid) grid = fit * cluster;
-        grid -= grid % cluster;
+        const int fit = cluster * resident_clusters(reinterpret_cast<const void*>(kern), Gm::T, Gm::SMEM, cluster);
+        const int together = (fit < grid ? fit : grid) / cluster * cluster;
+        if (together > 0) grid = together;
+        else cluster = 1;           // (a part of a GPU that holds no such cluster)
     }
     // One round of items: no L1 is of use, and the filters' transform, launched early behind this one, finds the SMs divided as it
     // needs them (S9 f58 f'6 36 x 44 k9 43.9 -> 37.7 us, S17 f34 f'6 50 x 57 k13 38.1 -> 34.3).
