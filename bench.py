@@ -54,42 +54,42 @@ MAX_BLOCKS = 400
 NCU_TRAFFIC_SOURCE = {
     "profile": "profiles/dram_traffic_per_launch_three_layer_configs.md",
     "ncu": "dram__bytes_read.sum + dram__bytes_write.sum, default cache control (caches flushed before each launch)",
-    "kernel_sources_sha256": "937859665318186b30ca1dcce928fa7456dd1d61d2dd2e00c93a7dc1e97defaf",
+    "kernel_sources_sha256": "fecd66d45ae2080b1e4cf0e0d294215b8341d4c6788aa133046e081851cdb5f0",
 }
 NCU_TRAFFIC = {
     "mid_S128_f96_fp256_31x31_k5/r2c_fft_first_operand/fprop": 54.0e6,
-    "mid_S128_f96_fp256_31x31_k5/r2c_fft_small_planes/fprop": 40.4e6,
-    "mid_S128_f96_fp256_31x31_k5/bin_contraction/fprop": 226.1e6,
-    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/fprop": 192.7e6,
-    "mid_S128_f96_fp256_31x31_k5/r2c_fft_first_operand/bprop": 186.3e6,
-    "mid_S128_f96_fp256_31x31_k5/r2c_fft_small_planes/bprop": 41.0e6,
-    "mid_S128_f96_fp256_31x31_k5/bin_contraction/bprop": 261.1e6,
-    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/bprop": 54.7e6,
-    "mid_S128_f96_fp256_31x31_k5/r2c_fft_both_operands/accgrad": 286.9e6,
-    "mid_S128_f96_fp256_31x31_k5/bin_contraction/accgrad": 240.4e6,
-    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/accgrad": 101.5e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_first_operand/fprop": 226.6e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_small_planes/fprop": 7.7e6,
-    "largek_S128_f64_fp64_64x64_k11/bin_contraction/fprop": 280.7e6,
-    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/fprop": 187.5e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_first_operand/bprop": 183.0e6,
+    "mid_S128_f96_fp256_31x31_k5/r2c_fft_small_planes/fprop": 40.5e6,
+    "mid_S128_f96_fp256_31x31_k5/bin_contraction/fprop": 226.2e6,
+    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/fprop": 193.5e6,
+    "mid_S128_f96_fp256_31x31_k5/r2c_fft_first_operand/bprop": 186.2e6,
+    "mid_S128_f96_fp256_31x31_k5/r2c_fft_small_planes/bprop": 41.2e6,
+    "mid_S128_f96_fp256_31x31_k5/bin_contraction/bprop": 261.3e6,
+    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/bprop": 54.4e6,
+    "mid_S128_f96_fp256_31x31_k5/r2c_fft_both_operands/accgrad": 286.8e6,
+    "mid_S128_f96_fp256_31x31_k5/bin_contraction/accgrad": 240.3e6,
+    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/accgrad": 101.2e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_first_operand/fprop": 227.6e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_small_planes/fprop": 7.6e6,
+    "largek_S128_f64_fp64_64x64_k11/bin_contraction/fprop": 280.6e6,
+    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/fprop": 185.9e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_first_operand/bprop": 181.9e6,
     "largek_S128_f64_fp64_64x64_k11/r2c_fft_small_planes/bprop": 7.8e6,
-    "largek_S128_f64_fp64_64x64_k11/bin_contraction/bprop": 281.1e6,
-    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/bprop": 217.1e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_both_operands/accgrad": 457.2e6,
-    "largek_S128_f64_fp64_64x64_k11/bin_contraction/accgrad": 312.3e6,
+    "largek_S128_f64_fp64_64x64_k11/bin_contraction/bprop": 280.6e6,
+    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/bprop": 216.8e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_both_operands/accgrad": 475.4e6,
+    "largek_S128_f64_fp64_64x64_k11/bin_contraction/accgrad": 313.7e6,
     "largek_S128_f64_fp64_64x64_k11/c2r_ifft/accgrad": 67.2e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_first_operand/fprop": 38.9e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_first_operand/fprop": 38.6e6,
     "deep_S128_f384_fp384_13x13_k3/r2c_fft_small_planes/fprop": 99.7e6,
-    "deep_S128_f384_fp384_13x13_k3/bin_contraction/fprop": 225.4e6,
-    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/fprop": 56.7e6,
+    "deep_S128_f384_fp384_13x13_k3/bin_contraction/fprop": 225.0e6,
+    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/fprop": 56.8e6,
     "deep_S128_f384_fp384_13x13_k3/r2c_fft_first_operand/bprop": 26.3e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_small_planes/bprop": 99.4e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_small_planes/bprop": 99.2e6,
     "deep_S128_f384_fp384_13x13_k3/bin_contraction/bprop": 225.3e6,
     "deep_S128_f384_fp384_13x13_k3/c2r_ifft/bprop": 56.8e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_both_operands/accgrad": 114.9e6,
-    "deep_S128_f384_fp384_13x13_k3/bin_contraction/accgrad": 194.9e6,
-    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/accgrad": 172.3e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_both_operands/accgrad": 114.7e6,
+    "deep_S128_f384_fp384_13x13_k3/bin_contraction/accgrad": 195.8e6,
+    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/accgrad": 172.0e6,
 }
 
 
