@@ -213,7 +213,7 @@ int conv_plan_invalidate_spectra(conv_plan_t* plan);
  * n_tile == FFTCONV_TILE_AUTO lets the plan choose: it estimates a training step for every
  * admissible basis from the bytes each kernel moves and the sums it chains (Section 3.4's one strategy per problem size,
  * decided by a static model instead of trial runs) and keeps tiling off unless a tile basis is
- * estimated at least 10 % faster. */
+ * estimated at least 5 % faster. */
 #define FFTCONV_TILE_AUTO (-1)
 int conv_plan_set_tiling(conv_plan_t* plan, int n_tile);
 
