@@ -54,41 +54,41 @@ MAX_BLOCKS = 400
 NCU_TRAFFIC_SOURCE = {
     "profile": "profiles/dram_traffic_per_launch_three_layer_configs.md",
     "ncu": "dram__bytes_read.sum + dram__bytes_write.sum, default cache control (caches flushed before each launch)",
-    "kernel_sources_sha256": "fecd66d45ae2080b1e4cf0e0d294215b8341d4c6788aa133046e081851cdb5f0",
+    "kernel_sources_sha256": "249b6873da2bfb2a46c99553b20a08c2918e32f64f00f4cf92486b7aa7649934",
 }
 NCU_TRAFFIC = {
     "mid_S128_f96_fp256_31x31_k5/r2c_fft_first_operand/fprop": 54.0e6,
     "mid_S128_f96_fp256_31x31_k5/r2c_fft_small_planes/fprop": 40.5e6,
-    "mid_S128_f96_fp256_31x31_k5/bin_contraction/fprop": 226.2e6,
-    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/fprop": 193.5e6,
-    "mid_S128_f96_fp256_31x31_k5/r2c_fft_first_operand/bprop": 186.2e6,
-    "mid_S128_f96_fp256_31x31_k5/r2c_fft_small_planes/bprop": 41.2e6,
-    "mid_S128_f96_fp256_31x31_k5/bin_contraction/bprop": 261.3e6,
-    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/bprop": 54.4e6,
-    "mid_S128_f96_fp256_31x31_k5/r2c_fft_both_operands/accgrad": 286.8e6,
-    "mid_S128_f96_fp256_31x31_k5/bin_contraction/accgrad": 240.3e6,
+    "mid_S128_f96_fp256_31x31_k5/bin_contraction/fprop": 225.7e6,
+    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/fprop": 193.2e6,
+    "mid_S128_f96_fp256_31x31_k5/r2c_fft_first_operand/bprop": 186.6e6,
+    "mid_S128_f96_fp256_31x31_k5/r2c_fft_small_planes/bprop": 41.1e6,
+    "mid_S128_f96_fp256_31x31_k5/bin_contraction/bprop": 261.2e6,
+    "mid_S128_f96_fp256_31x31_k5/c2r_ifft/bprop": 54.6e6,
+    "mid_S128_f96_fp256_31x31_k5/r2c_fft_both_operands/accgrad": 286.5e6,
+    "mid_S128_f96_fp256_31x31_k5/bin_contraction/accgrad": 240.8e6,
     "mid_S128_f96_fp256_31x31_k5/c2r_ifft/accgrad": 101.2e6,
     "largek_S128_f64_fp64_64x64_k11/r2c_fft_first_operand/fprop": 227.6e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_small_planes/fprop": 7.6e6,
-    "largek_S128_f64_fp64_64x64_k11/bin_contraction/fprop": 280.6e6,
-    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/fprop": 185.9e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_first_operand/bprop": 181.9e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_small_planes/bprop": 7.8e6,
-    "largek_S128_f64_fp64_64x64_k11/bin_contraction/bprop": 280.6e6,
-    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/bprop": 216.8e6,
-    "largek_S128_f64_fp64_64x64_k11/r2c_fft_both_operands/accgrad": 475.4e6,
-    "largek_S128_f64_fp64_64x64_k11/bin_contraction/accgrad": 313.7e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_small_planes/fprop": 7.8e6,
+    "largek_S128_f64_fp64_64x64_k11/bin_contraction/fprop": 279.6e6,
+    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/fprop": 186.2e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_first_operand/bprop": 181.5e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_small_planes/bprop": 7.9e6,
+    "largek_S128_f64_fp64_64x64_k11/bin_contraction/bprop": 280.7e6,
+    "largek_S128_f64_fp64_64x64_k11/c2r_ifft/bprop": 216.3e6,
+    "largek_S128_f64_fp64_64x64_k11/r2c_fft_both_operands/accgrad": 471.6e6,
+    "largek_S128_f64_fp64_64x64_k11/bin_contraction/accgrad": 312.3e6,
     "largek_S128_f64_fp64_64x64_k11/c2r_ifft/accgrad": 67.2e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_first_operand/fprop": 38.6e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_small_planes/fprop": 99.7e6,
-    "deep_S128_f384_fp384_13x13_k3/bin_contraction/fprop": 225.0e6,
-    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/fprop": 56.8e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_first_operand/bprop": 26.3e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_small_planes/bprop": 99.2e6,
-    "deep_S128_f384_fp384_13x13_k3/bin_contraction/bprop": 225.3e6,
-    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/bprop": 56.8e6,
-    "deep_S128_f384_fp384_13x13_k3/r2c_fft_both_operands/accgrad": 114.7e6,
-    "deep_S128_f384_fp384_13x13_k3/bin_contraction/accgrad": 195.8e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_first_operand/fprop": 38.8e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_small_planes/fprop": 100.0e6,
+    "deep_S128_f384_fp384_13x13_k3/bin_contraction/fprop": 225.5e6,
+    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/fprop": 56.7e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_first_operand/bprop": 26.1e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_small_planes/bprop": 99.5e6,
+    "deep_S128_f384_fp384_13x13_k3/bin_contraction/bprop": 225.0e6,
+    "deep_S128_f384_fp384_13x13_k3/c2r_ifft/bprop": 56.7e6,
+    "deep_S128_f384_fp384_13x13_k3/r2c_fft_both_operands/accgrad": 114.6e6,
+    "deep_S128_f384_fp384_13x13_k3/bin_contraction/accgrad": 195.5e6,
     "deep_S128_f384_fp384_13x13_k3/c2r_ifft/accgrad": 172.0e6,
 }
 
